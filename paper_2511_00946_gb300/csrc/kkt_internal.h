@@ -144,6 +144,7 @@ struct Info {
 // global memory.
 struct FacLayout {
   int q, R, Rs, ldD, ldZ, ldT, oDfac, oM, oRinv, oRinvZ, oZ, oT, oTab, oDfac2, oRinv2, oCorner, total;
+  int oF[2];  // exponents of split panel rows (kkt_oz.cuh; FP64 CTA tasks), two buffers for a pair's consumer
 };
 __host__ __device__ inline int kkt_align16(int b) { return (b + 15) & ~15; }
 // `dbl`: a second pivot buffer (and rinv) so that warp 4 can write the
@@ -170,7 +171,9 @@ __host__ __device__ inline FacLayout fac_layout(int n, int m, int zb, bool fill 
   L.oRinv2 = L.oDfac2 + (dbl ? kkt_align16(8 * L.q * L.ldD) : 0);
   // sum of the lower levels' corner partials (m x m), formed before the corner
   L.oCorner = L.oRinv2 + (dbl ? kkt_align16(8 * L.q) : 0);
-  L.total = L.oCorner + kkt_align16(8 * kMaxM * kMaxM);
+  L.oF[0] = L.oCorner + kkt_align16(8 * kMaxM * kMaxM);
+  L.oF[1] = L.oF[0] + (zb == 8 ? kkt_align16(4 * L.Rs) : 0);
+  L.total = L.oF[1] + (zb == 8 ? kkt_align16(4 * L.Rs) : 0);
   return L;
 }
 // One warp's slice for a small-block segment task (k_factor_w): the same

@@ -26,6 +26,7 @@
 #include "kkt_internal.h"
 #include "kkt_bulk.cuh"
 #include "kkt_numerics.cuh"
+#include "kkt_oz.cuh"
 #include "kkt_tc.cuh"
 
 namespace kkt {
@@ -429,6 +430,53 @@ __device__ void syrk_trap(double* T, int ldt, const TZ* Zlo, const TZ* Z, int zs
   gsync(g);
 }
 
+// ---------------------------------------------------------------------------
+// FP64 Schur products on the tensor cores (kkt_oz.cuh).
+// ---------------------------------------------------------------------------
+
+// Panel rows [r0, r1) of Z to digits in place, their exponents to rowf: eight
+// lanes a row. By the whole group; the caller synchronizes before and after.
+__device__ void oz_encode(double* Z, int ldz, int r0, int r1, int n, int* rowf, Grp G) {
+  const int sub = G.tid & 7, span = r0 + ((r1 - r0 + 3) & ~3);  // (whole warps: four rows each)
+  for (int r = r0 + (G.tid >> 3); r < span; r += G.nt >> 3) {
+    oz::u64* z = (oz::u64*)(Z + (r < r1 ? r : r1 - 1) * ldz);
+    int em = 0;
+    for (int k = sub; k < n; k += 8) em = max(em, oz::expo(z[k]));
+    for (int o = 4; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
+    if (r < r1) {
+      const int f = oz::row_exp(em);
+      if (f != oz::kFp64Row)
+        for (int k = sub; k < n; k += 8) z[k] = oz::encode(z[k], f);
+      if (sub == 0) rowf[r] = f;
+    }
+  }
+}
+
+// T[a][b] -= sum_t Z[a][t] Z[b][t] for ra0 <= a < ra1, cb0 <= b <= a (cb0 <=
+// ra0), rows in digits (oz_encode). Panel rows below `zsplit` are read from
+// (Zlo, flo), the others from (Z, fz). One 16 x 8 tile per warp at a time.
+// Every element is an exact sum rounded once, so the result does not depend
+// on the tiling. Ends with the group's barrier.
+__device__ void oz_syrk(double* T, int ldt, const double* Zlo, const int* flo, const double* Z, const int* fz,
+                        int zsplit, int ldz, int ra0, int ra1, int cb0, int n, Grp G) {
+  const int lane = G.tid & 31, nw = G.nt >> 5, w0 = ra0 - cb0;
+  // row tile i has cols(i) column tiles; this warp takes every nw-th tile
+  int i = 0, j = G.tid >> 5;
+  for (;;) {
+    int cols;
+    for (;; ++i) {
+      if (ra0 + 16 * i >= ra1) break;
+      cols = (w0 + min(16 * i + 16, ra1 - ra0) + 7) >> 3;
+      if (j < cols) break;
+      j -= cols;
+    }
+    if (ra0 + 16 * i >= ra1) break;
+    oz::tile(T, ldt, Zlo, flo, Z, fz, zsplit, ldz, ra0 + 16 * i, ra1, cb0 + 8 * j, ra1, n, lane);
+    j += nw;
+  }
+  gsync(G);
+}
+
 // Tensor-core form of the mixed Schur update (whole-CTA layout, eight warps):
 // T[a][b] -= (Z Z^T)[a][b] for r0 <= b <= a < pr1, with Z (FP32, ld ldz)
 // rounded to TF32 or BF16 and the products accumulated in FP32 by tcgen05
@@ -612,16 +660,9 @@ __device__ __forceinline__ SegGeom seg_geom(const LevelDesc& d, int k) {
 // E- and G-rows, and their Schur updates D_{i+1}, G_{i+1}, R~_k. The consumer
 // runs the fill-in rows: W_i D-hat_i^{-T} and the updates A~_k, Q~_k^T and
 // W_{i+1}, which read the producer's D-hat_i, E-hat_i and G-hat_i but feed
-// nothing back into the chain, so the consumer may lag a stage behind. Three
+// nothing back into the chain, so the consumer may lag a stage behind. Two
 // layouts (`mode`):
-//   kWhole  one CTA runs both (segment 1, the top level, and mixed levels
-//           that are not paired);
-//   kSplit  one CTA, warps 0-3 producer and warps 4-7 consumer (FP64 levels
-//           with more segments than SM pairs): the producer factors D_{i+1}
-//           while the consumer is still on stage i. Hand-offs are named
-//           barriers, each used once per stage by both roles:
-//             kBarFullM  M_i, rinv_i ready       kBarFreeM  M_i read
-//             kBarFullZ  E-hat_i, G-hat_i ready  kBarFreeZ  E-hat_i, G-hat_i read
+//   kWhole  one CTA runs both;
 //   kPair   a cluster of two CTAs (levels with few segments): CTA 0 is the
 //           producer, CTA 1 the consumer, each on an SM of its own, so a
 //           segment gets two SMs' FP64 pipes. After its trsm of stage i the
@@ -633,9 +674,7 @@ __device__ __forceinline__ SegGeom seg_geom(const LevelDesc& d, int k) {
 //           A last phase, after every remote store, ends the task.
 // ---------------------------------------------------------------------------
 static_assert(kFactorThreads == 256, "the factor roles assume 8 warps per CTA");
-constexpr int kWhole = 0, kSplit = 1, kPair = 2;
-constexpr int kBarProd = 2, kBarCons = 3, kBarFullM = 4, kBarFreeM = 5, kBarFullZ = 6, kBarFreeZ = 7;
-constexpr int kRoleThreads = 128;
+constexpr int kWhole = 0, kPair = 2;
 
 // Pairs (i, k) with 1 <= k <= i < n ordered by k descending (packed
 // i << 16 | k): the updates by column j are the prefix of length
@@ -883,9 +922,11 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
                              const int* skip, unsigned char* smraw, Grp G, int fwd_done, int c0 = 0);
 
 // MINB: CTAs per SM the register allocation must allow. Launches of CTA pairs
-// (one CTA per SM, latency-bound) take the unconstrained allocation (1);
-// the others four (at most 64 registers), so that several segment CTAs share
-// an SM when shared memory allows it.
+// (one CTA per SM, latency-bound) take the unconstrained allocation (1), the
+// FP64 launches two (128 registers: the fragments and accumulators of a digit
+// product; with three CTAs and 80 registers they spill: 67.1 against 63.8 ms
+// on 4096 uneven systems), the mixed ones four (at most 64 registers), so that
+// several segment CTAs share an SM when shared memory allows it.
 // TC: the instantiation with the tensor-core Schur products (mixed launches
 // that use them); the others carry none of that code.
 // One segment task of the factorization by the whole CTA (or, with `pair`,
@@ -914,13 +955,15 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
   TZ* const Z = cx.Z;
   int* const tab = cx.tab;
   const SegGeom g = cx.g;
-  const int mode = pair ? kPair : (g.hasW && !mixed) ? kSplit : kWhole;
+  const int mode = pair ? kPair : kWhole;
   // consumer buffers of the pair layout: buffer 0 is (M, rinvZ, Z rows [0, n+m)),
   // buffer 1 reuses the pivot block, rinv and the first rows of T, which a
   // consumer CTA has no other use for
   auto Mbuf = [&](int b) { return b ? (TZ*)Dfac : M; };
   auto rinvbuf = [&](int b) { return b ? (TZ*)rinv : rinvZ; };
   auto Zbuf = [&](int b) { return b ? (TZ*)T : Z; };
+  auto fbuf = [&](int b) { return (int*)(smraw + lay.oF[b]); };  // exponents of split rows (FP64)
+  int* const rowf = fbuf(0);
   const bool eg = mode != kPair || rank == 0;       // this CTA holds the E/G rows
   const bool wr = g.hasW && (mode != kPair || rank == 1);  // this CTA holds the W rows
 
@@ -963,18 +1006,16 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
     cluster_wait();
   }
 
-  const bool producer = mode == kWhole || (mode == kSplit && (int)threadIdx.x < kRoleThreads) ||
-                        (mode == kPair && rank == 0);
+  const bool producer = mode == kWhole || rank == 0;
   auto store_pivot = [&](int j, const double* Dp_, const double* rv, const TZ* Ms, Grp G) {
     cx.store_pivot(j, Dp_, rv, Ms, G);
   };
   auto store_panel = [&](int j, int r0, int r1, int rows, Grp G) { cx.store_panel(j, r0, r1, rows, G); };
-  // hand the trsm operand (strict lower triangle of Msrc, ld ldD), its
-  // 1/diag and panel rows [r0, r1) of stage i to the consumer CTA of a pair
-  auto push_stage = [&](int i, const TZ* Msrc, const TZ* rsrc, int r0, int r1, Grp G) {
-    const int b = i & 1;
-    const unsigned aM = cluster_addr(Mbuf(b), 1), aR = cluster_addr(rinvbuf(b), 1),
-                   aZ = cluster_addr(Zbuf(b), 1);
+  // hand the trsm operand (strict lower triangle of Msrc, ld ldD) and its
+  // 1/diag of stage i to the consumer CTA of a pair; then panel rows [r0, r1)
+  // (FP64: in digits, with their exponents)
+  auto push_pivot = [&](int i, const TZ* Msrc, const TZ* rsrc, Grp G) {
+    const unsigned aM = cluster_addr(Mbuf(i & 1), 1), aR = cluster_addr(rinvbuf(i & 1), 1);
     const int ntri = (n - 1) * n / 2;
     for (int e = G.tid; e < ntri; e += G.nt) {
       int a, c;
@@ -983,48 +1024,23 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
       st_cluster(aM + off * (unsigned)sizeof(TZ), Msrc[off]);
     }
     for (int e = G.tid; e < n; e += G.nt) st_cluster(aR + e * (unsigned)sizeof(TZ), rsrc[e]);
+  };
+  auto push_rows = [&](int i, int r0, int r1, Grp G) {
+    const unsigned aZ = cluster_addr(Zbuf(i & 1), 1);
     for (int e = G.tid; e < (r1 - r0) * n; e += G.nt) {
       const int r = r0 + e / n, c = e - (r - r0) * n;
       const int off = r * ldZ + c;
       st_cluster(aZ + off * (unsigned)sizeof(TZ), Z[off]);
     }
+    if constexpr (!mixed) {
+      const unsigned aF = cluster_addr(fbuf(i & 1), 1);
+      for (int r = r0 + G.tid; r < r1; r += G.nt) st_cluster(aF + r * 4u, __int_as_float(rowf[r]));
+    }
   };
   auto rotate = [&](int i, int j, bool withW, Grp G) { cx.rotate(i, j, withW, G); };
 
-  if (producer && mode == kSplit) {
-    // FP64, E- and G-rows on warps 0-3 (the consumer warps run the W-rows)
-    const Grp P{(int)threadIdx.x, kRoleThreads, kBarProd};
-    const int pr1 = n + m;
-    potrf_sm(Dfac, ldD, n, rinv, tab, &bad, false);
-    for (int i = 0; i < g.len; ++i) {
-      const int j = g.f + i;
-      const bool eRows = (i < g.len - 1) || g.hasF;
-      const int r0 = eRows ? 0 : n;
-      if (threadIdx.x == 0 && bad) { record_breakdown(info, d.sys, d.nat[j], d.level); bad = 0; }
-      if (i > 0) group_bar(kBarFreeM, kFactorThreads);
-      panel_operand(M, Dfac, ldD, n, rinv, P);
-      for (int e = P.tid; e < n; e += P.nt) rinvZ[e] = (TZ)rinv[e];
-      gsync(P);
-      group_arrive(kBarFullM, kFactorThreads);
-      trsm_panel(Z, ldZ, r0, pr1, M, ldD, n, rinvZ, P);
-      group_arrive(kBarFullZ, kFactorThreads);
-      if (d.mr) cx.store_y(j, yb, ldyb, P);
-      store_pivot(j, Dfac, rinv, M, P);
-      store_panel(j, r0, pr1, pr1, P);
-      syrk_trap(T, ldT, Z, Z, 0, ldZ, r0, pr1, r0, n, P);
-      if (i + 1 < g.len) {
-        // D_{i+1} is final: factor it now, then rotate the panel once the
-        // consumer has read E-hat_i and G-hat_i
-        copy_blk(Dfac, ldD, T, ldT, n, n, P);
-        gsync(P);
-        potrf_sm(Dfac, ldD, n, rinv, tab, &bad, false);
-        group_bar(kBarFreeZ, kFactorThreads);
-        rotate(i, j, false, P);
-      }
-    }
-  } else if (producer) {
-    // Whole CTA on the E- and G-rows (and the W-rows in the whole layout of a
-    // mixed level; FP64 levels with fill-in rows split or pair). Per stage:
+  if (producer) {
+    // Whole CTA on the E- and G-rows (and the W-rows in the whole layout). Per stage:
     // the fused pivot factorization and panel solve (warps 0-3 and 5-7)
     // while warp 4 writes the previous stage's pivot blocks from the other
     // pivot buffer; then the hand-off to the consumer, the Schur update and
@@ -1060,10 +1076,22 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
         for (int e = P.tid; e < n; e += P.nt) rinvZ[e] = (TZ)rvbuf(cur)[e];
         __syncthreads();
         if (i > 0) cluster_wait();  // the consumer is done with stage i-2 (buffer i % 2)
-        push_stage(i, M, rinvZ, r0, n + m, P);
-        cluster_arrive();
+        push_pivot(i, M, rinvZ, P);
+        if constexpr (mixed) {
+          push_rows(i, r0, n + m, P);
+          cluster_arrive();
+        }
       }
       store_panel(j, r0, pr1, mode == kWhole ? R : n + m, P);
+      if constexpr (!mixed) {
+        __syncthreads();  // the doubles are read
+        oz_encode((double*)Z, ldZ, r0, pr1, n, rowf, P);
+        __syncthreads();
+        if (push) {
+          push_rows(i, r0, n + m, P);
+          cluster_arrive();
+        }
+      }
       bool tc_done = false;
       if constexpr (mixed && TC) {
         if (use_tc) {
@@ -1074,7 +1102,10 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
           tc_done = true;
         }
       }
-      if (!tc_done) syrk_trap(T, ldT, Z, Z, 0, ldZ, r0, pr1, r0, n, P);
+      if constexpr (!mixed)
+        oz_syrk(T, ldT, (double*)Z, rowf, (double*)Z, rowf, 0, ldZ, r0, pr1, r0, n, P);
+      else if (!tc_done)
+        syrk_trap(T, ldT, Z, Z, 0, ldZ, r0, pr1, r0, n, P);
       if (i + 1 < g.len) {
         copy_blk(Dbuf(cur ^ 1), ldD, T, ldT, n, n, P);                      // D_{i+1}
         rotate(i, j, mode == kWhole && g.hasW, P);
@@ -1085,16 +1116,14 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
     if (push) cluster_wait();  // phase of the last stage
   } else if (wr) {
     // fill-in rows W
-    const Grp C = mode == kSplit ? Grp{(int)threadIdx.x - kRoleThreads, kRoleThreads, kBarCons} : cta_grp();
+    const Grp C = cta_grp();
     for (int i = 0; i < g.len; ++i) {
       const int j = g.f + i;
       const bool eRows = (i < g.len - 1) || g.hasF;
       const int r0 = eRows ? 0 : n;
-      const int b = mode == kPair ? (i & 1) : 0;
+      const int b = i & 1;
       const bool own = i == 0 && own0;
-      if (mode == kSplit) {
-        group_bar(kBarFullM, kFactorThreads);
-      } else if (own) {
+      if (own) {
         cluster_arrive();  // (stage -1)
         int bad0 = 0;      // a breakdown is the producer's to report
         potrf_sm(Dfac2c, ldD, n, rinv2c, tab, &bad0);
@@ -1107,7 +1136,6 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
         cluster_wait();    // stage i's blocks are in buffer b
       }
       if (!own) trsm_panel(Z, ldZ, oW, R, Mbuf(b), ldD, n, rinvbuf(b), C);
-      if (mode == kSplit && i + 1 < g.len) group_arrive(kBarFreeM, kFactorThreads);
       {
         double* Pd = d.Lp + (size_t)j * R * n + (size_t)oW * n;
         float* Pf = mixed ? d.Lpf + (size_t)j * R * n + (size_t)oW * n : nullptr;
@@ -1118,10 +1146,17 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
           if (mixed) Pf[e] = (float)v;
         }
       }
-      if (mode == kSplit) group_bar(kBarFullZ, kFactorThreads);
-      syrk_trap(T, ldT, Zbuf(b), Z, oW, ldZ, oW, R, r0, n, C);
+      if constexpr (!mixed) {
+        // (the W-rows' exponents live in buffer 0's array, of which the
+        // producer writes the rows below oW only)
+        __syncthreads();
+        oz_encode((double*)Z, ldZ, oW, R, n, rowf, C);
+        __syncthreads();
+        oz_syrk(T, ldT, (double*)Zbuf(b), fbuf(b), (double*)Z, rowf, oW, ldZ, oW, R, r0, n, C);
+      } else {
+        syrk_trap(T, ldT, Zbuf(b), Z, oW, ldZ, oW, R, r0, n, C);
+      }
       if (i + 1 < g.len) {
-        if (mode == kSplit) group_arrive(kBarFreeZ, kFactorThreads);
         copy_blk(Z + oW * ldZ, ldZ, T + oW * ldT, ldT, n, n, C);               // W_{i+1}
         gsync(C);
         load_blk(T + oW * ldT, ldT, (const double*)nullptr, (const double*)nullptr, n, n, false, C);  // W_{i+2} <- 0
@@ -1248,6 +1283,7 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
   double* const T = cx.T;
   double* const M = cx.M;
   double* const Z = cx.Z;
+  int* const rowf = (int*)(smraw + lay.oF[0]);
   // panel rows [r0, r1): the E-rows when a next separator exists, the G-rows,
   // the W-rows when a previous one does
   const int r0 = g.hasF ? 0 : n, r1 = g.hasW ? cx.R : n + m, h = r1 - r0;
@@ -1330,9 +1366,24 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
     const int ry = oG + m - d.mr;  // the bordered row: y_j of the forward substitution
     if (ry >= t0 && ry < t1) cx.store_y(j, yb, ldyb, cta_grp());
   }
+  // its panel rows to device memory (rank 0 also writes the zero rows [0, r0)),
+  // then in digits to the other CTAs
+  {
+    double* Pd = d.Lp + (size_t)j * cx.R * n;
+    const int p0 = rank == 0 ? 0 : t0;
+    for (int e = tid; e < (t1 - p0) * n; e += nt) {
+      const int r = p0 + e / n, c = e - (r - p0) * n;
+      Pd[(size_t)r * n + c] = r >= r0 ? Z[r * ldZ + c] : 0.0;
+    }
+  }
+  __syncthreads();
+  oz_encode(Z, ldZ, t0, t1, n, rowf, cta_grp());
+  __syncthreads();
   cluster_wait();  // every CTA of the cluster runs
   {
     for (int q = 1; q < C; ++q) {
+      const unsigned af = cluster_addr(rowf, (unsigned)((rank + q) % C));
+      if (tid < t1 - t0) st_cluster(af + (t0 + tid) * 4u, __int_as_float(rowf[t0 + tid]));
       const unsigned az = cluster_addr(Z, (unsigned)((rank + q) % C));
       for (int e = tid; e < (t1 - t0) * n; e += nt) {
         const int r = t0 + e / n, c = e - (r - t0) * n;
@@ -1347,16 +1398,8 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
     if (tid == 0 && bad) record_breakdown(info, d.sys, d.nat[j], d.level);
     cx.store_pivot(j, Dfac, rinv, M, cta_grp());
   }
-  {
-    double* Pd = d.Lp + (size_t)j * cx.R * n;
-    const int p0 = rank == 0 ? 0 : t0;  // rank 0 also writes the zero rows [0, r0)
-    for (int e = tid; e < (t1 - p0) * n; e += nt) {
-      const int r = p0 + e / n, c = e - (r - p0) * n;
-      Pd[(size_t)r * n + c] = r >= r0 ? Z[r * ldZ + c] : 0.0;
-    }
-  }
   cluster_wait();  // every solved panel row is here
-  syrk_trap(T, ldT, Z, Z, 0, ldZ, s0, s1, r0, n, cta_grp());
+  oz_syrk(T, ldT, Z, rowf, Z, rowf, 0, ldZ, s0, s1, r0, n, cta_grp());
   {
     const unsigned a0 = cluster_addr(T, 0u), a1 = cluster_addr(T, 1u);
     const int w0 = s0 - r0;  // row s0 + i holds w0 + i + 1 elements
@@ -3061,7 +3104,7 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
   if (top_solve) sm = std::max(sm, solve_smem_bytes(maxn, maxm, 0, fill));
   const void* fn = mixed ? (pair ? (const void*)k_factor<float, 1>
                                  : tcm ? (const void*)k_factor<float, 4, true> : (const void*)k_factor<float, 4>)
-                          : (pair ? (const void*)k_factor<double, 1> : (const void*)k_factor<double, 4>);
+                          : (pair ? (const void*)k_factor<double, 1> : (const void*)k_factor<double, 2>);
   int e = set_smem(fn, sm);
   if (e) return e;
   if (dbl && !pair && !top_solve) {
@@ -3099,7 +3142,7 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
                                                 dbl, 0);
   return pair ? (int)cudaLaunchKernelEx(&cfg, k_factor<double, 1>, d, t, D, E, G, R, info, p, b, ldb, top_solve,
                                         dbl, 0)
-              : (int)cudaLaunchKernelEx(&cfg, k_factor<double, 4>, d, t, D, E, G, R, info, p, b, ldb, top_solve,
+              : (int)cudaLaunchKernelEx(&cfg, k_factor<double, 2>, d, t, D, E, G, R, info, p, b, ldb, top_solve,
                                         dbl, 0);
 }
 
