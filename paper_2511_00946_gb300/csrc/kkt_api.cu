@@ -235,7 +235,7 @@ struct kkt_handle {
   kkt::PCons* pcons = nullptr;
   Task* ptasks = nullptr;
   int* pready = nullptr;        // [pn] counters, then the ticket
-  int pn = 0, pgrid = 0, pslice = 0, pdbl = 1, pmixed = 0, punmet = 0;
+  int pn = 0, pgrid = 0, pslice = 0, pmixed = 0, punmet = 0;
   size_t psmem = 0;
   long long pwait = 1LL << 31;  // clock cycles a dependency wait may take (about a second)
   std::vector<kkt::PItem> hpitems;
@@ -971,17 +971,8 @@ kkt_status build_persistent(kkt_handle* h) {
   }
   const int slice = any_w ? (int)kkt::factor_w_slice_bytes(wn, wm, mixed, wfill) : 0;
   const int wpc = any_w ? std::max(1, std::min(8, (200 * 1024) / slice)) : 8;
-  int dbl = 1, best_occ = -1;
-  size_t smem = 0;
-  // mixed levels without the second pivot buffer (warp 4 joins the sweep's
-  // workers), FP64 with it unless dropping it lets more CTAs share an SM
-  for (int db = mixed ? 0 : 1; db >= 0; --db) {
-    const size_t sc = any_cta ? kkt::factor_smem_bytes(cn, cm, mixed, cfill, db) : 0;
-    const size_t sm = std::max(sc, (size_t)wpc * slice);
-    const int occ = kkt::persist_occupancy(mixed, sm);
-    if (occ > best_occ) { best_occ = occ; dbl = db; smem = sm; }
-    if (!any_cta) break;
-  }
+  const size_t smem = std::max(any_cta ? kkt::factor_smem_bytes(cn, cm, mixed, cfill) : 0, (size_t)wpc * slice);
+  const int best_occ = kkt::persist_occupancy(mixed, smem);
   if (best_occ < 1) return KKT_ERR_ARG;
   // items
   struct Cand { double cost; std::vector<std::pair<int, int>> tasks; bool warp; };
@@ -1081,7 +1072,6 @@ kkt_status build_persistent(kkt_handle* h) {
   h->pgrid = (int)std::min<long long>((long long)n_it, (long long)best_occ * sms);
   h->psmem = smem;
   h->pslice = slice;
-  h->pdbl = dbl;
   h->pmixed = mixed;
   h->punmet = 0;
   return KKT_OK;
@@ -1166,7 +1156,7 @@ kkt_status kkt_factor(kkt_handle* h, const double* D, const double* E, const dou
   if (h->persistent) {
     if (cudaMemsetAsync(h->pready, 0, sizeof(int) * (h->pn + 1), (cudaStream_t)stream) != cudaSuccess ||
         kkt::launch_factor_persist(h->ddesc, h->ptasks, h->pitems, h->pn, h->pcons, h->pready, h->pmixed, D, E, G, R,
-                                   h->dinfo, h->pgrid, h->psmem, h->pslice, h->pdbl, h->pwait, stream) ||
+                                   h->dinfo, h->pgrid, h->psmem, h->pslice, h->pwait, stream) ||
         !mark(h, 0, stream))
       return KKT_ERR_CUDA;
     h->factored = true;

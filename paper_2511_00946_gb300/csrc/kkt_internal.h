@@ -143,14 +143,11 @@ struct Info {
 // lets more CTAs share an SM; R stays the panel height of the factor in
 // global memory.
 struct FacLayout {
-  int q, R, Rs, ldD, ldZ, ldT, oDfac, oM, oRinv, oRinvZ, oZ, oT, oTab, oDfac2, oRinv2, oCorner, total;
-  int oF[2];  // exponents of split panel rows (kkt_oz.cuh; FP64 CTA tasks), two buffers for a pair's consumer
+  int q, R, Rs, ldD, ldZ, ldT, oDfac, oM, oRinv, oRinvZ, oZ, oT, oTab, oCorner, total;
+  int oDig, oDex, oF[2];  // cta_layout only
 };
 __host__ __device__ inline int kkt_align16(int b) { return (b + 15) & ~15; }
-// `dbl`: a second pivot buffer (and rinv) so that warp 4 can write the
-// previous stage's pivot blocks while the next ones are being factored; a
-// launch goes without it when that lets more CTAs share an SM.
-__host__ __device__ inline FacLayout fac_layout(int n, int m, int zb, bool fill = true, bool dbl = true) {
+__host__ __device__ inline FacLayout fac_layout(int n, int m, int zb, bool fill = true) {
   FacLayout L;
   L.q = n > m ? n : m;
   L.R = 2 * n + m;
@@ -165,24 +162,43 @@ __host__ __device__ inline FacLayout fac_layout(int n, int m, int zb, bool fill 
   L.oZ = L.oRinvZ + kkt_align16(zb * L.q);
   L.oT = L.oZ + kkt_align16(zb * L.Rs * L.ldZ);
   L.oTab = L.oT + kkt_align16(8 * L.Rs * L.ldT);  // potrf element table, q(q-1)/2 ints
-  // second pivot block and rinv: the next stage's pivot factorization runs
-  // while the current stage's factor blocks are still being written
-  L.oDfac2 = L.oTab + kkt_align16(4 * (L.q * (L.q - 1) / 2 + 1));
-  L.oRinv2 = L.oDfac2 + (dbl ? kkt_align16(8 * L.q * L.ldD) : 0);
   // sum of the lower levels' corner partials (m x m), formed before the corner
-  L.oCorner = L.oRinv2 + (dbl ? kkt_align16(8 * L.q) : 0);
-  L.oF[0] = L.oCorner + kkt_align16(8 * kMaxM * kMaxM);
-  L.oF[1] = L.oF[0] + (zb == 8 ? kkt_align16(4 * L.Rs) : 0);
-  L.total = L.oF[1] + (zb == 8 ? kkt_align16(4 * L.Rs) : 0);
+  L.oCorner = L.oTab + kkt_align16(4 * (L.q * (L.q - 1) / 2 + 1));
+  L.total = L.oCorner + kkt_align16(8 * kMaxM * kMaxM);
   return L;
 }
 // One warp's slice for a small-block segment task (k_factor_w): the same
-// blocks without the second pivot buffer, and an m x m corner sum.
+// blocks with an m x m corner sum.
 __host__ __device__ inline FacLayout fac_layout_w(int n, int m, int zb, bool fill = true) {
   FacLayout L = fac_layout(n, m, zb, fill);
-  L.oDfac2 = L.oRinv2 = 0;
-  L.oCorner = L.oTab + kkt_align16(4 * (L.q * (L.q - 1) / 2 + 1));
   L.total = L.oCorner + kkt_align16(8 * (m * m > 0 ? m * m : 1));
+  return L;
+}
+// FP64 segment task of a CTA (k_factor_fp64, k_factor_clus): the pivot block,
+// its panel operand M, the panel and T as above; digit blocks of the sweep
+// (kkt_oz.cuh: eight columns of M and of the panel) with their exponents; the
+// exponents of the solved panel rows, two buffers (a pair's consumer alternates).
+__host__ __device__ inline FacLayout cta_layout(int n, int m, bool fill = true) {
+  FacLayout L{};
+  L.q = n > m ? n : m;
+  L.R = 2 * n + m;
+  L.Rs = fill ? L.R : n + m;
+  L.ldD = L.q | 1;
+  L.ldZ = n | 1;
+  L.ldT = L.Rs | 1;
+  L.oDfac = 0;
+  L.oM = L.oDfac + kkt_align16(8 * L.q * L.ldD);
+  L.oRinv = L.oM + kkt_align16(8 * n * L.ldD);
+  L.oRinvZ = L.oRinv + kkt_align16(8 * L.q);
+  L.oZ = L.oRinvZ + kkt_align16(8 * L.q);
+  L.oT = L.oZ + kkt_align16(8 * L.Rs * L.ldZ);
+  L.oTab = L.oT + kkt_align16(8 * L.Rs * L.ldT);  // the corner's element table
+  L.oDig = L.oTab + kkt_align16(4 * (m * (m - 1) / 2 + 1));
+  L.oDex = L.oDig + 64 * (n + L.Rs);
+  L.oF[0] = L.oDex + kkt_align16(4 * (n + L.Rs));
+  L.oF[1] = L.oF[0] + kkt_align16(4 * L.Rs);
+  L.oCorner = L.oF[1] + kkt_align16(4 * L.Rs);
+  L.total = L.oCorner + kkt_align16(8 * kMaxM * kMaxM);
   return L;
 }
 constexpr int kWarpMaxN = 16;  // largest stage block of the warp-per-task kernels
@@ -388,18 +404,17 @@ int launch_fill_identity(const LevelDesc* d, const int* sys_desc, int count, dou
 // items [0, nitems) over `grid` CTAs with `smem` bytes of shared memory;
 // ready[0..nitems) and the ticket counter ready[nitems] must be zero; a
 // dependency wait gives up after wait_cycles clock cycles (KKT_ERR_TIMEOUT).
-// `slice`: shared memory of one warp task; `dbl`: the CTA tasks keep the
-// second pivot buffer.
+// `slice`: shared memory of one warp task.
 int launch_factor_persist(const LevelDesc* d, const Task* t, const PItem* items, int nitems, const PCons* cons,
                           int* ready, int mixed, const double* D, const double* E, const double* G,
-                          const double* R, Info* info, int grid, size_t smem, int slice, int dbl,
+                          const double* R, Info* info, int grid, size_t smem, int slice,
                           long long wait_cycles, void* stream);
 // the debug build's index-check record (status 8 on a failed check; zero in
 // the normal build); `clear` resets it
 int debug_info(Info* out, int clear);
 // occupancy (CTAs per SM) of the persistent kernel with `smem` bytes
 int persist_occupancy(int mixed, size_t smem);
-size_t factor_smem_bytes(int maxn, int maxm, int mixed, int fill = 1, int dbl = 1);
+size_t factor_smem_bytes(int maxn, int maxm, int mixed, int fill = 1);
 size_t factor_w_slice_bytes(int maxn, int maxm, int mixed, int fill = 1);
 size_t solve_smem_bytes(int maxn, int maxm, int single, int fill = 1);
 

@@ -36,6 +36,15 @@ constexpr int kMaxDevices = 64;  // devices whose kernel attributes are recorded
 
 __device__ __forceinline__ int odd(int c) { return c | 1; }
 
+// e / d for 0 <= e < 2^20 / d (every block: at most 112 x 48 elements, d <= 113)
+// by a multiplication: an integer division costs about 20 instructions, and
+// the block loops below run one per element.
+struct Div {
+  unsigned inv;
+  __device__ __forceinline__ explicit Div(int d) : inv((1u << 20) / (unsigned)d + 1u) {}
+  __device__ __forceinline__ int operator()(int e) const { return (int)((unsigned)e * inv >> 20); }
+};
+
 // Row-by-row enumeration of a lower triangle (diagonal included):
 // e -> (a, b) with 0 <= b <= a, e = a(a+1)/2 + b.
 __device__ __forceinline__ void tri_rc(int e, int& a, int& b) {
@@ -114,9 +123,6 @@ __device__ __forceinline__ Grp cta_grp() { return Grp{(int)threadIdx.x, (int)blo
 __device__ __forceinline__ void group_bar(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
-__device__ __forceinline__ void group_arrive(int id, int nthreads) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 __device__ __forceinline__ void gsync(const Grp& g) {
   if (g.bar == 0) __syncthreads();
   else if (g.bar < 0) __syncwarp();
@@ -136,10 +142,11 @@ template <int U = 1, typename T>
 __device__ void load_blk(T* dst, int ld, const double* A, const double* B, int rows, int cols,
                          bool trans, Grp g = cta_grp()) {
   const int tot = rows * cols;
+  const Div by(trans ? rows : cols);
   auto at = [&](int e) {
     int r, c;
-    if (trans) { c = e / rows; r = e - c * rows; }
-    else { r = e / cols; c = e - r * cols; }
+    if (trans) { c = by(e); r = e - c * rows; }
+    else { r = by(e); c = e - r * cols; }
     return r * ld + c;
   };
   auto batched = [&](auto get) {
@@ -174,10 +181,11 @@ template <typename TD, typename TS>
 __device__ void store_blk(TD* dst, const TS* src, int ld, int rows, int cols, bool trans,
                           bool lower, Grp g = cta_grp()) {
   const int tot = rows * cols;
+  const Div by(trans ? rows : cols);
   for (int e = g.tid; e < tot; e += g.nt) {
     int r, c;
-    if (trans) { c = e / rows; r = e - c * rows; }
-    else { r = e / cols; c = e - r * cols; }
+    if (trans) { c = by(e); r = e - c * rows; }
+    else { r = by(e); c = e - r * cols; }
     TS v = src[r * ld + c];
     if (lower && c > r) v = TS(0);
     dst[e] = (TD)v;
@@ -188,8 +196,9 @@ __device__ void store_blk(TD* dst, const TS* src, int ld, int rows, int cols, bo
 template <typename TD, typename TS>
 __device__ void copy_blk(TD* dst, int ldd, const TS* src, int lds, int rows, int cols,
                          Grp g = cta_grp()) {
+  const Div by(cols);
   for (int e = g.tid; e < rows * cols; e += g.nt) {
-    const int r = e / cols, c = e - r * cols;
+    const int r = by(e), c = e - r * cols;
     dst[r * ldd + c] = (TD)src[r * lds + c];
   }
 }
@@ -264,58 +273,23 @@ __device__ __forceinline__ void potrf_trailing(double* A, int ld, int n, const i
   }
 }
 
-// In-place lower Cholesky by the first four warps (one per FP64 sub-pipe).
-// With `whole`, the CTA's other threads wait at the closing __syncthreads;
-// otherwise only warps 0-3 call it and it closes with their own barrier.
-constexpr int kPotrfThreads = 128;
-constexpr int kPotrfUpd = kPotrfThreads - 32;  // threads of warps 1-3
-
-__device__ void potrf_sm(double* A, int ld, int n, double* rinv, const int* tab, int* bad,
-                         bool whole = true) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid < 32) potrf_col0(A, ld, n, rinv, bad, lane);
-  if (tid < kPotrfThreads) {
-    group_bar(1, kPotrfThreads);
-    for (int j = 0; j + 1 < n; ++j) {
-      if (tid < 32) potrf_lookahead(A, ld, n, rinv, bad, j, lane);
-      else potrf_trailing(A, ld, n, tab, j, tid - 32, kPotrfUpd);
-      group_bar(1, kPotrfThreads);
-    }
-  }
-  if (whole) __syncthreads();
-}
-
-// Fused pivot factorization (FP64) and panel solve (in the panel type TZ:
-// FP64, or FP32 in the mixed variant): the Cholesky above and
-// Z[r0, r1) <- Z[r0, r1) L^{-T} in the division-free form of trsm_panel (the
-// same operations in the same order, so the results are bitwise those of
-// potrf_sm + panel_operand + trsm_panel). Warp 0 runs the pivot chain; in the
-// phase of column j the workers (warps 1-3 and 5-7) run, each as a tight
-// strided loop,
+// Fused pivot factorization (FP64) and panel solve (in the panel type TZ: FP32
+// in the mixed variant) by the whole CTA: the Cholesky above and Z[r0, r1) <-
+// Z[r0, r1) L^{-T} in the division-free form of trsm_panel (the same operations
+// in the same order). Warp 0 runs the pivot chain; in the phase of column j the
+// other warps run, each as a tight strided loop,
 //   - the trailing updates of columns j+2.. by column j,
 //   - the panel operand column M[c][j] = L[c][j] / L[j][j] (c > j),
 //   - the panel updates z_c -= z_{j-1} M[c][j-1] (c >= j) of every row,
 // so the panel lags the factorization by two columns and runs beside the
-// pivot chain instead of after it. x_c = z_c / L_cc closes the sweep. Warp 4 does not take part: it
-// returns at once and may run other work, touching neither A, rinv, M nor
-// panel rows [r0, r1). One named barrier (id 1, 224 threads) per phase; the
-// caller synchronizes the CTA before the results are read.
-constexpr int kFusedThreads = 224;
-constexpr int kFusedWorkers = 192;  // warps 1-3 and 5-7
-
-// all7: warp 4 works too (seven worker warps, a barrier over the whole CTA).
-// A warp's FP64 instructions issue on sub-partition (warp % 4): with warps
-// 1-3 and 5-7 the workers' FP64 work (trailing updates, panel solve) runs on
-// three of the four FP64 pipes while the pivot chain leaves sub-partition 0's
-// nearly idle; with warp 4 on board all four take a share.
+// pivot chain instead of after it. x_c = z_c / L_cc closes the sweep. One
+// barrier per phase; the caller synchronizes the CTA before the results are read.
 template <typename TZ>
 __device__ void potrf_trsm_sm(double* A, int ld, int n, double* rinv, TZ* M, const int* tab, int* bad,
-                              TZ* Z, int ldz, int r0, int r1, bool all7 = false) {
+                              TZ* Z, int ldz, int r0, int r1) {
   const int tid = threadIdx.x, lane = tid & 31;
-  if (!all7 && tid >= kPotrfThreads && tid < kPotrfThreads + 32) return;  // warp 4
-  const int w = all7 ? tid - 32 : (tid < kPotrfThreads ? tid - 32 : tid - 64);  // worker index
-  const int nwk = all7 ? kFactorThreads - 32 : kFusedWorkers;
-  const int nbar = all7 ? kFactorThreads : kFusedThreads;
+  const int w = tid - 32;  // worker index
+  const int nwk = kFactorThreads - 32;
   const int rows = r1 - r0;
   // panel mapping: `per` workers on a row, each on every per-th column
   const int per = rows > 0 ? max(1, nwk / rows) : 0;
@@ -323,7 +297,7 @@ __device__ void potrf_trsm_sm(double* A, int ld, int n, double* rinv, TZ* M, con
   const int pr = pact ? w % rows : 0, pc = pact ? w / rows : 0;
   TZ* zr = Z + (r0 + pr) * ldz;
   if (tid < 32) potrf_col0(A, ld, n, rinv, bad, lane);
-  group_bar(1, nbar);
+  group_bar(1, kFactorThreads);
   for (int j = 0; j < n; ++j) {
     if (tid < 32) {
       if (j + 1 < n) potrf_lookahead(A, ld, n, rinv, bad, j, lane);
@@ -335,7 +309,7 @@ __device__ void potrf_trsm_sm(double* A, int ld, int n, double* rinv, TZ* M, con
         for (int c = j + pc; c < n; c += per) zr[c] = fma(-zj, M[c * ld + j - 1], zr[c]);
       }
     }
-    group_bar(1, nbar);
+    group_bar(1, kFactorThreads);
   }
   if (tid >= 32)
     for (int e = w; e < rows * n; e += nwk) {
@@ -434,26 +408,8 @@ __device__ void syrk_trap(double* T, int ldt, const TZ* Zlo, const TZ* Z, int zs
 // FP64 Schur products on the tensor cores (kkt_oz.cuh).
 // ---------------------------------------------------------------------------
 
-// Panel rows [r0, r1) of Z to digits in place, their exponents to rowf: eight
-// lanes a row. By the whole group; the caller synchronizes before and after.
-__device__ void oz_encode(double* Z, int ldz, int r0, int r1, int n, int* rowf, Grp G) {
-  const int sub = G.tid & 7, span = r0 + ((r1 - r0 + 3) & ~3);  // (whole warps: four rows each)
-  for (int r = r0 + (G.tid >> 3); r < span; r += G.nt >> 3) {
-    oz::u64* z = (oz::u64*)(Z + (r < r1 ? r : r1 - 1) * ldz);
-    int em = 0;
-    for (int k = sub; k < n; k += 8) em = max(em, oz::expo(z[k]));
-    for (int o = 4; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
-    if (r < r1) {
-      const int f = oz::row_exp(em);
-      if (f != oz::kFp64Row)
-        for (int k = sub; k < n; k += 8) z[k] = oz::encode(z[k], f);
-      if (sub == 0) rowf[r] = f;
-    }
-  }
-}
-
 // T[a][b] -= sum_t Z[a][t] Z[b][t] for ra0 <= a < ra1, cb0 <= b <= a (cb0 <=
-// ra0), rows in digits (oz_encode). Panel rows below `zsplit` are read from
+// ra0), rows in digits (panel_out). Panel rows below `zsplit` are read from
 // (Zlo, flo), the others from (Z, fz). One 16 x 8 tile per warp at a time.
 // Every element is an exact sum rounded once, so the result does not depend
 // on the tiling. Ends with the group's barrier.
@@ -463,10 +419,8 @@ __device__ void oz_syrk(double* T, int ldt, const double* Zlo, const int* flo, c
   // row tile i has cols(i) column tiles; this warp takes every nw-th tile
   int i = 0, j = G.tid >> 5;
   for (;;) {
-    int cols;
-    for (;; ++i) {
-      if (ra0 + 16 * i >= ra1) break;
-      cols = (w0 + min(16 * i + 16, ra1 - ra0) + 7) >> 3;
+    for (; ra0 + 16 * i < ra1; ++i) {
+      const int cols = (w0 + min(16 * i + 16, ra1 - ra0) + 7) >> 3;
       if (j < cols) break;
       j -= cols;
     }
@@ -475,6 +429,296 @@ __device__ void oz_syrk(double* T, int ldt, const double* Zlo, const int* flo, c
     j += nw;
   }
   gsync(G);
+}
+
+// ---------------------------------------------------------------------------
+// Pivot factorization and panel solve of one FP64 stage, in blocks of eight
+// columns. Within a block the columns are eliminated in the square-root-free
+// form: with v_c the column after the earlier updates and d_c = v_cc, m_c =
+// v_c / d_c (the panel operand L_rc / L_cc) and v_i -= v_c m_ic. So the chain
+// from one pivot to the next is a shuffle, a reciprocal in integer arithmetic
+// (pivot_rcp), one multiply and one FMA (the lanes keep their own diagonal
+// elements up to date), against six dependent FP64 instructions and a block
+// barrier per column before (1080-1250 cycles a column); 1 / L_cc =
+// 1 / sqrt(d_c) is formed off the chain. The updates of the panel behind a
+// block (u m^T, u the unscaled solution) are tensor-core products of eight
+// columns (oz::tile8); in FP64 FMAs they were most of the sweep's FP64
+// instructions.
+// Schedule: warp 0 eliminates block J. Meanwhile the other warps finish block
+// J - 1: the pivot block's columns beyond block J, the panel's block J - 1
+// (one row per thread, or eight lanes per row where the rows are few) and the
+// panel behind it. Then all warps update the pivot block's next eight columns.
+// ---------------------------------------------------------------------------
+constexpr int kLB = 8;         // columns per block
+constexpr int kBarSweep = 2;   // barrier of warps 1 and up
+struct SweepBuf {              // digit blocks (kLB per row) and their exponents
+  oz::u64 *m, *u;              // panel operand rows, panel rows
+  int *em, *eu;
+};
+__device__ __forceinline__ SweepBuf sweep_buf(unsigned char* sm, const FacLayout& lay, int n) {
+  SweepBuf b;
+  b.m = (oz::u64*)(sm + lay.oDig);
+  b.u = b.m + kLB * n;
+  b.em = (int*)(sm + lay.oDex);
+  b.eu = b.em + n;
+  return b;
+}
+
+// Warp 0: columns [c0, c0 + cn) of the pivot block A (row-major FP64, updated
+// by the blocks before), rows c0 + lane + 32 q: v and d into A, m into M (same
+// ld). Every lane keeps its own row's diagonal element up to date, d_r -=
+// v_rc^2 / d_c with the square formed beforehand, so the chain from pivot to
+// pivot is one shuffle, one reciprocal and one FMA. FULL: cn = kLB. Without SAFE
+// the code has no branch inside (the updates fill the reciprocal's latency:
+// 4.3k cycles a block against 5.5k) and returns false, with nothing written to A,
+// where a pivot fails pivot_rcp_ok; SAFE divides, forms no square and takes any
+// pivot, *bad is then the first column + 1 that is not positive.
+template <int SL, bool FULL, bool SAFE>
+__device__ __forceinline__ bool ldl_block_t(double* A, double* M, int ld, int n, int c0, int cn, int* bad, int lane) {
+  double v[SL][kLB];
+#pragma unroll
+  for (int q = 0; q < SL; ++q) {
+    const int r = c0 + lane + 32 * q;
+#pragma unroll
+    for (int c = 0; c < kLB; ++c) v[q][c] = r < n && (FULL || c < cn) && c0 + c < r ? A[r * ld + c0 + c] : 0.0;
+  }
+  double dg = lane < cn ? A[(c0 + lane) * ld + c0 + lane] : 1.0;  // this lane's diagonal element
+  double vv = v[0][0] * v[0][0];
+  int first = 0;
+  bool ok = true;
+#pragma unroll
+  for (int c = 0; c < kLB; ++c) {
+    if (FULL || c < cn) {  // warp-uniform
+      const double d = __shfl_sync(0xffffffffu, dg, c);
+      double m[SL], dn;
+      if (SAFE) {
+        if (not_positive(d) && first == 0) first = c0 + c + 1;
+#pragma unroll
+        for (int q = 0; q < SL; ++q) m[q] = not_positive(d) ? __longlong_as_double(0x7ff8000000000000LL) : v[q][c] / d;
+        dn = fma(-v[0][c], m[0], dg);
+      } else {
+        ok = ok && pivot_rcp_ok(d);
+        const double ri = pivot_rcp(d);
+        dn = fma(-vv, ri, dg);
+#pragma unroll
+        for (int q = 0; q < SL; ++q) m[q] = v[q][c] * ri;
+      }
+      dg = lane > c ? dn : dg;  // (lane c keeps d)
+#pragma unroll
+      for (int q = 0; q < SL; ++q) {
+        const int r = c0 + lane + 32 * q;
+        if (r < n && r > c0 + c) M[r * ld + c0 + c] = m[q];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int i = c + 1; i < kLB; ++i) {
+        if (FULL || i < cn) {
+          const double mi = M[(c0 + i) * ld + c0 + c];
+#pragma unroll
+          for (int q = 0; q < SL; ++q) v[q][i] = fma(-v[q][c], mi, v[q][i]);
+        }
+        if (!SAFE && i == c + 1) vv = v[0][i] * v[0][i];
+      }
+    }
+  }
+  if (!SAFE && !ok) return false;
+#pragma unroll
+  for (int q = 0; q < SL; ++q) {
+    const int r = c0 + lane + 32 * q;
+#pragma unroll
+    for (int c = 1; c < kLB; ++c)
+      if (r < n && (FULL || c < cn) && c0 + c < r) A[r * ld + c0 + c] = v[q][c];
+  }
+  if (lane < cn) A[(c0 + lane) * ld + c0 + lane] = dg;
+  if (SAFE && lane == 0 && first && *bad == 0) *bad = first;
+  return true;
+}
+__device__ __noinline__ void ldl_block_safe(double* A, double* M, int ld, int n, int c0, int cn, int* bad, int lane) {
+  ldl_block_t<2, false, true>(A, M, ld, n, c0, cn, bad, lane);
+}
+__device__ __forceinline__ void ldl_block(double* A, double* M, int ld, int n, int c0, int cn, int* bad, int lane) {
+  const bool done = cn < kLB      ? ldl_block_t<1, false, false>(A, M, ld, n, c0, cn, bad, lane)
+                    : n - c0 > 32 ? ldl_block_t<2, true, false>(A, M, ld, n, c0, cn, bad, lane)
+                                  : ldl_block_t<1, true, false>(A, M, ld, n, c0, cn, bad, lane);
+  if (!done) ldl_block_safe(A, M, ld, n, c0, cn, bad, lane);
+}
+
+// Columns [c0, c0 + cn) of the panel rows [r0, r1): u_i = z_i - sum_{c < i} u_c
+// m_ic, c in order: one row per thread, or eight lanes per row (a lane per
+// column: 7 shuffle and FMA steps instead of 28 FMAs) where that fits the
+// group at once. The same operations per element.
+__device__ __forceinline__ void ldl_rows(double* Z, int ldz, int r0, int r1, const double* M, int ld, int c0, int cn,
+                                         Grp G) {
+  if (8 * (r1 - r0) <= G.nt) {
+    if ((G.tid & ~31) < 8 * (r1 - r0)) {  // whole warps
+      const int sub = G.tid & 7, r = min(r0 + (G.tid >> 3), r1 - 1);
+      const bool on = sub < cn && r0 + (G.tid >> 3) < r1;
+      double u = on ? Z[r * ldz + c0 + sub] : 0.0;
+      for (int c = 0; c + 1 < cn; ++c) {
+        const double uc = __shfl_sync(0xffffffffu, u, c, 8);
+        const double mi = on && sub > c ? M[(c0 + sub) * ld + c0 + c] : 0.0;
+        const double w = fma(-uc, mi, u);
+        if (sub > c) u = w;
+      }
+      if (on) Z[r * ldz + c0 + sub] = u;
+    }
+    return;
+  }
+  for (int r = r0 + G.tid; r < r1; r += G.nt) {
+    double* z = Z + r * ldz + c0;
+    double u[kLB];
+#pragma unroll
+    for (int c = 0; c < kLB; ++c) u[c] = c < cn ? z[c] : 0.0;
+#pragma unroll
+    for (int c = 0; c < kLB - 1; ++c) {
+      if (c + 1 < cn) {
+#pragma unroll
+        for (int i = c + 1; i < kLB; ++i)
+          if (i < cn) u[i] = fma(-u[c], M[(c0 + i) * ld + c0 + c], u[i]);
+      }
+    }
+#pragma unroll
+    for (int c = 1; c < kLB; ++c)
+      if (c < cn) z[c] = u[c];
+  }
+}
+
+// digits of the eight columns [c0, c0 + kLB) of rows [r0, r1) of src (ld) into
+// dst[(r - r0) kLB ..] with exponents ex[r - r0]; eight lanes a row
+__device__ __forceinline__ void oz_encode8(const double* src, int ld, int c0, int r0, int r1, oz::u64* dst, int* ex,
+                                           Grp G) {
+  const int sub = G.tid & 7, cnt = (r1 - r0 + 3) & ~3;  // (whole warps: four rows each)
+  for (int r = G.tid >> 3; r < cnt; r += G.nt >> 3) {
+    const int rr = min(r0 + r, r1 - 1);
+    const oz::u64 b = oz::dbits(src[rr * ld + c0 + sub]);
+    int em = oz::mag(b);
+    for (int o = 4; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
+    const int f = oz::row_exp(em);
+    if (r0 + r < r1) {
+      dst[r * kLB + sub] = f == oz::kFp64Row ? b : oz::encode(b, f);
+      if (sub == 0) ex[r] = f;
+    }
+  }
+}
+
+// Panel rows [r0, r1) behind the solved block [c0, c0 + kLB): Z[r][c] -= u_r
+// m_c^T for c >= c0 + kLB; by group G, which synchronizes before (u) and after.
+__device__ __forceinline__ void ldl_panel_update(double* Z, int ldz, int n, int r0, int r1, const double* M, int ld,
+                                                 int c0, const SweepBuf& B, Grp G) {
+  const int cb = c0 + kLB, nc = (n - cb + 7) >> 3, nr = (r1 - r0 + 15) >> 4, nw = G.nt >> 5;
+  oz_encode8(Z, ldz, c0, r0, r1, B.u, B.eu, G);
+  oz_encode8(M, ld, c0, cb, n, B.m + cb * kLB, B.em + cb, G);
+  gsync(G);
+  for (int t = G.tid >> 5; t < nr * nc; t += nw) {
+    const int i = t / nc, j = t - i * nc;
+    oz::tile8(Z, ldz, B.u, B.eu, r0, B.m, B.em, 0, r0 + 16 * i, r1, cb + 8 * j, n, G.tid & 31);
+  }
+}
+
+// element (a, b) of the pivot block behind block [c0, c0 + kLB)
+__device__ __forceinline__ void ldl_trail(double* A, const double* M, int ld, int c0, int a, int b) {
+  const double *va = A + a * ld + c0, *mb = M + b * ld + c0;
+  double x = A[a * ld + b];
+#pragma unroll
+  for (int k = 0; k < kLB; ++k) x = fma(-va[k], mb[k], x);
+  A[a * ld + b] = x;
+}
+
+// Pivot factorization of A and panel solve Z[r0, r1) <- Z L^{-T} diag(L) by the
+// whole CTA (at least two warps). On return A holds v (strict lower part, L_rc
+// = v_rc / L_cc) and d on its diagonal, M the panel operand L_rc / L_cc, rinv
+// 1 / L_cc and Z the unscaled solution u (x_c = u_c rinv_c). The inputs are
+// complete on entry; ends with a block barrier.
+__device__ void ldl_sweep(double* A, int ld, int n, double* M, double* rinv, int* bad, double* Z, int ldz, int r0,
+                          int r1, const SweepBuf& B) {
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const Grp W{tid - 32, nt - 32, kBarSweep};
+  for (int c0 = 0; c0 < n + kLB; c0 += kLB) {
+    const int cn = min(kLB, n - c0), cb = c0 + kLB;
+    if (tid < 32) {
+      if (cn > 0) ldl_block(A, M, ld, n, c0, cn, bad, lane);
+    } else if (c0 > 0) {
+      const int p0 = c0 - kLB, pn = min(kLB, n - p0);
+      if (W.tid >= W.nt - kLB && p0 + W.tid - (W.nt - kLB) < n) {
+        const int c = p0 + W.tid - (W.nt - kLB);
+        rinv[c] = pivot_rsqrt(A[c * ld + c]);
+      }
+      // the pivot block behind block J - 1 from column cb on
+      const int h = max(n - cb, 0);
+      for (int e = W.tid; e < h * (h + 1) / 2; e += W.nt) {
+        int a, b;
+        tri_rc(e, a, b);
+        ldl_trail(A, M, ld, p0, cb + a, cb + b);
+      }
+      ldl_rows(Z, ldz, r0, r1, M, ld, p0, pn, W);
+      if (cn > 0) {
+        gsync(W);
+        ldl_panel_update(Z, ldz, n, r0, r1, M, ld, p0, B, W);
+      }
+    }
+    __syncthreads();
+    if (cb < n) {  // the pivot block's next columns
+      const int w = min(kLB, n - cb);
+      for (int e = tid; e < (n - cb) * kLB; e += nt) {
+        const int a = cb + (e >> 3), b = cb + (e & 7);
+        if ((e & 7) < w && b <= a) ldl_trail(A, M, ld, c0, a, b);
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// Panel rows [r0, r1) against a pivot block received as M: the operations of
+// ldl_sweep (u, unscaled). By the whole CTA; ends with a block barrier.
+__device__ void ldl_panel(double* Z, int ldz, int r0, int r1, const double* M, int ld, int n, const SweepBuf& B) {
+  const Grp C = cta_grp();
+  for (int c0 = 0; c0 < n; c0 += kLB) {
+    ldl_rows(Z, ldz, r0, r1, M, ld, c0, min(kLB, n - c0), C);
+    __syncthreads();
+    if (c0 + kLB < n) {
+      ldl_panel_update(Z, ldz, n, r0, r1, M, ld, c0, B, C);
+      __syncthreads();
+    }
+  }
+}
+
+// The solved panel rows [r0, r1): x = u rinv to Pd (row-major, n columns; null
+// ydst: no bordered row, otherwise row ry also to ydst with stride yld), and in
+// digits into Z with the exponents in rowf. Rows [z0, r0) and [r1, z1) of Pd
+// are zeroed. Eight lanes a row; by the whole group, which synchronizes
+// before and after.
+__device__ void panel_out(double* Z, int ldz, int r0, int r1, int n, const double* rinv, int* rowf, double* Pd, int z0,
+                          int z1, int ry, double* ydst, long long yld, Grp G) {
+  const int sub = G.tid & 7, span = r0 + ((r1 - r0 + 3) & ~3);  // (whole warps: four rows each)
+  for (int r = r0 + (G.tid >> 3); r < span; r += G.nt >> 3) {
+    double* z = Z + min(r, r1 - 1) * ldz;
+    double x[kMaxN / 8];
+    int em = 0;
+#pragma unroll
+    for (int q = 0; q < kMaxN / 8; ++q) {
+      const int k = sub + 8 * q;
+      if (8 * q < n) {  // warp-uniform
+        x[q] = k < n ? z[k] * rinv[k] : 0.0;
+        em = max(em, oz::mag(oz::dbits(x[q])));
+      }
+    }
+    for (int o = 4; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
+    const int f = oz::row_exp(em);
+    if (r < r1) {
+      if (sub == 0) rowf[r] = f;
+#pragma unroll
+      for (int q = 0; q < kMaxN / 8; ++q) {
+        const int k = sub + 8 * q;
+        if (k < n) {
+          Pd[(size_t)r * n + k] = x[q];
+          if (ydst && r == ry) ydst[(size_t)k * yld] = x[q];
+          ((oz::u64*)z)[k] = f == oz::kFp64Row ? oz::dbits(x[q]) : oz::encode(oz::dbits(x[q]), f);
+        }
+      }
+    }
+  }
+  for (int e = G.tid + z0 * n; e < r0 * n; e += G.nt) Pd[e] = 0.0;
+  for (int e = G.tid + r1 * n; e < z1 * n; e += G.nt) Pd[e] = 0.0;
 }
 
 // Tensor-core form of the mixed Schur update (whole-CTA layout, eight warps):
@@ -604,8 +848,11 @@ __device__ __forceinline__ void st_cluster(unsigned addr, float v) {
 // waits for one L2 round trip per four steps instead of one per step.
 template <typename Fpart, typename Fout>
 __device__ void sum_partials(Grp G, int nout, int np, Fpart part, Fout out) {
+  // (the split, and with it the order of the sum, of a whole CTA is that of
+  // kFactorThreads threads also where it runs with half of them)
+  const int nt = G.nt == kFactorThreads / 2 ? kFactorThreads : G.nt;
   int sp = 1;
-  while (sp < 32 && sp * 2 * nout <= G.nt) sp *= 2;
+  while (sp < 32 && sp * 2 * nout <= nt) sp *= 2;
   const int groups = G.nt / sp, sub = G.tid & (sp - 1);
   for (int o0 = 0; o0 < nout; o0 += groups) {
     const int o = o0 + G.tid / sp;
@@ -664,14 +911,16 @@ __device__ __forceinline__ SegGeom seg_geom(const LevelDesc& d, int k) {
 // layouts (`mode`):
 //   kWhole  one CTA runs both;
 //   kPair   a cluster of two CTAs (levels with few segments): CTA 0 is the
-//           producer, CTA 1 the consumer, each on an SM of its own, so a
-//           segment gets two SMs' FP64 pipes. After its trsm of stage i the
-//           producer stores M_i, rinv_i, E-hat_i, G-hat_i into buffer i % 2
-//           of the consumer's shared memory and arrives at cluster barrier
-//           phase i; the consumer arrives at phase i when it is done with
-//           stage i-1 and waits for it before stage i; the producer waits for
-//           phase i-1 before it overwrites buffer i % 2 (double buffering).
-//           A last phase, after every remote store, ends the task.
+//           producer, CTA 1 the consumer, each on an SM of its own. After its
+//           panel solve of stage i the producer stores the pivot factor and
+//           the E- and G-rows into buffer i % 2 of the consumer's shared
+//           memory and arrives at cluster barrier phase i; the consumer
+//           arrives at phase i when it is done with stage i-1 and waits for
+//           it before stage i; the producer waits for phase i-1 before it
+//           overwrites buffer i % 2 (double buffering). A last phase, after
+//           every remote store, ends the task.
+// FP64 tasks run factor_task_fp64 (k_factor_fp64, block fixed point), mixed ones
+// (FP32 panel) factor_task (k_factor).
 // ---------------------------------------------------------------------------
 static_assert(kFactorThreads == 256, "the factor roles assume 8 warps per CTA");
 constexpr int kWhole = 0, kPair = 2;
@@ -723,22 +972,13 @@ __device__ int potrf_w(double* A, int ld, int n, double* rinv, const int* tab, i
 // bordered right-hand sides, which are solved against it instead of pivoted
 // (their diagonal is never formed): row r gets (Rs[r][k] - sum_{t<k}
 // Rs[r][t] R-hat[k][t]) / R-hat[k][k], the forward solution y_g of the
-// corner. Writes R-hat (m x m, upper part zero) and 1/diag; group G; the
-// pivot factorization uses warps 0-3 (potrf_sm) or one warp (potrf_w).
-template <bool WARP>
+// corner. Writes R-hat (m x m, upper part zero) and 1/diag. By one warp, G.
 __device__ void corner_factor(double* Rs, int ldR, int m, int mr, double* rinv, int* tab, const LevelDesc& d,
-                              Info* info, int* bad, Grp G) {
+                              Info* info, Grp G) {
   const int mk = m - mr;
-  if (WARP) {
-    pair_table_w(tab, mk, G.tid);
-    const int bd = potrf_w(Rs, ldR, mk, rinv, tab, G.tid);
-    if (G.tid == 0 && bd) record_breakdown(info, d.sys, d.Nnat, d.level);
-  } else if (mk > 0) {
-    potrf_table(tab, mk);
-    __syncthreads();
-    potrf_sm(Rs, ldR, mk, rinv, tab, bad);
-    if (*bad && threadIdx.x == 0) record_breakdown(info, d.sys, d.Nnat, d.level);
-  }
+  pair_table_w(tab, mk, G.tid);
+  const int bd = potrf_w(Rs, ldR, mk, rinv, tab, G.tid);
+  if (G.tid == 0 && bd) record_breakdown(info, d.sys, d.Nnat, d.level);
   // bordered rows: a forward substitution with the corner factor, one row per thread
   for (int r = mk + G.tid; r < m; r += G.nt) {
     double* z = Rs + r * ldR;
@@ -867,13 +1107,46 @@ struct FacCtx {
     for (int e = G.tid; e < n; e += G.nt) dst[(size_t)e * ld] = (double)yr[e];
   }
 
+  // where y_j of a bordered pass goes (stride ld; null without one), as store_y
+  __device__ double* y_dst(int j, double* b, int ldb, long long& ld) const {
+    if (!d->mr) return nullptr;
+    if (d->level == 1) { ld = ldb; return b + (size_t)(d->offB + (long long)j * n) * ldb; }
+    ld = kRhsChunk;
+    return d->X + (size_t)j * n * kRhsChunk;
+  }
+
+  // store_pivot from the square-root-free form: A holds v (L_rc = v_rc rv_c) and
+  // d on its diagonal, Mp the panel operand L_rc / L_cc
+  __device__ void store_pivot_ldl(int j, const double* A, const double* Mp, const double* rv, Grp G) const {
+    double *Ldj = d->Ld + (size_t)j * nn, *LdRj = d->LdR + (size_t)j * nn, *LdMj = d->LdM + (size_t)j * nn;
+    const Div by(n);
+    for (int e = G.tid; e < n * n; e += G.nt) {
+      const int r = by(e), c = e - r * n;
+      if (c > r) {
+        Ldj[e] = 0.0;
+        LdRj[e] = 0.0;
+      }
+      // (LdM is stored transposed: element e is (c, r))
+      LdMj[e] = c > r ? Mp[c * ldD + r] : c == r ? rv[r] : 0.0;
+    }
+    for (int e = G.tid; e < n * (n + 1) / 2; e += G.nt) {
+      int r, c;
+      tri_rc(e, r, c);
+      const double l = A[r * ldD + c] * rv[c], lr = l * rv[r];
+      Ldj[r * n + c] = l;
+      LdRj[r * n + c] = r == c ? rv[r] : lr;
+    }
+    for (int e = G.tid; e < n; e += G.nt) d->Lri[(size_t)j * n + e] = rv[e];
+  }
+
   // panel rows [0, rows) of Lp for stage j: rows outside [r0, r1) are zero
   // (a consumer writes the W-rows of a split or paired segment)
   __device__ void store_panel(int j, int r0, int r1, int rows, Grp G) const {
     double* Pd = d->Lp + (size_t)j * R * n;
     float* Pf = mixed ? d->Lpf + (size_t)j * R * n : nullptr;
+    const Div by(n);
     for (int e = G.tid; e < rows * n; e += G.nt) {
-      const int r = e / n, c = e - r * n;
+      const int r = by(e), c = e - r * n;
       const TZ v = (r >= r0 && r < r1) ? Z[r * ldZ + c] : TZ(0);
       Pd[e] = (double)v;
       if (mixed) Pf[e] = (float)v;
@@ -899,6 +1172,67 @@ struct FacCtx {
     gsync(G);
   }
 
+  // rotate for the FP64 CTA tasks, with D_{i+1} to Dfac: the loads of stage i+1's
+  // E and of D and G of stage i+2 go out first, up to ten per thread, and their
+  // latency passes during the copies within shared memory
+  __device__ void rotate_cta(int i, int j, bool withW, Grp G) const {
+    const bool e1 = (i + 1 < g.len - 1) || g.hasF, d2 = i + 2 < g.len;
+    const double *pE = e1 ? Dp(Ein, j + 1) : nullptr, *pD = d2 ? Dp(Din, j + 2) : nullptr,
+                 *qD = d2 ? Dp(D2, j + 2) : nullptr, *pG = d2 && m ? Gp(Gin, j + 2) : nullptr,
+                 *qG = d2 && m ? Gp(G2, j + 2) : nullptr;
+    constexpr int U = 4;
+    double ve[U], vd[U], vg;
+    auto at = [&](const double* p, const double* q, int e, int tot) {
+      return p && e < tot ? (q ? p[e] + q[e] : p[e]) : 0.0;
+    };
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      ve[u] = at(pE, nullptr, G.tid + u * G.nt, n * n);
+      vd[u] = at(pD, qD, G.tid + u * G.nt, n * n);
+    }
+    vg = at(pG, qG, G.tid, m * n);
+    copy_blk(Dfac, ldD, T, ldT, n, n, G);                                 // D_{i+1}
+    if (m) copy_blk(Z + oG * ldZ, ldZ, T + oG * ldT, ldT, m, n, G);      // G_{i+1}
+    if (withW) copy_blk(Z + oW * ldZ, ldZ, T + oW * ldT, ldT, n, n, G);  // W_{i+1}
+    const Div by(n);
+    if (e1) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = G.tid + u * G.nt, r = by(e);
+        if (e < n * n) Z[r * ldZ + e - r * n] = (TZ)ve[u];
+      }
+      for (int e = G.tid + U * G.nt; e < n * n; e += G.nt) Z[by(e) * ldZ + e - by(e) * n] = (TZ)pE[e];
+    }
+    gsync(G);
+    if (withW) load_blk<1>(T + oW * ldT, ldT, (const double*)nullptr, (const double*)nullptr, n, n, false, G);  // W_{i+2} <- 0
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = G.tid + u * G.nt, r = by(e);
+      if (e < n * n) T[r * ldT + e - r * n] = vd[u];
+    }
+    for (int e = G.tid + U * G.nt; e < n * n; e += G.nt) T[by(e) * ldT + e - by(e) * n] = at(pD, qD, e, n * n);
+    for (int e = G.tid; e < m * n; e += G.nt) {
+      const int r = by(e);
+      T[(oG + r) * ldT + e - r * n] = e < G.nt ? vg : at(pG, qG, e, m * n);
+    }
+    gsync(G);
+  }
+
+  // stages j+1's E and j+2's D and G towards L2 (rotate_cta reads them at the end
+  // of the current stage)
+  __device__ void prefetch_next(int i, int j, Grp G) const {
+    auto pull = [&](const double* p, int cnt) {
+      if (p)
+        for (int e = 16 * G.tid; e < cnt; e += 16 * G.nt) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + e));
+    };
+    if (i + 1 >= g.len) return;
+    if ((i + 1 < g.len - 1) || g.hasF) pull(Dp(Ein, j + 1), n * n);
+    if (i + 2 < g.len) {
+      pull(Dp(Din, j + 2), n * n);
+      if (m) pull(Gp(Gin, j + 2), m * n);
+    }
+  }
+
   // the next level's slots of segment k (not on the top level)
   __device__ void store_slots(int k, bool eg, bool wr, Grp G) const {
     if (eg && g.hasF) {
@@ -921,15 +1255,189 @@ template <typename TS>
 __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs, double* b, int ldb, int nr,
                              const int* skip, unsigned char* smraw, Grp G, int fwd_done, int c0 = 0);
 
+// One FP64 segment task by the whole CTA or, with `pair`, by this CTA's half
+// of a two-CTA cluster: the body of k_factor_fp64, also run task after task by
+// the persistent kernel. In a pair CTA 0 runs the chain (pivot, E- and
+// G-rows), CTA 1 the fill-in rows one stage behind with the panel operand and
+// the E- and G-rows received through distributed shared memory (buffer i % 2);
+// see the roles above. Every element is computed by the same operations
+// whatever the layout.
+__device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc* __restrict__ descs,
+                                               const double* __restrict__ uD, const double* __restrict__ uE,
+                                               const double* __restrict__ uG, const double* __restrict__ uR,
+                                               Info* info, int pair, double* yb, int ldyb, int top_solve,
+                                               unsigned char* smraw, int& bad) {
+  const unsigned rank = pair ? cluster_rank() : 0u;
+  const LevelDesc& d = descs[tk.desc];
+  const FacLayout lay = cta_layout(d.n, d.m, d.P > 1);
+  if (!task_geometry_ok(d, tk.seg, smraw, lay.total)) return;  // debug build only (both CTAs of a pair alike)
+  const FacCtx<double, 4> cx(d, tk.seg, smraw, lay, uD, uE, uG);
+  const int n = cx.n, m = cx.m, R = cx.R, ldD = cx.ldD, ldZ = cx.ldZ, ldT = cx.ldT, oG = cx.oG, oW = cx.oW;
+  double* const Dfac = cx.Dfac;
+  double* const rinv = cx.rinv;
+  double* const T = cx.T;
+  double* const Z = cx.Z;
+  double* const M = cx.M;
+  const SegGeom g = cx.g;
+  // the consumer's buffer 1 reuses the pivot block, rinv and the first rows of
+  // T, which a consumer CTA has no other use for
+  auto Mbuf = [&](int b) { return b ? Dfac : M; };
+  auto rinvbuf = [&](int b) { return b ? rinv : cx.rinvZ; };
+  auto Zbuf = [&](int b) { return b ? T : Z; };
+  auto fbuf = [&](int b) { return (int*)(smraw + lay.oF[b]); };  // exponents of the solved rows
+  int* const rowf = fbuf(0);
+  const SweepBuf SB = sweep_buf(smraw, lay, n);
+  const bool eg = !pair || rank == 0;             // this CTA holds the E/G rows
+  const bool wr = g.hasW && (!pair || rank == 1);  // this CTA holds the W rows
+  const Grp C = cta_grp();
+  if (threadIdx.x == 0) bad = 0;
+  for (int e = threadIdx.x; e < lay.Rs * ldT; e += blockDim.x) T[e] = 0.0;
+  __syncthreads();
+  cx.load_first(eg, wr, C);
+  __syncthreads();
+  if (pair) {
+    // both CTAs have started before any remote store
+    cluster_arrive();
+    cluster_wait();
+  }
+  if (eg) {
+    const int pr1 = n + m + (wr ? n : 0);  // end of the CTA's panel rows
+    const bool push = pair && g.hasW;
+    for (int i = 0; i < g.len; ++i) {
+      const int j = g.f + i;
+      const bool eRows = (i < g.len - 1) || g.hasF;
+      const int r0 = eRows ? 0 : n;
+      if (d.level == 1) cx.prefetch_next(i, j, C);
+      ldl_sweep(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, r0, pr1, SB);
+      if (threadIdx.x == 0 && bad) { record_breakdown(info, d.sys, d.nat[j], d.level); bad = 0; }
+      long long yld = 1;
+      double* const yd = cx.y_dst(j, yb, ldyb, yld);
+      panel_out(Z, ldZ, r0, pr1, n, rinv, rowf, d.Lp + (size_t)j * R * n, 0, pair ? n + m : R, oG + m - d.mr, yd, yld, C);
+      __syncthreads();
+      if (push) {
+        if (i > 0) cluster_wait();  // the consumer is done with stage i-2 (buffer i % 2)
+        const int b = i & 1;
+        const unsigned aM = cluster_addr(Mbuf(b), 1), aR = cluster_addr(rinvbuf(b), 1), aF = cluster_addr(fbuf(b), 1),
+                       aZ = cluster_addr(Zbuf(b), 1);
+        for (int e = C.tid; e < (n - 1) * n / 2; e += C.nt) {
+          int a, c;
+          tri_rc(e, a, c);
+          const int off = (a + 1) * ldD + c;
+          st_cluster(aM + off * 8u, M[off]);
+        }
+        for (int e = C.tid; e < n; e += C.nt) st_cluster(aR + e * 8u, rinv[e]);
+        for (int e = r0 + C.tid; e < n + m; e += C.nt) st_cluster(aF + e * 4u, __int_as_float(rowf[e]));
+        for (int e = C.tid; e < (n + m - r0) * n; e += C.nt) {
+          const int r = r0 + e / n, c = e - (r - r0) * n;
+          st_cluster(aZ + (r * ldZ + c) * 8u, Z[r * ldZ + c]);
+        }
+        cluster_arrive();
+      }
+      cx.store_pivot_ldl(j, Dfac, M, rinv, C);
+      oz_syrk(T, ldT, Z, rowf, Z, rowf, 0, ldZ, r0, pr1, r0, n, C);
+      if (i + 1 < g.len) cx.rotate_cta(i, j, wr, C);
+    }
+    if (push) cluster_wait();  // phase of the last stage
+  } else if (wr) {
+    // fill-in rows W of a pair
+    for (int i = 0; i < g.len; ++i) {
+      const int j = g.f + i;
+      const bool eRows = (i < g.len - 1) || g.hasF;
+      const int r0 = eRows ? 0 : n, b = i & 1;
+      cluster_arrive();  // done with stage i-1
+      cluster_wait();    // stage i's blocks are in buffer b
+      ldl_panel(Z, ldZ, oW, R, Mbuf(b), ldD, n, SB);
+      // (the W-rows' exponents live in buffer 0's array, of which the producer
+      // writes the rows below oW only)
+      panel_out(Z, ldZ, oW, R, n, rinvbuf(b), rowf, d.Lp + (size_t)j * R * n, oW, R, -1, nullptr, 1, C);
+      __syncthreads();
+      oz_syrk(T, ldT, Zbuf(b), fbuf(b), Z, rowf, oW, ldZ, oW, R, r0, n, C);
+      if (i + 1 < g.len) {
+        copy_blk(Z + oW * ldZ, ldZ, T + oW * ldT, ldT, n, n, C);  // W_{i+1}
+        gsync(C);
+        load_blk(T + oW * ldT, ldT, (const double*)nullptr, (const double*)nullptr, n, n, false, C);  // W_{i+2} <- 0
+        gsync(C);
+      }
+    }
+  }
+  __syncthreads();
+
+  if (!d.is_top) {
+    cx.store_slots(tk.seg, eg, wr, C);
+  } else if (m) {
+    // corner: R-hat = chol(R + sum_k R~_k over every level), in a fixed order:
+    // the lower levels' partials are summed by the pair's idle CTA while this
+    // one runs the stages (or here, without a pair), then R and this level's
+    // own partial are added
+    double* Psum = (double*)(smraw + lay.oCorner);
+    auto part = [&](int p, int o) { return d.Rpart_all[(size_t)p * m * m + o]; };
+    if (pair && rank == 1) {
+      const unsigned aP = cluster_addr(Psum, 0);
+      sum_partials(C, m * m, d.nRpart_all, part,
+                   [&](int o, double v) { st_cluster(aP + o * (unsigned)sizeof(double), v); });
+    } else if (!pair) {
+      sum_partials(C, m * m, d.nRpart_all, part, [&](int o, double v) { Psum[o] = v; });
+    }
+    if (pair) {
+      cluster_arrive();
+      cluster_wait();
+    } else {
+      __syncthreads();
+    }
+  }
+  if (d.is_top && eg && m) {
+    double* Psum = (double*)(smraw + lay.oCorner);
+    double* Rs = Dfac;  // reuse
+    const int ldR = odd(m);
+    const double* Ru = uR + d.offR;
+    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+      const int r = e / m, c = e - r * m;
+      Rs[r * ldR + c] = (Ru[e] + Psum[e]) + T[(oG + r) * ldT + oG + c];
+    }
+    __syncthreads();
+    // by one warp: at m <= 16 a per-column block barrier costs more than the
+    // column's work
+    if (threadIdx.x < 32)
+      corner_factor(Rs, ldR, m, d.mr, rinv, cx.tab, d, info, Grp{(int)threadIdx.x, 32, -1});
+    __syncthreads();
+  }
+  // bordered pass, top level: the corner solve x_g = R-hat^{-T} y_g and the
+  // backward sweep of the top level's stages (Algorithm 3, sequential phase)
+  // here instead of in a launch of their own; the blocks it reads were
+  // written by this CTA, and the shared memory is free by now
+  if (top_solve && d.is_top && d.mr && yb && eg) {
+    __syncthreads();
+    forward_task<double>(tk, descs, yb, ldyb, 1, nullptr, smraw, C, 1);
+  }
+  if (pair) {
+    // a segment without fill-in leaves its consumer idle; every CTA of the
+    // pair then meets once more, after which no remote store is in flight
+    cluster_arrive();
+    cluster_wait();
+  }
+}
+
+// Two CTAs of 256 threads per SM: up to 128 registers (the products' fragments).
+__global__ void __launch_bounds__(kFactorThreads, 2) k_factor_fp64(const LevelDesc* __restrict__ descs,
+                                                                 const Task* __restrict__ tasks,
+                                                                 const double* __restrict__ uD,
+                                                                 const double* __restrict__ uE,
+                                                                 const double* __restrict__ uG,
+                                                                 const double* __restrict__ uR, Info* info, int pair,
+                                                                 double* yb, int ldyb, int top_solve) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ int bad;
+  factor_task_fp64(tasks[pair ? blockIdx.x >> 1 : blockIdx.x], descs, uD, uE, uG, uR, info, pair, yb, ldyb, top_solve,
+                   smraw, bad);
+}
+
 // MINB: CTAs per SM the register allocation must allow. Launches of CTA pairs
-// (one CTA per SM, latency-bound) take the unconstrained allocation (1), the
-// FP64 launches two (128 registers: the fragments and accumulators of a digit
-// product; with three CTAs and 80 registers they spill: 67.1 against 63.8 ms
-// on 4096 uneven systems), the mixed ones four (at most 64 registers), so that
-// several segment CTAs share an SM when shared memory allows it.
+// (one CTA per SM, latency-bound) take the unconstrained allocation (1);
+// the others four (at most 64 registers), so that several segment CTAs share
+// an SM when shared memory allows it.
 // TC: the instantiation with the tensor-core Schur products (mixed launches
 // that use them); the others carry none of that code.
-// One segment task of the factorization by the whole CTA (or, with `pair`,
+// One segment task of the mixed factorization (TZ = float) by the whole CTA (or, with `pair`,
 // by this CTA's half of a two-CTA cluster): the body of k_factor, also run
 // task after task by the persistent kernel. `bad`, `tslot`, `tbar`: shared
 // variables of the caller (breakdown flag, TMEM address slot, mbarrier).
@@ -937,13 +1445,13 @@ template <typename TZ, bool TC>
 __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __restrict__ descs,
                                             const double* __restrict__ uD, const double* __restrict__ uE,
                                             const double* __restrict__ uG, const double* __restrict__ uR,
-                                            Info* info, int pair, double* yb, int ldyb, int top_solve, int dbl,
+                                            Info* info, int pair, double* yb, int ldyb,
                                             int tcm, unsigned char* smraw, int& bad, uint32_t& tslot,
                                             uint64_t& tbar) {
   const unsigned rank = pair ? cluster_rank() : 0u;
   const LevelDesc& d = descs[tk.desc];
   constexpr bool mixed = sizeof(TZ) == 4;
-  const FacLayout lay = fac_layout(d.n, d.m, (int)sizeof(TZ), d.P > 1, dbl != 0);
+  const FacLayout lay = fac_layout(d.n, d.m, (int)sizeof(TZ), d.P > 1);
   if (!task_geometry_ok(d, tk.seg, smraw, lay.total)) return;  // debug build only (both CTAs of a pair alike)
   const FacCtx<TZ, 4> cx(d, tk.seg, smraw, lay, uD, uE, uG);
   const int n = cx.n, m = cx.m, R = cx.R, ldD = cx.ldD, ldZ = cx.ldZ, ldT = cx.ldT, oG = cx.oG, oW = cx.oW;
@@ -962,14 +1470,12 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
   auto Mbuf = [&](int b) { return b ? (TZ*)Dfac : M; };
   auto rinvbuf = [&](int b) { return b ? (TZ*)rinv : rinvZ; };
   auto Zbuf = [&](int b) { return b ? (TZ*)T : Z; };
-  auto fbuf = [&](int b) { return (int*)(smraw + lay.oF[b]); };  // exponents of split rows (FP64)
-  int* const rowf = fbuf(0);
   const bool eg = mode != kPair || rank == 0;       // this CTA holds the E/G rows
   const bool wr = g.hasW && (mode != kPair || rank == 1);  // this CTA holds the W rows
 
-  // tensor-core Schur products (mixed whole-CTA layout without the second
-  // pivot buffer, whose region then stages the operands)
-  const bool use_tc = TC && mixed && tcm && mode == kWhole && !dbl;
+  // tensor-core Schur products (mixed whole-CTA layout; the pivot buffers'
+  // region stages the operands)
+  const bool use_tc = TC && mixed && tcm && mode == kWhole;
   const uint32_t tc_cols = ((lay.Rs + 15) & ~15) <= 64 ? 64u : 128u;
   uint32_t tmem = 0u, tphase = 0u;
   if constexpr (TC) {
@@ -979,17 +1485,9 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
       tc::fence_before();
     }
   }
-  // An FP64 pair's consumer factors the first stage's pivot block as well,
-  // in the second pivot buffer (no hand-off ever writes there), so that its
-  // W-rows' panel solve of that stage runs while the producer's sweep and
-  // hand-off are still under way; the result is bitwise the producer's
-  // (potrf_sm + panel_operand is the fused sweep's arithmetic).
-  const bool own0 = mode == kPair && rank == 1 && g.hasW && dbl && !mixed;
-  double* const Dfac2c = (double*)(smraw + lay.oDfac2);
-  double* const rinv2c = (double*)(smraw + lay.oRinv2);
   if (threadIdx.x == 0) bad = 0;
   for (int e = threadIdx.x; e < lay.Rs * ldT; e += blockDim.x) T[e] = 0.0;
-  if (eg || own0) potrf_table(tab, n);
+  if (eg) potrf_table(tab, n);
   __syncthreads();
   if constexpr (TC) {
     if (use_tc) {
@@ -998,7 +1496,6 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
     }
   }
   cx.load_first(eg, wr, cta_grp());
-  if (own0) cx.load_D(Dfac2c, g.f, cta_grp());
   __syncthreads();
   if (mode == kPair) {
     // both CTAs have started before any remote store
@@ -1011,11 +1508,12 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
     cx.store_pivot(j, Dp_, rv, Ms, G);
   };
   auto store_panel = [&](int j, int r0, int r1, int rows, Grp G) { cx.store_panel(j, r0, r1, rows, G); };
-  // hand the trsm operand (strict lower triangle of Msrc, ld ldD) and its
-  // 1/diag of stage i to the consumer CTA of a pair; then panel rows [r0, r1)
-  // (FP64: in digits, with their exponents)
-  auto push_pivot = [&](int i, const TZ* Msrc, const TZ* rsrc, Grp G) {
-    const unsigned aM = cluster_addr(Mbuf(i & 1), 1), aR = cluster_addr(rinvbuf(i & 1), 1);
+  // hand the trsm operand (strict lower triangle of Msrc, ld ldD), its
+  // 1/diag and panel rows [r0, r1) of stage i to the consumer CTA of a pair
+  auto push_stage = [&](int i, const TZ* Msrc, const TZ* rsrc, int r0, int r1, Grp G) {
+    const int b = i & 1;
+    const unsigned aM = cluster_addr(Mbuf(b), 1), aR = cluster_addr(rinvbuf(b), 1),
+                   aZ = cluster_addr(Zbuf(b), 1);
     const int ntri = (n - 1) * n / 2;
     for (int e = G.tid; e < ntri; e += G.nt) {
       int a, c;
@@ -1024,74 +1522,38 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
       st_cluster(aM + off * (unsigned)sizeof(TZ), Msrc[off]);
     }
     for (int e = G.tid; e < n; e += G.nt) st_cluster(aR + e * (unsigned)sizeof(TZ), rsrc[e]);
-  };
-  auto push_rows = [&](int i, int r0, int r1, Grp G) {
-    const unsigned aZ = cluster_addr(Zbuf(i & 1), 1);
     for (int e = G.tid; e < (r1 - r0) * n; e += G.nt) {
       const int r = r0 + e / n, c = e - (r - r0) * n;
       const int off = r * ldZ + c;
       st_cluster(aZ + off * (unsigned)sizeof(TZ), Z[off]);
     }
-    if constexpr (!mixed) {
-      const unsigned aF = cluster_addr(fbuf(i & 1), 1);
-      for (int r = r0 + G.tid; r < r1; r += G.nt) st_cluster(aF + r * 4u, __int_as_float(rowf[r]));
-    }
   };
   auto rotate = [&](int i, int j, bool withW, Grp G) { cx.rotate(i, j, withW, G); };
 
   if (producer) {
-    // Whole CTA on the E- and G-rows (and the W-rows in the whole layout). Per stage:
-    // the fused pivot factorization and panel solve (warps 0-3 and 5-7)
-    // while warp 4 writes the previous stage's pivot blocks from the other
-    // pivot buffer; then the hand-off to the consumer, the Schur update and
-    // the rotation.
+    // Whole CTA on the E- and G-rows (and the W-rows in the whole layout). Per
+    // stage: the fused pivot factorization and panel solve, the pivot blocks'
+    // store, then the hand-off to the consumer, the Schur update and the rotation.
     const Grp P = cta_grp();
-    const Grp W4{(int)(threadIdx.x & 31), 32, -1};
-    const bool w4 = (threadIdx.x >> 5) == 4;
     const int pr1 = n + m + (mode == kWhole && g.hasW ? n : 0);  // end of the CTA's panel rows
     const bool push = mode == kPair && g.hasW;
-    double* const Dfac2 = (double*)(smraw + lay.oDfac2);
-    double* const rinv2 = (double*)(smraw + lay.oRinv2);
-    // without the second pivot buffer (dbl = 0) the pivot blocks of a stage
-    // are written by the whole CTA right after its sweep
-    auto Dbuf = [&](int b) { return b && dbl ? Dfac2 : Dfac; };
-    auto rvbuf = [&](int b) { return b && dbl ? rinv2 : rinv; };
     for (int i = 0; i < g.len; ++i) {
       const int j = g.f + i;
-      const int cur = i & 1;
       const bool eRows = (i < g.len - 1) || g.hasF;
       const int r0 = eRows ? 0 : n;
-      if (!dbl) {
-        potrf_trsm_sm(Dbuf(cur), ldD, n, rvbuf(cur), M, tab, &bad, Z, ldZ, r0, pr1, true);
-      } else if (w4) {
-        if (i > 0) store_pivot(j - 1, Dbuf(cur ^ 1), rvbuf(cur ^ 1), nullptr, W4);
-      } else {
-        potrf_trsm_sm(Dbuf(cur), ldD, n, rvbuf(cur), M, tab, &bad, Z, ldZ, r0, pr1);
-      }
+      potrf_trsm_sm(Dfac, ldD, n, rinv, M, tab, &bad, Z, ldZ, r0, pr1);
       __syncthreads();
       if (threadIdx.x == 0 && bad) { record_breakdown(info, d.sys, d.nat[j], d.level); bad = 0; }
-      if (!dbl) store_pivot(j, Dfac, rinv, nullptr, P);  // read before the copy of D_{i+1} below
+      store_pivot(j, Dfac, rinv, nullptr, P);  // read before the copy of D_{i+1} below
       if (d.mr) cx.store_y(j, yb, ldyb, P);
       if (push) {
-        for (int e = P.tid; e < n; e += P.nt) rinvZ[e] = (TZ)rvbuf(cur)[e];
+        for (int e = P.tid; e < n; e += P.nt) rinvZ[e] = (TZ)rinv[e];
         __syncthreads();
         if (i > 0) cluster_wait();  // the consumer is done with stage i-2 (buffer i % 2)
-        push_pivot(i, M, rinvZ, P);
-        if constexpr (mixed) {
-          push_rows(i, r0, n + m, P);
-          cluster_arrive();
-        }
+        push_stage(i, M, rinvZ, r0, n + m, P);
+        cluster_arrive();
       }
       store_panel(j, r0, pr1, mode == kWhole ? R : n + m, P);
-      if constexpr (!mixed) {
-        __syncthreads();  // the doubles are read
-        oz_encode((double*)Z, ldZ, r0, pr1, n, rowf, P);
-        __syncthreads();
-        if (push) {
-          push_rows(i, r0, n + m, P);
-          cluster_arrive();
-        }
-      }
       bool tc_done = false;
       if constexpr (mixed && TC) {
         if (use_tc) {
@@ -1102,15 +1564,10 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
           tc_done = true;
         }
       }
-      if constexpr (!mixed)
-        oz_syrk(T, ldT, (double*)Z, rowf, (double*)Z, rowf, 0, ldZ, r0, pr1, r0, n, P);
-      else if (!tc_done)
-        syrk_trap(T, ldT, Z, Z, 0, ldZ, r0, pr1, r0, n, P);
+      if (!tc_done) syrk_trap(T, ldT, Z, Z, 0, ldZ, r0, pr1, r0, n, P);
       if (i + 1 < g.len) {
-        copy_blk(Dbuf(cur ^ 1), ldD, T, ldT, n, n, P);                      // D_{i+1}
+        copy_blk(Dfac, ldD, T, ldT, n, n, P);  // D_{i+1}
         rotate(i, j, mode == kWhole && g.hasW, P);
-      } else if (dbl) {
-        store_pivot(j, Dbuf(cur), rvbuf(cur), nullptr, P);
       }
     }
     if (push) cluster_wait();  // phase of the last stage
@@ -1122,20 +1579,9 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
       const bool eRows = (i < g.len - 1) || g.hasF;
       const int r0 = eRows ? 0 : n;
       const int b = i & 1;
-      const bool own = i == 0 && own0;
-      if (own) {
-        cluster_arrive();  // (stage -1)
-        int bad0 = 0;      // a breakdown is the producer's to report
-        potrf_sm(Dfac2c, ldD, n, rinv2c, tab, &bad0);
-        panel_operand(Dfac2c, Dfac2c, ldD, n, rinv2c, cta_grp());  // in place: M_cj = L_cj / L_jj
-        __syncthreads();
-        trsm_panel(Z, ldZ, oW, R, (const TZ*)Dfac2c, ldD, n, (const TZ*)rinv2c, cta_grp());
-        cluster_wait();    // stage 0's E- and G-rows are in buffer 0
-      } else {
-        cluster_arrive();  // done with stage i-1
-        cluster_wait();    // stage i's blocks are in buffer b
-      }
-      if (!own) trsm_panel(Z, ldZ, oW, R, Mbuf(b), ldD, n, rinvbuf(b), C);
+      cluster_arrive();  // done with stage i-1
+      cluster_wait();    // stage i's blocks are in buffer b
+      trsm_panel(Z, ldZ, oW, R, Mbuf(b), ldD, n, rinvbuf(b), C);
       {
         double* Pd = d.Lp + (size_t)j * R * n + (size_t)oW * n;
         float* Pf = mixed ? d.Lpf + (size_t)j * R * n + (size_t)oW * n : nullptr;
@@ -1146,16 +1592,7 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
           if (mixed) Pf[e] = (float)v;
         }
       }
-      if constexpr (!mixed) {
-        // (the W-rows' exponents live in buffer 0's array, of which the
-        // producer writes the rows below oW only)
-        __syncthreads();
-        oz_encode((double*)Z, ldZ, oW, R, n, rowf, C);
-        __syncthreads();
-        oz_syrk(T, ldT, (double*)Zbuf(b), fbuf(b), (double*)Z, rowf, oW, ldZ, oW, R, r0, n, C);
-      } else {
-        syrk_trap(T, ldT, Zbuf(b), Z, oW, ldZ, oW, R, r0, n, C);
-      }
+      syrk_trap(T, ldT, Zbuf(b), Z, oW, ldZ, oW, R, r0, n, C);
       if (i + 1 < g.len) {
         copy_blk(Z + oW * ldZ, ldZ, T + oW * ldT, ldT, n, n, C);               // W_{i+1}
         gsync(C);
@@ -1200,20 +1637,10 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
     }
     __syncthreads();
     // by one warp: at m <= 16 a per-column block barrier costs more than the
-    // column's work (the operations per element are potrf_sm's)
+    // column's work
     if (threadIdx.x < 32)
-      corner_factor<true>(Rs, ldR, m, d.mr, rinv, tab, d, info, nullptr, Grp{(int)threadIdx.x, 32, -1});
+      corner_factor(Rs, ldR, m, d.mr, rinv, tab, d, info, Grp{(int)threadIdx.x, 32, -1});
     __syncthreads();
-  }
-  if constexpr (!mixed) {
-    // bordered pass, top level: the corner solve x_g = R-hat^{-T} y_g and the
-    // backward sweep of the top level's stages (Algorithm 3, sequential
-    // phase) here instead of in a launch of their own; the blocks it reads
-    // were written by this CTA, and the shared memory is free by now
-    if (top_solve && d.is_top && d.mr && yb && eg) {
-      __syncthreads();
-      forward_task<double>(tk, descs, yb, ldyb, 1, nullptr, smraw, cta_grp(), 1);
-    }
   }
   if (mode == kPair) {
     // a segment without fill-in leaves its consumer idle; every CTA of the
@@ -1238,13 +1665,13 @@ __global__ void __launch_bounds__(kFactorThreads, MINB) k_factor(const LevelDesc
                                                            const double* __restrict__ uG,
                                                            const double* __restrict__ uR,
                                                            Info* info, int pair, double* yb, int ldyb,
-                                                           int top_solve, int dbl, int tcm) {
+                                                           int tcm) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int bad;
   __shared__ uint32_t tslot;               // TMEM address of the tensor-core accumulator
   __shared__ __align__(8) uint64_t tbar;   // its completion mbarrier
   factor_task<TZ, TC>(tasks[pair ? blockIdx.x >> 1 : blockIdx.x], descs, uD, uE, uG, uR, info, pair, yb, ldyb,
-                      top_solve, dbl, tcm, smraw, bad, tslot, tbar);
+                      tcm, smraw, bad, tslot, tbar);
 }
 
 // ---------------------------------------------------------------------------
@@ -1255,7 +1682,7 @@ __global__ void __launch_bounds__(kFactorThreads, MINB) k_factor(const LevelDesc
 // panel solve and Schur update (Alg. 1) run at two FP64 FMAs per clock per
 // SM. Here the stage is spread over the cluster:
 //   - every CTA factors the pivot block itself and solves a contiguous band
-//     of about 1/C of the panel rows with the fused sweep (potrf_trsm_sm),
+//     of about 1/C of the panel rows (ldl_sweep),
 //     then stores its solved rows into every other CTA's shared memory;
 //   - every CTA applies the Schur update to a band of trapezoid rows holding
 //     about 1/C of the elements and stores the results into the shared
@@ -1272,7 +1699,7 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
                                           unsigned char* smraw, int& bad) {
   const int rank = (int)cluster_rank();
   const LevelDesc& d = descs[tk.desc];
-  const FacLayout lay = fac_layout(d.n, d.m, 8, true, false);
+  const FacLayout lay = cta_layout(d.n, d.m);
   if (!task_geometry_ok(d, tk.seg, smraw, lay.total)) return;  // debug build only (every CTA alike)
   const FacCtx<double, 4> cx(d, tk.seg, smraw, lay, uD, uE, uG);
   const int n = cx.n, m = cx.m, ldD = cx.ldD, ldZ = cx.ldZ, ldT = cx.ldT, oG = cx.oG, oW = cx.oW;
@@ -1301,7 +1728,6 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
   const int s0 = band0(rank), s1 = band0(rank + 1);
   cluster_arrive();  // this CTA runs: the others may store into its shared memory after their wait
   if (tid == 0) bad = 0;
-  potrf_table(cx.tab, n);
   // inputs: the pivot block D_j, the panel rows of the solve band, and the
   // initial values of the Schur band (A_k and Q_k^T in its W-rows, zero
   // elsewhere). Every load is an L2 round trip, so the three sets form one
@@ -1360,30 +1786,22 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
     }
   }
   __syncthreads();
-  potrf_trsm_sm(Dfac, ldD, n, rinv, M, cx.tab, &bad, Z, ldZ, t0, t1, true);
-  __syncthreads();
-  if (d.mr) {
-    const int ry = oG + m - d.mr;  // the bordered row: y_j of the forward substitution
-    if (ry >= t0 && ry < t1) cx.store_y(j, yb, ldyb, cta_grp());
-  }
-  // its panel rows to device memory (rank 0 also writes the zero rows [0, r0)),
-  // then in digits to the other CTAs
+  ldl_sweep(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, t0, t1, sweep_buf(smraw, lay, n));
+  // its panel rows to device memory (rank 0 also writes the zero rows [0, r0);
+  // the bordered row is y_j of the forward substitution), then in digits to the
+  // other CTAs
   {
-    double* Pd = d.Lp + (size_t)j * cx.R * n;
-    const int p0 = rank == 0 ? 0 : t0;
-    for (int e = tid; e < (t1 - p0) * n; e += nt) {
-      const int r = p0 + e / n, c = e - (r - p0) * n;
-      Pd[(size_t)r * n + c] = r >= r0 ? Z[r * ldZ + c] : 0.0;
-    }
+    long long yld = 1;
+    double* const yd = cx.y_dst(j, yb, ldyb, yld);
+    panel_out(Z, ldZ, t0, t1, n, rinv, rowf, d.Lp + (size_t)j * cx.R * n, rank == 0 ? 0 : t0, t1, oG + m - d.mr, yd, yld,
+              cta_grp());
   }
-  __syncthreads();
-  oz_encode(Z, ldZ, t0, t1, n, rowf, cta_grp());
   __syncthreads();
   cluster_wait();  // every CTA of the cluster runs
   {
     for (int q = 1; q < C; ++q) {
       const unsigned af = cluster_addr(rowf, (unsigned)((rank + q) % C));
-      if (tid < t1 - t0) st_cluster(af + (t0 + tid) * 4u, __int_as_float(rowf[t0 + tid]));
+      for (int r = t0 + tid; r < t1; r += nt) st_cluster(af + r * 4u, __int_as_float(rowf[r]));
       const unsigned az = cluster_addr(Z, (unsigned)((rank + q) % C));
       for (int e = tid; e < (t1 - t0) * n; e += nt) {
         const int r = t0 + e / n, c = e - (r - t0) * n;
@@ -1396,7 +1814,7 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
   // the pivot blocks: by the last rank, which stores no slots when C > 2
   if (rank == C - 1) {
     if (tid == 0 && bad) record_breakdown(info, d.sys, d.nat[j], d.level);
-    cx.store_pivot(j, Dfac, rinv, M, cta_grp());
+    cx.store_pivot_ldl(j, Dfac, M, rinv, cta_grp());
   }
   cluster_wait();  // every solved panel row is here
   oz_syrk(T, ldT, Z, rowf, Z, rowf, 0, ldZ, s0, s1, r0, n, cta_grp());
@@ -1523,7 +1941,7 @@ __device__ __forceinline__ void factor_task_w(const Task tk, const LevelDesc* __
       Rs[r * ldR + c] = (Ru[e] + Psum[e]) + cx.T[(oG + r) * ldT + oG + c];
     }
     __syncwarp();
-    corner_factor<true>(Rs, ldR, m, d.mr, cx.rinv, cx.tab, d, info, nullptr, W);
+    corner_factor(Rs, ldR, m, d.mr, cx.rinv, cx.tab, d, info, W);
   }
 }
 
@@ -1565,11 +1983,11 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
 }
 
 template <typename TZ>
-__global__ void __launch_bounds__(kFactorThreads, 3)
+__global__ void __launch_bounds__(kFactorThreads, sizeof(TZ) == 8 ? 2 : 3)
     k_factor_persist(const LevelDesc* __restrict__ descs, const Task* __restrict__ tasks,
                      const PItem* __restrict__ items, int nitems, const PCons* __restrict__ cons, int* ready,
                      const double* __restrict__ uD, const double* __restrict__ uE, const double* __restrict__ uG,
-                     const double* __restrict__ uR, Info* info, int slice, int dbl, long long wait_cycles) {
+                     const double* __restrict__ uR, Info* info, int slice, long long wait_cycles) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int bad;
   __shared__ uint32_t tslot;
@@ -1607,8 +2025,11 @@ __global__ void __launch_bounds__(kFactorThreads, 3)
     __syncthreads();
     if (ok) {
       if (!w.warp) {
-        factor_task<TZ, false>(tasks[w.first], descs, uD, uE, uG, uR, info, 0, nullptr, 1, 0, dbl, 0, smraw, bad,
-                               tslot, tbar);
+        if constexpr (sizeof(TZ) == 8)
+          factor_task_fp64(tasks[w.first], descs, uD, uE, uG, uR, info, 0, nullptr, 1, 0, smraw, bad);
+        else
+          factor_task<TZ, false>(tasks[w.first], descs, uD, uE, uG, uR, info, 0, nullptr, 1, 0, smraw, bad, tslot,
+                                 tbar);
       } else {
         const int wid = threadIdx.x >> 5;
         if (wid < w.cnt)
@@ -3003,8 +3424,8 @@ int set_smem(const void* fn, size_t bytes) {
 
 }  // namespace
 
-size_t factor_smem_bytes(int n, int m, int mixed, int fill, int dbl) {
-  return (size_t)fac_layout(n, m, mixed ? 4 : 8, fill != 0, dbl != 0).total;
+size_t factor_smem_bytes(int n, int m, int mixed, int fill) {
+  return (size_t)(mixed ? fac_layout(n, m, 4, fill != 0).total : cta_layout(n, m, fill != 0).total);
 }
 
 int debug_info(Info* out, int clear) {
@@ -3035,7 +3456,7 @@ int persist_occupancy(int mixed, size_t smem) {
 
 int launch_factor_persist(const LevelDesc* d, const Task* t, const PItem* items, int nitems, const PCons* cons,
                           int* ready, int mixed, const double* D, const double* E, const double* G,
-                          const double* R, Info* info, int grid, size_t smem, int slice, int dbl,
+                          const double* R, Info* info, int grid, size_t smem, int slice,
                           long long wait_cycles, void* stream) {
   if (nitems <= 0) return 0;
   const void* fn = mixed ? (const void*)k_factor_persist<float> : (const void*)k_factor_persist<double>;
@@ -3044,10 +3465,10 @@ int launch_factor_persist(const LevelDesc* d, const Task* t, const PItem* items,
   cudaStream_t st = (cudaStream_t)stream;
   if (mixed)
     k_factor_persist<float><<<grid, kFactorThreads, smem, st>>>(d, t, items, nitems, cons, ready, D, E, G, R, info,
-                                                                slice, dbl, wait_cycles);
+                                                                slice, wait_cycles);
   else
     k_factor_persist<double><<<grid, kFactorThreads, smem, st>>>(d, t, items, nitems, cons, ready, D, E, G, R,
-                                                                 info, slice, dbl, wait_cycles);
+                                                                 info, slice, wait_cycles);
   return (int)cudaGetLastError();
 }
 
@@ -3074,12 +3495,12 @@ int launch_factor_w(const LevelDesc* d, const Task* t, int ntasks, int maxn, int
 }
 
 // Tensor-core Schur products for a mixed launch of blocks n >= 32 when the
-// pivot-buffer region of the layout without the second pivot buffer can stage
-// the operand (Rs rows of K) and the packed product triangle, and the
-// layout spans the 128 operand rows the MMA addresses; 0 otherwise.
+// pivot-buffer region can stage the operand (Rs rows of K) and the packed
+// product triangle, and the layout spans the 128 operand rows the MMA
+// addresses; 0 otherwise.
 int tc_mode_for(int tc, int mixed, int pair, int maxn, int maxm, int fill) {
   if (!tc || !mixed || pair || maxn < 32) return 0;
-  const FacLayout L = fac_layout(maxn, maxm, 4, fill != 0, false);
+  const FacLayout L = fac_layout(maxn, maxm, 4, fill != 0);
   const int kin = tc == 2 ? 16 : 8, eb = tc == 2 ? 2 : 4;
   const long Kp = (maxn + kin - 1) / kin * kin;
   const long cap = L.oZ - L.oDfac;
@@ -3094,34 +3515,32 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
   if (ntasks <= 0) return 0;
   top_solve = top_solve && b && !mixed;
   const int tcm = tc_mode_for(tc, mixed, pair, maxn, maxm, fill);
-  // Mixed launches go without the second pivot buffer: warp 4 then joins the
-  // pivot sweep's workers, whose FP32 panel work keeps all four sub-partitions
-  // busy, and the pivot blocks are written right after the sweep (the uneven
-  // batch's mixed factorization 2-8 % faster). FP64 unpaired launches drop it
-  // only when that lets more CTAs share an SM (below); CTA pairs keep it.
-  int dbl = (mixed || tcm) ? 0 : 1;
-  size_t sm = factor_smem_bytes(maxn, maxm, mixed, fill, dbl);
+  size_t sm = factor_smem_bytes(maxn, maxm, mixed, fill);
   if (top_solve) sm = std::max(sm, solve_smem_bytes(maxn, maxm, 0, fill));
-  const void* fn = mixed ? (pair ? (const void*)k_factor<float, 1>
-                                 : tcm ? (const void*)k_factor<float, 4, true> : (const void*)k_factor<float, 4>)
-                          : (pair ? (const void*)k_factor<double, 1> : (const void*)k_factor<double, 2>);
-  int e = set_smem(fn, sm);
+  const void* fn = !mixed ? (const void*)k_factor_fp64
+                   : pair ? (const void*)k_factor<float, 1>
+                   : tcm  ? (const void*)k_factor<float, 4, true>
+                          : (const void*)k_factor<float, 4>;
+  const int e = set_smem(fn, sm);
   if (e) return e;
-  if (dbl && !pair && !top_solve) {
-    // the occupancy of this kernel with either request
-    const size_t sm1 = factor_smem_bytes(maxn, maxm, mixed, fill, 0);
-    int occ = 0, occ1 = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kFactorThreads, sm) == cudaSuccess &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, fn, kFactorThreads, sm1) == cudaSuccess &&
-        occ1 > occ) {
-      dbl = 0;
-      sm = sm1;
-    }
-  }
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   cfg.gridDim = dim3((unsigned)(pair ? 2 * ntasks : ntasks));
   cfg.blockDim = dim3(kFactorThreads);
+  if (!mixed && !pair) {
+    // more tasks than CTAs of 256 threads fit at once, and half as many threads
+    // let twice as many tasks share the SMs: their pivot chains then overlap
+    // (512 systems of n = 32: 19.1 against 21.9 ms; where shared memory allows two
+    // CTAs in either case, n = 48, the larger CTA is faster: 57.6 against 64.9 ms
+    // on 4096 uneven systems)
+    int dev = 0, sms = 0, o1 = 0, o2 = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, fn, kFactorThreads, sm) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, fn, kFactorThreads / 2, sm) == cudaSuccess &&
+        ntasks > o1 * sms && o2 >= 2 * o1)
+      cfg.blockDim = dim3(kFactorThreads / 2);
+  }
   cfg.dynamicSmemBytes = sm;
   cfg.stream = (cudaStream_t)stream;
   if (pair) {
@@ -3133,22 +3552,15 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
     cfg.numAttrs = 1;
   }
   const int p = pair ? 1 : 0;
-  if (mixed)
-    return pair ? (int)cudaLaunchKernelEx(&cfg, k_factor<float, 1>, d, t, D, E, G, R, info, p, b, ldb, top_solve,
-                                          dbl, 0)
-                : tcm ? (int)cudaLaunchKernelEx(&cfg, k_factor<float, 4, true>, d, t, D, E, G, R, info, p, b, ldb,
-                                                top_solve, dbl, tcm)
-                      : (int)cudaLaunchKernelEx(&cfg, k_factor<float, 4>, d, t, D, E, G, R, info, p, b, ldb, top_solve,
-                                                dbl, 0);
-  return pair ? (int)cudaLaunchKernelEx(&cfg, k_factor<double, 1>, d, t, D, E, G, R, info, p, b, ldb, top_solve,
-                                        dbl, 0)
-              : (int)cudaLaunchKernelEx(&cfg, k_factor<double, 2>, d, t, D, E, G, R, info, p, b, ldb, top_solve,
-                                        dbl, 0);
+  if (!mixed) return (int)cudaLaunchKernelEx(&cfg, k_factor_fp64, d, t, D, E, G, R, info, p, b, ldb, top_solve);
+  return pair ? (int)cudaLaunchKernelEx(&cfg, k_factor<float, 1>, d, t, D, E, G, R, info, p, b, ldb, 0)
+         : tcm ? (int)cudaLaunchKernelEx(&cfg, k_factor<float, 4, true>, d, t, D, E, G, R, info, p, b, ldb, tcm)
+               : (int)cudaLaunchKernelEx(&cfg, k_factor<float, 4>, d, t, D, E, G, R, info, p, b, ldb, 0);
 }
 
 int factor_clus_size(int ntasks, int maxn, int maxm, int sms) {
   if (ntasks <= 0) return 0;
-  const size_t sm = factor_smem_bytes(maxn, maxm, 0, 1, 0);
+  const size_t sm = factor_smem_bytes(maxn, maxm, 0, 1);
   if (set_smem((const void*)k_factor_clus, sm)) return 0;
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_factor_clus, kFactorThreads, sm) != cudaSuccess ||
@@ -3178,7 +3590,7 @@ int launch_factor_clus(const LevelDesc* d, const Task* t, int ntasks, int maxn, 
                        const double* E, const double* G, Info* info, void* stream, double* b, int ldb) {
   if (ntasks <= 0) return 0;
   if (C < 2 || C > 8) return (int)cudaErrorInvalidValue;
-  const size_t sm = factor_smem_bytes(maxn, maxm, 0, 1, 0);
+  const size_t sm = factor_smem_bytes(maxn, maxm, 0, 1);
   const int e = set_smem((const void*)k_factor_clus, sm);
   if (e) return e;
   cudaLaunchConfig_t cfg = {};

@@ -63,6 +63,39 @@ static __device__ __forceinline__ double pivot_rsqrt(double d) {
   return __longlong_as_double(__double_as_longlong(r) - ((long long)k << 52));
 }
 
+// 1/d for a pivot d > 0 in integer arithmetic: a dependent FP64 FMA takes 64
+// cycles on this part and holds the pipe that the pivot block's updates need.
+// With d = m 2^e (m in [1, 2), 53 bits), the single-precision estimate R 2^-24 ~
+// 1/m (24 bits, relative error below 2^-21) is corrected by 1/m = r (1 - s +
+// s^2 - ..), s = m r - 1: m R is formed modulo 2^64 in units of 2^-76, where
+// the leading 1 vanishes, and the series cut after s^2 leaves s^3 < 2^-63. The
+// result, 62 bits, is rounded to nearest once. Valid where 1/d is normal; no
+// branch, so that other work fills its latency.
+//
+// pivot_rcp_ok: d in [2^-500, 2^1017), the pivots of an elimination that forms
+// v_r^2 before it knows 1/d: with every pivot in this range a square that
+// underflows is below 2^-74 ulp of its row's pivot, and one that overflows
+// makes that pivot fail the test.
+static __device__ __forceinline__ bool pivot_rcp_ok(double d) {
+  return (unsigned)(__double2hiint(d) - (523 << 20)) < (unsigned)((2040 - 523) << 20);
+}
+static __device__ __forceinline__ double pivot_rcp(double d) {
+  const unsigned ml = (unsigned)__double2loint(d), dh = (unsigned)__double2hiint(d),
+                 mh = (dh & 0xfffffu) | 0x100000u;
+  const float mf = __uint_as_float(0x3f800000u | (mh & 0xfffffu) << 3 | ml >> 29);
+  float r0;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(mf));
+  r0 = fminf(r0, 0.999999940395355224609375f);
+  const unsigned R = (__float_as_uint(r0) & 0x7fffffu) | 0x800000u;  // units 2^-24
+  const unsigned long long S =
+      (unsigned long long)ml * R + ((unsigned long long)(mh * R) << 32);  // s, units 2^-76 (modulo 2^64)
+  const int sh = (int)(S >> 32);
+  const long long c1 = (long long)(int)R * sh + (long long)((unsigned long long)(unsigned)S * R >> 32);  // r s, 2^-68
+  const int s2 = (int)(((long long)sh * sh) >> 16);                                                     // s^2, 2^-72
+  const long long q = ((long long)R << 38) - (c1 >> 6) + (((long long)(int)R * s2) >> 34);               // 2^-62
+  return __longlong_as_double(((long long)(2044 - (int)(dh >> 20)) << 52) + ((q + 256) >> 9));
+}
+
 // |v| as a float for the |Psi| row sums that scale eta: the exponent rebased
 // and the mantissa cut to 20 bits with integer operations only (no FP64
 // instruction), so never above |v|; 0 below the float range, the largest

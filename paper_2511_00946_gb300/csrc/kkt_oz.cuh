@@ -32,8 +32,10 @@
 // issue alone; one system of N = 1024, n = 32, m = 8 factored and solved 708 ->
 // 653 us, N = 777, n = 45 1527 -> 1238 us, 4096 uneven systems 70.8 -> 63.6 ms.
 //
-// A row with infinities, NaN or an exponent outside +-400 keeps its doubles
-// (flag kFp64Row) and takes FP64 FMAs.
+// A row with infinities, NaN or an exponent above 400, or whose elements are
+// near the subnormal range, keeps its doubles (flag kFp64Row) and takes FP64
+// FMAs. Small exponents are otherwise split (the fill-in between distant
+// separators decays below 1e-130).
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -57,7 +59,8 @@ typedef unsigned long long u64;
 
 constexpr int kDig = 7;            // digits of nine bits
 constexpr int kLow = kDig - 1;     // smallest i + j of the products kept
-constexpr int kExpMax = 400;       // exponents of the rows split
+constexpr int kExpMax = 400;       // largest exponent of the rows split
+constexpr int kExpMin = -960;      // smallest one (elements 62 bits below it are normal)
 constexpr int kFp64Row = 1 << 20;  // exponent of a row that keeps its doubles
 // 256 in every digit: 256 (2^63 - 1) / 511
 constexpr u64 kBias = 256ull * ((1ull << 63) / 511);
@@ -82,11 +85,13 @@ KKT_OZ double bitsd(u64 b) {
 }
 KKT_OZ int expo(u64 b) { return (int)(b >> 52) & 0x7ff; }
 
-// the row exponent from the largest biased exponent of its elements
-KKT_OZ int row_exp(int emax) {
-  if (emax == 0) return -kExpMax;  // zero (and subnormal) elements only
-  const int f = emax - 1022;
-  return f < -kExpMax || f > kExpMax ? kFp64Row : f;  // (infinities and NaN included)
+// order of |v|: its high word, and 1 for the smallest subnormals
+KKT_OZ int mag(u64 b) { return (int)(b >> 32 & 0x7fffffff) | ((uint32_t)b != 0); }
+
+// the row exponent from the largest mag() of its elements (-1022: a zero row)
+KKT_OZ int row_exp(int m) {
+  const int f = (m >> 20) - 1022;
+  return f > kExpMax || (f < kExpMin && m != 0) ? kFp64Row : f;  // (infinities and NaN included)
 }
 
 // digits of z at exponent f (|z| < 2^f), 256 added to each
@@ -98,7 +103,7 @@ KKT_OZ u64 encode(u64 b, int f) {
   return (u64)v + kBias;
 }
 
-// u 2^e as a double, rounded to nearest (|e| <= 900: the result is normal)
+// u 2^e as a double, rounded to nearest (truncated below the normal range; e <= 900)
 KKT_OZ double to_double(i64 u, int e) {
   u64 a = u < 0 ? (u64)-u : (u64)u;
 #if defined(__CUDA_ARCH__)
@@ -108,7 +113,8 @@ KKT_OZ double to_double(i64 u, int e) {
 #endif
   a <<= (lz & 63);
   const u64 m = (a >> 11) + ((a >> 10) & 1);  // 53 bits; a carry moves the exponent up
-  const u64 b = ((u64)(1023 + 63 - 1 - lz + e) << 52) + m;
+  const int ex = 1023 + 63 - 1 - lz + e;
+  const u64 b = ex >= 0 ? ((u64)ex << 52) + m : m >> (-ex < 63 ? -ex : 63);
   return bitsd(u == 0 ? 0 : b | ((u64)u & 0x8000000000000000ull));
 }
 
@@ -228,6 +234,60 @@ __device__ __forceinline__ void tile(double* T, int ldt, const double* Zlo, cons
 #pragma unroll
       for (int i = 0; i < kDig; ++i) p[i] = (int)acc[i][e];
       T[a * ldt + b] -= to_double(combine(p), (e < 2 ? xa : xc) + (e & 1 ? x1 : x0) + kUnit);
+    }
+  }
+}
+
+__device__ __forceinline__ void mma_f16_k8(float* d, const uint32_t* a, uint32_t b) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a[0]), "r"(a[1]), "r"(b));
+}
+
+// One 16 x 8 tile of dst -= U V^T over eight columns by a warp: dst[a][b] for
+// a = a0 + 0..15 (< ea), b = b0 + 0..7 (< eb). U: digit
+// rows of the a (row a at U + (a - ua) 8, exponents eU[a - ua]), V: of the b
+// (V, eV indexed by b - vb).
+__device__ __forceinline__ void tile8(double* dst, int ldd, const u64* U, const int* eU, int ua,
+                                         const u64* V, const int* eV, int vb, int a0, int ea, int b0, int eb,
+                                         int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  const int ra = a0 + g, rc = ra + 8;
+  const int qa = min(ra, ea - 1) - ua, qc = min(rc, ea - 1) - ua, qb = min(b0 + g, eb - 1) - vb;
+  const int xa = eU[qa], xc = eU[qc], xb = eV[qb];
+  const int c0 = b0 + 2 * t, c1 = c0 + 1;
+  if (__any_sync(0xffffffffu, max(max(xa, xc), xb) == kFp64Row)) {
+    for (int e = 0; e < 4; ++e) {
+      const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
+      if (a < ea && b < eb)
+        element(dst + a * ldd + b, U + (a - ua) * 8, e < 2 ? xa : xc, V + (b - vb) * 8, eV[b - vb], 8);
+    }
+    return;
+  }
+  float acc[kDig][4];
+#pragma unroll
+  for (int i = 0; i < kDig; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
+  {
+    const ulonglong2 pa = *(const ulonglong2*)(U + qa * 8 + 2 * t), pc = *(const ulonglong2*)(U + qc * 8 + 2 * t),
+                     pb = *(const ulonglong2*)(V + qb * 8 + 2 * t);
+    const u64 u[4] = {pa.x, pa.y, pc.x, pc.y}, v[2] = {pb.x, pb.y};
+    uint32_t A[kDig][2], B[kDig][1];
+    Split<0>::run<2>(A, u);
+    Split<0>::run<1>(B, v);
+#pragma unroll
+    for (int i = 0; i < kDig; ++i)
+#pragma unroll
+      for (int j = kDig - 1; j >= kLow - i; --j) mma_f16_k8(acc[i + j - kLow], A[i], B[j][0]);
+  }
+  const int x0 = __shfl_sync(0xffffffffu, xb, 8 * t), x1 = __shfl_sync(0xffffffffu, xb, 8 * t + 4);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
+    if (a < ea && b < eb) {
+      int p[kDig];
+#pragma unroll
+      for (int i = 0; i < kDig; ++i) p[i] = (int)acc[i][e];
+      dst[a * ldd + b] -= to_double(combine(p), (e < 2 ? xa : xc) + (e & 1 ? x1 : x0) + kUnit);
     }
   }
 }

@@ -6,7 +6,7 @@ extern "C" {
 // exponent of a row of n elements, and its digits (u[n])
 int oz_row(const double* z, int n, unsigned long long* u) {
   int em = 0;
-  for (int k = 0; k < n; ++k) em = em > kkt::oz::expo(kkt::oz::dbits(z[k])) ? em : kkt::oz::expo(kkt::oz::dbits(z[k]));
+  for (int k = 0; k < n; ++k) em = em > kkt::oz::mag(kkt::oz::dbits(z[k])) ? em : kkt::oz::mag(kkt::oz::dbits(z[k]));
   const int f = kkt::oz::row_exp(em);
   if (f != kkt::oz::kFp64Row)
     for (int k = 0; k < n; ++k) u[k] = kkt::oz::encode(kkt::oz::dbits(z[k]), f);

@@ -11,7 +11,7 @@ __global__ void k_probe(double* Z, int ldz, int rows, int n, double* T, int ldt,
   for (int r = threadIdx.x; r < rows; r += blockDim.x) {
     oz::u64* z = (oz::u64*)(Z + r * ldz);
     int em = 0;
-    for (int k = 0; k < n; ++k) em = max(em, oz::expo(z[k]));
+    for (int k = 0; k < n; ++k) em = max(em, oz::mag(z[k]));
     f[r] = oz::row_exp(em);
     if (f[r] != oz::kFp64Row)
       for (int k = 0; k < n; ++k) z[k] = oz::encode(z[k], f[r]);

@@ -69,7 +69,7 @@ def test_rows_outside_the_split_take_fp64(probe):
     Z = rng.normal(size=(rows, n))
     ref, _ = probe(Z.copy(), np.zeros((rows, rows)))
     W = Z.copy()
-    W[5, 3], W[9, 0], W[13] = np.nan, np.inf, Z[13] * 1e-160
+    W[5, 3], W[9, 0], W[13] = np.nan, np.inf, Z[13] * 1e160
     out, f = probe(W.copy(), np.zeros((rows, rows)))
     assert (f[[5, 9, 13]] == 1 << 20).all() and (np.delete(f, [5, 9, 13]) < 401).all()
     keep = [r for r in range(rows) if r not in (5, 9, 13)]

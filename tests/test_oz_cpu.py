@@ -58,9 +58,24 @@ def test_digits_and_value(lib):
             assert abs(Fraction(lib.oz_value(int(v), f)) - Fraction(float(x))) <= Fraction(2) ** (f - 62)
             if abs(x) >= 2.0 ** (f - 9):  # within 2^-8 of the row's scale: exact
                 assert lib.oz_value(int(v), f) == x
-    assert row(lib, [0.0, -0.0, 5e-324])[0] == -400
-    for bad in (np.nan, np.inf, 1e300, 1e-200):
+    f, u = row(lib, [0.0, -0.0])
+    assert f == -1022 and all(lib.oz_value(int(v), f) == 0.0 for v in u)
+    f, u = row(lib, [3e-280, -1e-281])  # far below one: split like any other
+    assert [lib.oz_value(int(v), f) for v in u] == [3e-280, -1e-281]
+    for bad in (np.nan, np.inf, 1e300, 5e-324, 1e-300):
         assert row(lib, [bad, bad / 4])[0] == FP64_ROW
+
+
+def test_products_below_the_normal_range(lib):
+    """Gradual underflow: within the smallest subnormal of the exact product
+    (and the split's own bound)."""
+    rng = np.random.default_rng(3)
+    for s in (-480, -510, -516, -525, -560):
+        a, b = rng.normal(size=20) * 2.0 ** s, rng.normal(size=20) * 2.0 ** s
+        got, _, fa, fb = dot(lib, a, b)
+        x = exact(a, b)
+        assert abs(Fraction(got) - x) <= abs(x) / 2**53 + 20 * Fraction(2.0 ** -57.9) * Fraction(2) ** (fa + fb) + \
+            Fraction(2) ** -1074
 
 
 def test_to_double_rounds_to_nearest(lib):
