@@ -3007,14 +3007,13 @@ __global__ void k_axpy(const LevelDesc* __restrict__ descs, const ResTask* __res
 }
 
 // FP64 residual c = b - Psi x (blocks of Eq. (3)) over the stage rows of one
-// residual task (kResChunk consecutive stages of one system) per warp. A
-// pass takes res_spw(n) consecutive stages, chosen so that their rows fill
-// whole warps (up to three rows per lane: row r of the pass is lane r % 32,
-// slot r / 32), since an FP64 instruction costs its issue slot whether a
-// lane has a row or not. Each lane forms, for each of its rows,
+// residual task (kResChunk consecutive stages of one system) per CTA. The task's
+// rows, all stages in one list, go to the warps in groups of 32, one row per
+// lane, since an FP64 instruction costs its issue slot whether a lane has a row
+// or not. Each lane forms, for its row i of stage j,
 //   (E_{j-1} x_{j-1} + D_j x_j + E_j^T x_{j+1} + G_j^T x_g)_i
 // from the blocks in global memory (lower triangle of D_j by symmetry) as
-// three independent FMA chains, with the pass's x rows (and its neighbour
+// three independent FMA chains, with the x rows of the task (and its neighbour
 // stages') staged in shared memory, so Psi is read once. A matrix-vector
 // product does 2 flop per 8-byte element, more than the FP64 units sustain
 // at full HBM bandwidth on this part, so the kernel keeps FP64 work to the
@@ -3022,47 +3021,44 @@ __global__ void k_axpy(const LevelDesc* __restrict__ descs, const ResTask* __res
 // `norms` is set (the first sweep of a refinement; they depend on the matrix
 // alone). Per task it writes the g-row partials sum_j G_j x_j (m x nr),
 // max|c|, max|x|, max|b| and, with `norms`, the largest stage-row sum of
-// |Psi| and the |G| sums of the g rows; k_residual_final combines them per
-// system. MB: registers for up to MB arrow rows.
+// |Psi| and the |G| sums of the g rows, each the warps' partials in warp order;
+// k_residual_final combines them per system. MB: registers for up to MB arrow rows.
+//
+// Bound by the FP64 pipe (75 % busy; 1824 tasks of mixed sizes). With one warp
+// per task, three rows per lane, it was bound by the latency of its loads: 150
+// -> 27 us a sweep for one system of N = 256, n = 32, m = 8 (32 warps on the
+// whole chip), 2.7 -> 1.9 ms for 2048 uneven systems.
 template <int MB>
-__global__ void __launch_bounds__(256, 3) k_residual(const LevelDesc* __restrict__ descs,
-                                                  const ResTask* __restrict__ tasks, int ntasks,
+__global__ void __launch_bounds__(256, MB <= 8 ? 3 : 2) k_residual(const LevelDesc* __restrict__ descs,
+                                                  const ResTask* __restrict__ tasks,
                                                   const double* __restrict__ uD, const double* __restrict__ uE,
                                                   const double* __restrict__ uG, const double* __restrict__ b,
                                                   int ldb, const double* __restrict__ x, int ldx, double* c,
                                                   int nr, double* parts, const int* skip, int norms,
                                                   int xs_doubles) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int lane = threadIdx.x & 31;
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (t >= ntasks) return;  // whole warp
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+  const int t = blockIdx.x;
   const ResTask tk = tasks[t];
   const LevelDesc& d = descs[tk.desc];
   if (skip && skip[d.sys]) return;
   const int n = d.n, m = d.m, N = d.N;
-  const int spw = res_spw(n);  // stages per pass
   if (!dbg_ok(tk.j0 >= 0 && tk.j0 < d.N && d.n <= kMaxN && d.m <= MB && tk.part < tk.nparts &&
-                  (spw + 2) * n <= xs_doubles,
+                  (kResChunk + 2) * n <= xs_doubles,
               d))
     return;
-  const int j0 = tk.j0, j1 = min(tk.j0 + kResChunk, N);
+  const int j0 = tk.j0, cnt = min(kResChunk, N - j0), rows = cnt * n;
   const size_t nn = (size_t)n * n, mn = (size_t)m * n;
   const double* D = uD + d.offD;
   const double* E = uE ? uE + d.offE : nullptr;
   const double* G = m ? uG + d.offG : nullptr;
-  double* part = parts + (size_t)t * kResPartDoubles;
-  // x rows of stages jb-1 .. jb+spw of the current pass: xs[(s + 1) n + k] is
-  // row k of stage jb + s (zero outside 0..N-1)
-  double* const xs = reinterpret_cast<double*>(smraw) + (size_t)(threadIdx.x >> 5) * xs_doubles;
-  // this lane's rows of a pass: slot q is pass row lane + 32 q, i.e. row ri[q] of stage si[q]
-  const int rows = spw * n, slots = (rows + 31) >> 5;
-  int si[3], ri[3];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const int r = lane + 32 * q;
-    si[q] = r < rows ? r / n : 0;
-    ri[q] = r < rows ? r - si[q] * n : 0;
-  }
+  const Div by(n);
+  // x rows of stages j0 - 1 .. j0 + cnt: xs[(s + 1) n + k] is row k of stage j0 + s
+  // (zero outside 0..N-1)
+  double* const xs = reinterpret_cast<double*>(smraw);
+  // the warps' partials: kMaxM x kRhsChunk g rows, maxima and sums
+  double* const wpart = xs + xs_doubles;
+  double* const part = wpart + wid * kResWarpDoubles;
   double mr = 0.0, mx = 0.0, mb = 0.0;
   float mrow = 0.0f;
   for (int col = 0; col < nr; ++col) {
@@ -3070,57 +3066,56 @@ __global__ void __launch_bounds__(256, 3) k_residual(const LevelDesc* __restrict
     double gacc[MB];  // this lane's terms of sum_j G_j x_j per g row
 #pragma unroll
     for (int q = 0; q < MB; ++q) gacc[q] = 0.0;
-    for (int jb = j0; jb < j1; jb += spw) {
-      const int cnt = min(spw, j1 - jb);
-      __syncwarp();  // the previous pass is done with xs
-      for (int e = lane; e < (cnt + 2) * n; e += 32) {
-        const int s = e / n - 1, k = e - (s + 1) * n, jj = jb + s;
-        xs[e] = (jj >= 0 && jj < N) ? x[(size_t)(d.offB + (long long)jj * n + k) * ldx + col] : 0.0;
+    if (col) __syncthreads();  // the previous column is done with xs
+    {
+      const long long r0 = (long long)(j0 - 1) * n;  // first row, below 0 at the system's start
+      for (int e = tid; e < (cnt + 2) * n; e += nt) {
+        const long long r = r0 + e;
+        xs[e] = r >= 0 && r < (long long)N * n ? x[(size_t)(d.offB + r) * ldx + col] : 0.0;
       }
-      __syncwarp();
+    }
+    __syncthreads();
+    for (int g0 = wid * 32; g0 < rows; g0 += nw * 32) {
+      const bool ok = g0 + lane < rows;
+      const int r = ok ? g0 + lane : 0, s = by(r), i = r - s * n, j = j0 + s;
+      const double* Dj = D + (size_t)j * nn;
+      const bool hp = E && j > 0, hn = E && j < N - 1;
+      const double* Ep = hp ? E + (size_t)(j - 1) * nn : D;
+      const double* En = hn ? E + (size_t)j * nn : D;
+      const double* xp = xs + (size_t)s * n;  // x_{j-1}, x_j, x_{j+1} follow at n apart
+      // E_{j-1} x_{j-1}, D_j x_j (lower triangle by symmetry) and E_j^T
+      // x_{j+1} as three independent chains over k, then summed
+      double aP = 0.0, aD = 0.0, aN = 0.0;
+      float rs = 0.0f;
+#pragma unroll 4
+      for (int k = 0; k < n; ++k) {
+        const double dv = k <= i ? Dj[i * n + k] : Dj[k * n + i];
+        const double pv = hp ? Ep[i * n + k] : 0.0, qv = hn ? En[k * n + i] : 0.0;
+        aP = fma(pv, xp[k], aP);
+        aD = fma(dv, xp[n + k], aD);
+        aN = fma(qv, xp[2 * n + k], aN);
+        if (norms) rs += (abs_lo(dv) + abs_lo(pv)) + abs_lo(qv);
+      }
+      double acc = (aP + aD) + aN;
+      const double xo = ok ? xp[n + i] : 0.0;  // this row's x
+      if (m) {
+        const double* Gj = G + (size_t)j * mn;
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        if (q >= slots) break;  // warp-uniform
-        const bool ok = lane + 32 * q < cnt * n;
-        const int s = ok ? si[q] : 0, i = ok ? ri[q] : 0, j = jb + s;
-        const long long rb = d.offB + (long long)j * n;
-        const double* Dj = D + (size_t)j * nn;
-        const bool hp = E && j > 0, hn = E && j < N - 1;
-        const double* Ep = hp ? E + (size_t)(j - 1) * nn : D;
-        const double* En = hn ? E + (size_t)j * nn : D;
-        const double* xp = xs + (size_t)s * n;  // x_{j-1}, x_j, x_{j+1} follow at n apart
-        // E_{j-1} x_{j-1}, D_j x_j (lower triangle by symmetry) and E_j^T
-        // x_{j+1} as three independent chains over k, then summed
-        double aP = 0.0, aD = 0.0, aN = 0.0;
-        float rs = 0.0f;
-        for (int k = 0; k < n; ++k) {
-          const double dv = k <= i ? Dj[i * n + k] : Dj[k * n + i];
-          const double pv = hp ? Ep[i * n + k] : 0.0, qv = hn ? En[k * n + i] : 0.0;
-          aP = fma(pv, xp[k], aP);
-          aD = fma(dv, xp[n + k], aD);
-          aN = fma(qv, xp[2 * n + k], aN);
-          if (norms) rs += (abs_lo(dv) + abs_lo(pv)) + abs_lo(qv);
+        for (int g = 0; g < MB; ++g) {
+          if (g >= m) break;  // warp-uniform; full unrolling keeps gacc in registers
+          const double xq = __shfl_sync(0xffffffffu, xg_l, g);
+          const double gv = Gj[g * n + i];
+          acc = fma(gv, xq, acc);
+          gacc[g] = fma(gv, xo, gacc[g]);  // xo = 0 on lanes without a row
+          if (norms) rs += abs_lo(gv);
         }
-        double acc = (aP + aD) + aN;
-        const double xo = ok ? xp[n + i] : 0.0;  // this row's x
-        if (m) {
-          const double* Gj = G + (size_t)j * mn;
-#pragma unroll
-          for (int g = 0; g < MB; ++g) {
-            if (g >= m) break;  // warp-uniform; full unrolling keeps gacc in registers
-            const double xq = __shfl_sync(0xffffffffu, xg_l, g);
-            const double gv = Gj[g * n + i];
-            acc = fma(gv, xq, acc);
-            gacc[g] = fma(gv, xo, gacc[g]);  // xo = 0 on lanes without a row
-            if (norms) rs += abs_lo(gv);
-          }
-        }
-        if (ok) {
-          const double bv = b ? b[(size_t)(rb + i) * ldb + col] : 0.0, r = bv - acc;
-          c[(size_t)(rb + i) * kRhsChunk + col] = r;
-          mr = fmax(mr, fabs(r)); mb = fmax(mb, fabs(bv)); mx = fmax(mx, fabs(xo));
-          if (norms) mrow = fmaxf(mrow, rs);
-        }
+      }
+      if (ok) {
+        const size_t row = (size_t)(d.offB + (long long)j * n + i);
+        const double bv = b ? b[row * ldb + col] : 0.0, res = bv - acc;
+        c[row * kRhsChunk + col] = res;
+        mr = fmax(mr, fabs(res)); mb = fmax(mb, fabs(bv)); mx = fmax(mx, fabs(xo));
+        if (norms) mrow = fmaxf(mrow, rs);
       }
     }
     // g-row partials of this column: lane sums, then a shuffle tree
@@ -3132,9 +3127,9 @@ __global__ void __launch_bounds__(256, 3) k_residual(const LevelDesc* __restrict
       if (lane == 0) part[g * kRhsChunk + col] = v;
     }
   }
-  float gab = 0.0f;  // |G| sum of g row `lane` (lane < m) over the task's stages
+  float gab = 0.0f;  // |G| sum of g row `lane` (lane < m) over the warp's stages
   if (norms && m && lane < m)
-    for (int j = j0; j < j1; ++j) {
+    for (int j = j0 + wid; j < j0 + cnt; j += nw) {
       const double* Gj = G + (size_t)j * mn;
       for (int i = 0; i < n; ++i) gab += abs_lo(Gj[lane * n + i]);
     }
@@ -3144,12 +3139,29 @@ __global__ void __launch_bounds__(256, 3) k_residual(const LevelDesc* __restrict
     mb = fmax(mb, __shfl_xor_sync(0xffffffffu, mb, o));
     if (norms) mrow = fmaxf(mrow, __shfl_xor_sync(0xffffffffu, mrow, o));
   }
-  double* pm = part + kMaxM * kRhsChunk;
+  double* const pm = part + kMaxM * kRhsChunk;
   if (lane == 0) {
     pm[0] = mr; pm[1] = mx; pm[2] = mb;
     if (norms) pm[3] = (double)mrow;
   }
   if (norms && lane < m) pm[4 + lane] = (double)gab;
+  __syncthreads();
+  double* const slot = parts + (size_t)t * kResPartDoubles;
+  for (int e = tid; e < m * nr; e += nt) {
+    const int q = e / nr, o = q * kRhsChunk + (e - q * nr);
+    double v = wpart[o];
+    for (int w = 1; w < nw; ++w) v += wpart[w * kResWarpDoubles + o];
+    slot[o] = v;
+  }
+  if (tid < (norms ? 4 + m : 3)) {
+    const double* const wm = wpart + kMaxM * kRhsChunk + tid;
+    double v = wm[0];
+    for (int w = 1; w < nw; ++w) {
+      const double u = wm[w * kResWarpDoubles];
+      v = tid < 4 ? fmax(v, u) : v + u;
+    }
+    slot[kMaxM * kRhsChunk + tid] = v;
+  }
 }
 
 // Finish the g rows of one system from the chunk partials, then eta and the
@@ -3184,26 +3196,32 @@ __global__ void k_residual_final(const LevelDesc* __restrict__ descs, const int*
     const double* pm = parts + (size_t)(p0 + p) * kResPartDoubles + kMaxM * kRhsChunk;
     mr = fmax(mr, pm[0]); mx = fmax(mx, pm[1]); mb = fmax(mb, pm[2]); mrow = fmax(mrow, pm[3]);
   }
-  for (int q = threadIdx.x; q < m; q += blockDim.x) {
+  // a warp per g row, its lanes over the chunks
+  const int lane = threadIdx.x & 31;
+  auto warp_sum = [](double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  for (int q = threadIdx.x >> 5; q < m; q += blockDim.x >> 5) {
     double ga = 0.0;
-    for (int p = 0; p < np; ++p) ga += parts[(size_t)(p0 + p) * kResPartDoubles + kMaxM * kRhsChunk + 4 + q];
-    for (int k = 0; k < m; ++k) ga += fabs(k <= q ? R[q * m + k] : R[k * m + q]);
-    gsum[q] = ga;
+    for (int p = lane; p < np; p += 32) ga += parts[(size_t)(p0 + p) * kResPartDoubles + kMaxM * kRhsChunk + 4 + q];
+    if (lane < m) ga += fabs(lane <= q ? R[q * m + lane] : R[lane * m + q]);
+    ga = warp_sum(ga);
+    if (lane == 0) gsum[q] = ga;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < m * nr; e += blockDim.x) {
+  for (int e = threadIdx.x >> 5; e < m * nr; e += blockDim.x >> 5) {
     const int q = e / nr, col = e - q * nr;
-    double acc = 0.0;
-    for (int p = 0; p < np; ++p) acc += parts[(size_t)(p0 + p) * kResPartDoubles + q * kRhsChunk + col];
-    for (int k = 0; k < m; ++k)
-      acc = fma(k <= q ? R[q * m + k] : R[k * m + q], x[(size_t)(d.rowG + k) * ldx + col], acc);
     const size_t row = (size_t)(d.rowG + q);
-    const double bv = b ? b[row * ldb + col] : 0.0;
-    const double r = bv - acc;
-    c[row * kRhsChunk + col] = r;
+    const double bv = b ? b[row * ldb + col] : 0.0, xv = x[row * ldx + col];
+    double acc = 0.0;
+    for (int p = lane; p < np; p += 32) acc += parts[(size_t)(p0 + p) * kResPartDoubles + q * kRhsChunk + col];
+    if (lane < m) acc = fma(lane <= q ? R[q * m + lane] : R[lane * m + q], x[(size_t)(d.rowG + lane) * ldx + col], acc);
+    const double r = bv - warp_sum(acc);
+    if (lane == 0) c[row * kRhsChunk + col] = r;
     mr = fmax(mr, fabs(r));
     mb = fmax(mb, fabs(bv));
-    mx = fmax(mx, fabs(x[row * ldx + col]));
+    mx = fmax(mx, fabs(xv));
   }
   for (int q = threadIdx.x; q < m; q += blockDim.x) mrow = fmax(mrow, gsum[q]);
   red[0][threadIdx.x] = mr; red[1][threadIdx.x] = mx; red[2][threadIdx.x] = mb; red[3][threadIdx.x] = mrow;
@@ -3779,15 +3797,16 @@ int launch_adjoint_grad(const LevelDesc* d, const ResTask* t, int ntasks, const 
 
 int launch_residual(const LevelDesc* d, const ResTask* t, int ntasks, const double* D, const double* E,
                     const double* G, const double* b, int ldb, const double* x, int ldx, double* c, int nr,
-                    double* parts, const int* skip, int norms, void* stream, int xs_doubles, int maxm) {
+                    double* parts, const int* skip, int norms, void* stream, int maxn, int maxm) {
   if (ntasks <= 0) return 0;
+  const int xs_doubles = (kResChunk + 2) * maxn;
   cudaStream_t st = (cudaStream_t)stream;
-  const unsigned grid = (unsigned)((ntasks + 7) / 8);
-  const size_t sm = (size_t)8 * xs_doubles * sizeof(double);
+  const int nw = std::min(8, (kResChunk * maxn + 31) / 32);  // a warp per 32 rows of a task
+  const size_t sm = ((size_t)xs_doubles + nw * kResWarpDoubles) * sizeof(double);
   auto go = [&](auto kern) -> int {
     const int e = set_smem((const void*)kern, sm);
     if (e) return e;
-    kern<<<grid, 256, sm, st>>>(d, t, ntasks, D, E, G, b, ldb, x, ldx, c, nr, parts, skip, norms, xs_doubles);
+    kern<<<ntasks, 32 * nw, sm, st>>>(d, t, D, E, G, b, ldb, x, ldx, c, nr, parts, skip, norms, xs_doubles);
     return (int)cudaGetLastError();
   };
   if (maxm <= 4) return go(k_residual<4>);
