@@ -1251,7 +1251,7 @@ struct FacCtx {
 // Forward substitution task of the solve kernels (defined below); the factor
 // kernel of a bordered pass runs it for the top level (corner solve and the
 // backward sweep of the top level) right after the corner.
-template <typename TS>
+template <typename TS, bool W = false>
 __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs, double* b, int ldb, int nr,
                              const int* skip, unsigned char* smraw, Grp G, int fwd_done, int c0 = 0);
 
@@ -2067,16 +2067,33 @@ __device__ __forceinline__ VecView level_vec(const LevelDesc& d, double* b, int 
   return v;
 }
 
+// level_vec of every stage (the descriptor is read once: a level's fields would
+// be loaded again behind every store)
+struct VecViews {
+  double* p;
+  size_t step;
+  int ld;
+  __device__ VecViews(const LevelDesc& d, double* b, int ldb, int c0) {
+    const VecView v = level_vec(d, b, ldb, 0, c0);
+    p = v.p;
+    ld = v.ld;
+    step = (size_t)d.n * ld;
+  }
+  __device__ double* at(int j) const { return p + j * step; }
+};
+
 // dst (rows x nr, smem ld) <- src rows (global, stride lds) (+ src2, stride kRhsChunk)
 template <typename TS>
 __device__ void load_vec(TS* dst, int ldd, const double* src, int lds, const double* src2, int rows,
                          int nr, Grp G) {
   if (src2) {
+#pragma unroll 2
     for (int e = G.tid; e < rows * nr; e += G.nt) {
       const int r = e / nr, c = e - r * nr;
       dst[r * ldd + c] = (TS)(src[(size_t)r * lds + c] + src2[(size_t)r * kRhsChunk + c]);
     }
   } else {
+#pragma unroll 2
     for (int e = G.tid; e < rows * nr; e += G.nt) {
       const int r = e / nr, c = e - r * nr;
       dst[r * ldd + c] = (TS)src[(size_t)r * lds + c];
@@ -2086,11 +2103,52 @@ __device__ void load_vec(TS* dst, int ldd, const double* src, int lds, const dou
 
 template <typename TS>
 __device__ void store_vec(double* dst, int ldd, const TS* src, int lds, int rows, int nr, Grp G) {
+#pragma unroll 2
   for (int e = G.tid; e < rows * nr; e += G.nt) {
     const int r = e / nr, c = e - r * nr;
     dst[(size_t)r * ldd + c] = (double)src[r * lds + c];
   }
 }
+
+// load_vec in two parts: the loads into registers, and the stores some work
+// later (up to U elements per thread; further ones are loaded late). U = 3:
+// kMaxN x kRhsChunk elements by 256 threads.
+template <int U>
+struct VecPrefetch {
+  double v[U + 1], w[U + 1];
+  const double *src, *src2;
+  int lds;
+  __device__ __forceinline__ void load(const double* s, int ld, const double* s2, int rows, int nr, const Div& by,
+                                       Grp G) {
+    src = s;
+    src2 = s2;
+    lds = ld;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = G.tid + u * G.nt, r = by(e), c = e - r * nr;
+      w[u] = 0.0;
+      if (G.tid >= 0 && e < rows * nr) {
+        v[u] = s[(size_t)r * ld + c];
+        if (s2) w[u] = s2[(size_t)r * kRhsChunk + c];
+      }
+    }
+  }
+  template <typename TS>
+  __device__ __forceinline__ void store(TS* dst, int ldd, int rows, int nr, const Div& by, Grp G) const {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = G.tid + u * G.nt, r = by(e);
+      if (G.tid >= 0 && e < rows * nr) dst[r * ldd + e - r * nr] = (TS)(src2 ? v[u] + w[u] : v[u]);
+    }
+    if (G.tid < 0) return;
+#pragma unroll 1
+    for (int e = G.tid + U * G.nt; e < rows * nr; e += G.nt) {
+      const int r = by(e), c = e - r * nr;
+      const double x = src[(size_t)r * lds + c];
+      dst[r * ldd + c] = (TS)(src2 ? x + src2[(size_t)r * kRhsChunk + c] : x);
+    }
+  }
+};
 
 __device__ __forceinline__ double shfl_idx(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 __device__ __forceinline__ float shfl_idx(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
@@ -2110,78 +2168,118 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // every group but the two most recent ones complete
 __device__ __forceinline__ void cp_async_wait_2() { asm volatile("cp.async.wait_group 2;" ::: "memory"); }
 
-// t <- L^{-1} t (forward) or t <- L^{-T} t (backward) for nr columns, one
-// warp per column (warp-synchronous: shuffles, no block barriers). Rows i
-// and i + 32 of a column live in lane i. Forward uses M (columns of L divided
-// by their diagonal): u_i -= M_ij u_j, x = u * rinv. Backward uses MR (rows
-// of L divided by their diagonal): u_i -= MR_ji u_j for i < j, x = u * rinv.
-// The group's warps take the columns in turn; ends with the group's barrier.
-template <typename TS>
-__device__ void trsv_warp(TS* t, int ldt, const TS* M, int ldl, const TS* rinv, int n, int nr,
-                          bool backward, Grp G) {
-  const int lane = G.tid & 31, warp = G.tid >> 5, nw = G.nt >> 5;
-  const int i0 = lane, i1 = lane + 32;
-  for (int c = warp; c < nr; c += nw) {
-    TS u0 = i0 < n ? t[i0 * ldt + c] : TS(0);
-    if (n <= 32) {  // one row per lane (warp-uniform branch: no predicated FP64 slots)
-      const int ir = i0 < n ? i0 : n - 1;  // clamp the multiplier row of idle lanes
-      if (!backward) {
-        int j = 0;
-        for (; j + 4 < n; j += 4) {  // multipliers of four steps loaded ahead
-          const TS m0 = M[ir * ldl + j], m1 = M[ir * ldl + j + 1], m2 = M[ir * ldl + j + 2],
-                   m3 = M[ir * ldl + j + 3];
-          TS uj = shfl_idx(u0, j);
-          if (i0 > j) u0 = fma(-m0, uj, u0);
-          uj = shfl_idx(u0, j + 1);
-          if (i0 > j + 1) u0 = fma(-m1, uj, u0);
-          uj = shfl_idx(u0, j + 2);
-          if (i0 > j + 2) u0 = fma(-m2, uj, u0);
-          uj = shfl_idx(u0, j + 3);
-          if (i0 > j + 3) u0 = fma(-m3, uj, u0);
-        }
-        for (; j < n - 1; ++j) {
-          const TS uj = shfl_idx(u0, j);
-          if (i0 > j) u0 = fma(-M[ir * ldl + j], uj, u0);
-        }
-      } else {
-        int j = n - 1;
-        for (; j - 3 > 0; j -= 4) {
-          const TS m0 = M[j * ldl + ir], m1 = M[(j - 1) * ldl + ir], m2 = M[(j - 2) * ldl + ir],
-                   m3 = M[(j - 3) * ldl + ir];
-          TS uj = shfl_idx(u0, j);
-          if (i0 < j) u0 = fma(-m0, uj, u0);
-          uj = shfl_idx(u0, j - 1);
-          if (i0 < j - 1) u0 = fma(-m1, uj, u0);
-          uj = shfl_idx(u0, j - 2);
-          if (i0 < j - 2) u0 = fma(-m2, uj, u0);
-          uj = shfl_idx(u0, j - 3);
-          if (i0 < j - 3) u0 = fma(-m3, uj, u0);
-        }
-        for (; j > 0; --j) {
-          const TS uj = shfl_idx(u0, j);
-          if (i0 < j) u0 = fma(-M[j * ldl + ir], uj, u0);
-        }
-      }
-    } else {
-      TS u1 = i1 < n ? t[i1 * ldt + c] : TS(0);
-      if (!backward) {
-        for (int j = 0; j < n - 1; ++j) {
-          const TS uj = shfl_idx(j < 32 ? u0 : u1, j & 31);
-          if (i0 > j) u0 = fma(-M[i0 * ldl + j], uj, u0);
-          if (i1 > j && i1 < n) u1 = fma(-M[i1 * ldl + j], uj, u1);
-        }
-      } else {
-        for (int j = n - 1; j > 0; --j) {
-          const TS uj = shfl_idx(j < 32 ? u0 : u1, j & 31);
-          if (i0 < j) u0 = fma(-M[j * ldl + i0], uj, u0);
-          if (i1 < j) u1 = fma(-M[j * ldl + i1], uj, u1);
-        }
-      }
-      if (i1 < n) t[i1 * ldt + c] = u1 * rinv[i1];
-    }
-    if (i0 < n) t[i0 * ldt + c] = u0 * rinv[i0];
+// cp.async of `cnt` contiguous elements by the group: 16 bytes at a time where both ends are aligned
+template <typename T>
+__device__ __forceinline__ void cp_async_flat(T* dst, const T* src, int cnt, Grp G) {
+  constexpr int V = 16 / (int)sizeof(T);
+  if ((((size_t)dst | (size_t)src) & 15) == 0 && cnt % V == 0) {
+#pragma unroll 2
+    for (int e = V * G.tid; e < cnt; e += V * G.nt)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst + e)),
+                   "l"(src + e)
+                   : "memory");
+  } else {
+#pragma unroll 2
+    for (int e = G.tid; e < cnt; e += G.nt) cp_async_elem(dst + e, src + e);
   }
-  gsync(G);
+}
+
+// t <- L^{-1} t (forward) or t <- L^{-T} t (backward) for nr columns, warp-
+// synchronous, without the group's barrier. Rows i and i + 32 of a column live
+// in lane i. M holds the multipliers of step j as its row j (forward: columns
+// of L divided by their diagonal, backward: rows of L): u_i -= M_ji u_j for the
+// rows i behind j, x = u * rinv.
+// A step is the broadcast of u_j and one FP64 FMA: 115 cycles in a row (a
+// device probe), 83 per column where a warp takes two (NC = 2), against 163
+// with a branch per step and its multipliers' latency: they are read four steps
+// ahead. (A broadcast through shared memory takes 119; one broadcast for two steps and
+// another FMA in its place, 133.)
+template <typename TS, int NC, bool TWO, bool BW, bool EXACT = false>
+__device__ __forceinline__ void trsv_cols(TS* t, int ldt, const TS* M, int ldl, const TS* rinv, int n, int c, int dc,
+                                          int lane) {
+  const int i0 = lane, i1 = lane + 32, r0 = min(i0, n - 1), r1 = min(i1, n - 1);  // (r: rows for addresses)
+  TS u0[NC], u1[NC], ma0[4], ma1[4], mb0[4], mb1[4];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    u0[q] = i0 < n ? t[i0 * ldt + c + q * dc] : TS(0);
+    u1[q] = TWO && i1 < n ? t[i1 * ldt + c + q * dc] : TS(0);
+  }
+  const int steps = n - 1;
+  auto load = [&](int s0, TS* m0, TS* m1) {
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const int k = min(s0 + s, steps), j = BW ? n - 1 - k : k;
+      m0[s] = M[j * ldl + r0];
+      m1[s] = TWO ? M[j * ldl + r1] : TS(0);
+    }
+  };
+  // four steps (those past the last one change dead rows only; EXACT leaves them
+  // out, where the FP64 pipe is the limit); no branch a lane could take alone
+  auto run = [&](int s0, const TS* m0, const TS* m1) {
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      if (EXACT && s0 + s >= steps) break;
+      const int j = BW ? n - 1 - s0 - s : s0 + s;
+      TS x[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) x[q] = shfl_idx(TWO && j >= 32 ? u1[q] : u0[q], j & 31);
+      if (!TWO || BW || j < 31) {
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          const TS v = fma(-m0[s], x[q], u0[q]);
+          u0[q] = (BW ? i0 < j : i0 > j) ? v : u0[q];
+        }
+      }
+      if (TWO && (!BW || j > 32)) {
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          const TS v = fma(-m1[s], x[q], u1[q]);
+          u1[q] = (BW ? i1 < j : i1 > j) ? v : u1[q];
+        }
+      }
+    }
+  };
+  load(0, ma0, ma1);
+#pragma unroll 1
+  for (int s0 = 0; s0 < steps; s0 += 4) {
+    load(s0 + 4, mb0, mb1);
+    run(s0, ma0, ma1);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      ma0[s] = mb0[s];
+      ma1[s] = mb1[s];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    if (i0 < n) t[i0 * ldt + c + q * dc] = u0[q] * rinv[i0];
+    if (TWO && i1 < n) t[i1 * ldt + c + q * dc] = u1[q] * rinv[i1];
+  }
+}
+template <typename TS, bool BW>
+__device__ __noinline__ void trsv_warp(TS* t, int ldt, const TS* M, int ldl, const TS* rinv, int n, int nr, Grp G) {
+  const int lane = G.tid & 31, nw = G.nt >> 5;
+  for (int c = G.tid >> 5; c < nr; c += 2 * nw) {
+    const bool two = c + nw < nr;
+    if (n <= 32) {
+      if (two) trsv_cols<TS, 2, false, BW>(t, ldt, M, ldl, rinv, n, c, nw, lane);
+      else trsv_cols<TS, 1, false, BW>(t, ldt, M, ldl, rinv, n, c, nw, lane);
+    } else {
+      if (two) trsv_cols<TS, 2, true, BW>(t, ldt, M, ldl, rinv, n, c, nw, lane);
+      else trsv_cols<TS, 1, true, BW>(t, ldt, M, ldl, rinv, n, c, nw, lane);
+    }
+  }
+}
+// (W: the one-warp tasks of small blocks, n <= 32 and a column at a time, which
+// share an SM by the dozen and want few registers)
+template <typename TS, bool W, bool BW>
+__device__ __forceinline__ void trsv_group(TS* t, int ldt, const TS* M, int ldl, const TS* rinv, int n, int nr,
+                                           Grp G) {
+  if (W) {
+    for (int c = 0; c < nr; ++c) trsv_cols<TS, 1, false, BW, true>(t, ldt, M, ldl, rinv, n, c, 0, G.tid);
+    return;
+  }
+  trsv_warp<TS, BW>(t, ldt, M, ldl, rinv, n, nr, G);
 }
 
 // Shared-memory view of a substitution task: double-buffered factor blocks
@@ -2201,7 +2299,7 @@ __device__ __forceinline__ SolveSmem<TS> solve_smem(unsigned char* sm, int n, in
   SolveSmem<TS> S;
   const SolLayout L = sol_layout(n, m, (int)sizeof(TS), fill);
   S.Rs = L.R;
-  S.ldL = odd(n);
+  S.ldL = n;
   S.ldZ = L.ldZ;
   S.ldV = L.ldV;
   S.L0 = (TS*)(sm + L.oL[0]);
@@ -2227,26 +2325,30 @@ __device__ __forceinline__ FactorView<float> factor_view(const LevelDesc& d, flo
 }
 
 // Start the asynchronous load of the factor blocks of stage j into buffer q
-// (D-hat with its columns (forward) or rows (backward) divided by the
-// diagonal, 1/diag, panel rows [r0, r1)).
+// (the multipliers of trsv_warp, both stored as its rows, 1/diag, panel rows
+// [r0, r1)).
 template <typename TS>
-__device__ void prefetch_stage_factor(const SolveSmem<TS>& S, int q, const LevelDesc& d, int j, int r0,
-                                      int r1, bool backward, Grp G) {
-  const int n = d.n, R = 2 * n + d.m;
-  const FactorView<TS> F = factor_view(d, TS(0));
-  // (the forward multipliers are stored transposed: element e is (e % n, e / n))
-  const TS* Lg = (backward ? F.MR : F.M) + (size_t)j * n * n;
-  for (int e = G.tid; e < n * n; e += G.nt) {
-    const int a = e / n, c = e - a * n;
-    cp_async_elem(S.L(q) + (backward ? a * S.ldL + c : c * S.ldL + a), Lg + e);
-  }
+__device__ void prefetch_stage_factor(const SolveSmem<TS>& S, int q, const FactorView<TS>& F, int n, int m, int j,
+                                      int r0, int r1, bool backward, Grp G) {
+  if (G.tid < 0) return;
+  const int R = 2 * n + m;
+  cp_async_flat(S.L(q), (backward ? F.MR : F.M) + (size_t)j * n * n, n * n, G);
   for (int e = G.tid; e < n; e += G.nt) cp_async_elem(S.rinv(q) + e, F.ri + (size_t)j * n + e);
   const TS* P = F.P + (size_t)j * R * n;
+  const Div by(n);
+#pragma unroll 2
   for (int e = G.tid + r0 * n; e < r1 * n; e += G.nt) {
-    const int r = e / n, c = e - r * n;
+    const int r = by(e), c = e - r * n;
     cp_async_elem(S.Z(q) + r * S.ldZ + c, P + e);
   }
   cp_async_commit();
+}
+
+// the warps without a column of trsv_warp, for the copies beside it; all of them
+// where every warp has one
+__device__ __forceinline__ Grp beside(Grp G, int nr) {
+  const int used = 32 * nr < G.nt ? 32 * nr : 0;
+  return Grp{G.tid - used, G.nt - used, G.bar};
 }
 
 __device__ __forceinline__ void stage_rows(const SegGeom& g, int i, int n, int m, int& r0, int& r1) {
@@ -2261,57 +2363,70 @@ __device__ __forceinline__ void stage_rows(const SegGeom& g, int i, int n, int m
 // blocks of the next stage stream in while the current one is solved.
 // (prefetched: the last stage's factor blocks were already requested into
 // buffer 0, see backward_prefetch)
-template <typename TS>
+template <typename TS, bool W>
 __device__ void backward_segment(const SolveSmem<TS>& S, const LevelDesc& d, const SegGeom& g,
                                  double* b, int ldb, int nr, int c0, Grp G, bool prefetched = false) {
   const int n = d.n, m = d.m;
   int r0, r1;
   stage_rows(g, g.len - 1, n, m, r0, r1);
-  if (!prefetched) prefetch_stage_factor(S, 0, d, g.f + g.len - 1, r0, r1, true, G);
+  const FactorView<TS> F = factor_view(d, TS(0));
+  const VecViews X(d, b, ldb, c0);
+  const Grp B = beside(G, nr);
+  if (!prefetched) prefetch_stage_factor(S, 0, F, n, m, g.f + g.len - 1, r0, r1, true, G);
+  const Div by(nr);
+  TS *t = S.t, *xe = S.V;  // y_j, then x_j; the E-rows of v: x_{j+1}
+  load_vec(t, S.ldV, (const double*)X.at(g.f + g.len - 1), X.ld, (const double*)nullptr, n, nr, G);
   for (int i = g.len - 1; i >= 0; --i) {
     const int j = g.f + i, q = (g.len - 1 - i) & 1;
     stage_rows(g, i, n, m, r0, r1);
-    const VecView y = level_vec(d, b, ldb, j, c0);
+    VecPrefetch<W ? 0 : 3> yp;  // y_{j-1}: its loads pass during this stage
     cp_async_wait_all();
     gsync(G);
     if (i > 0) {
-      int p0, p1;
-      stage_rows(g, i - 1, n, m, p0, p1);
-      prefetch_stage_factor(S, q ^ 1, d, j - 1, p0, p1, true, G);
+      yp.load(X.at(j - 1), X.ld, nullptr, n, nr, by, B);
     }
     const TS* Z = S.Z(q);
     // t = y_j - Z^T v over the active panel rows: four lanes per output (each
     // a quarter of the rows, two partial sums), shuffle-reduced
     {
       const int outs = n * nr, span = (outs * 4 + 31) & ~31, rows = r1 - r0;
+      auto v = [&](int r, int c) { return (r < n ? xe : S.V)[r * S.ldV + c]; };
+#pragma unroll 1
       for (int e = G.tid; e < span; e += G.nt) {
         const int o = e >> 2, qq = e & 3;
         const bool act = o < outs;
         const int oo = act ? o : 0;
-        const int c2 = oo / nr, c = oo - c2 * nr;
+        const int c2 = by(oo), c = oo - c2 * nr;
         const int ra = r0 + ((qq * rows) >> 2), rb = r0 + (((qq + 1) * rows) >> 2);
         TS a0 = 0, a1 = 0;
         int r = ra;
         if (act) {
+#pragma unroll(W ? 1 : 4)
           for (; r + 1 < rb; r += 2) {
-            a0 = fma(Z[r * S.ldZ + c2], S.V[r * S.ldV + c], a0);
-            a1 = fma(Z[(r + 1) * S.ldZ + c2], S.V[(r + 1) * S.ldV + c], a1);
+            a0 = fma(Z[r * S.ldZ + c2], v(r, c), a0);
+            a1 = fma(Z[(r + 1) * S.ldZ + c2], v(r + 1, c), a1);
           }
-          if (r < rb) a0 = fma(Z[r * S.ldZ + c2], S.V[r * S.ldV + c], a0);
+          if (r < rb) a0 = fma(Z[r * S.ldZ + c2], v(r, c), a0);
         }
         TS a = a0 + a1;
         a += __shfl_xor_sync(0xffffffffu, a, 1);
         a += __shfl_xor_sync(0xffffffffu, a, 2);
-        if (act && qq == 0) S.t[c2 * S.ldV + c] = (TS)y.p[(size_t)c2 * y.ld + c] - a;
+        if (act && qq == 0) t[c2 * S.ldV + c] -= a;
       }
     }
     gsync(G);
-    trsv_warp(S.t, S.ldV, S.L(q), S.ldL, S.rinv(q), n, nr, true, G);
-    store_vec(y.p, y.ld, S.t, S.ldV, n, nr, G);
-    for (int e = G.tid; e < n * nr; e += G.nt) {
-      const int r = e / nr, c = e - r * nr;
-      S.V[r * S.ldV + c] = S.t[r * S.ldV + c];
+    if (i > 0) {
+      int p0, p1;
+      stage_rows(g, i - 1, n, m, p0, p1);
+      prefetch_stage_factor(S, q ^ 1, F, n, m, j - 1, p0, p1, true, B);
     }
+    trsv_group<TS, W, true>(t, S.ldV, S.L(q), S.ldL, S.rinv(q), n, nr, G);
+    if (i > 0) yp.store(xe, S.ldV, n, nr, by, B);
+    gsync(G);
+    store_vec(X.at(j), X.ld, t, S.ldV, n, nr, G);
+    TS* const sw = t;
+    t = xe;
+    xe = sw;
   }
   gsync(G);
 }
@@ -2319,7 +2434,7 @@ __device__ void backward_segment(const SolveSmem<TS>& S, const LevelDesc& d, con
 // Forward substitution (Algorithm 2) for one segment; the top level (P = 1)
 // also solves the corner and runs its own backward sweep (Algorithm 3,
 // sequential phase). `skip`: per-system flags; a set flag returns at once.
-template <typename TS>
+template <typename TS, bool W>
 __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs, double* b, int ldb, int nr,
                              const int* skip, unsigned char* smraw, Grp G, int fwd_done, int c0) {
   const LevelDesc& d = descs[tk.desc];
@@ -2331,77 +2446,86 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
   const int oG = n, oW = n + m;
   const SegGeom g = seg_geom(d, tk.seg);
   const int k = tk.seg;
-  auto rhs = [&](int j, TS* dst) {  // this level's right-hand side of stage j
-    if (d.level == 1) {
-      const VecView v = level_vec(d, b, ldb, j, c0);
-      load_vec(dst, S.ldV, v.p, v.ld, (const double*)nullptr, n, nr, G);
-    } else {
-      load_vec(dst, S.ldV, d.RA + (size_t)j * n * kRhsChunk + c0, kRhsChunk,
-               d.RB + (size_t)j * n * kRhsChunk + c0, n, nr, G);
-    }
-  };
   int r0, r1;
   stage_rows(g, 0, n, m, r0, r1);
-  if (!fwd_done) prefetch_stage_factor(S, 0, d, g.f, r0, r1, false, G);
+  const FactorView<TS> F = factor_view(d, TS(0));
+  const VecViews X(d, b, ldb, c0);
+  // right-hand side of stage j of this level: the caller's, or RA + RB
+  const double* const ra = d.level == 1 ? X.p : d.RA + c0;
+  const double* const rb = d.level == 1 ? nullptr : d.RB + c0;
+  const int ldr = d.level == 1 ? X.ld : kRhsChunk;
+  const Grp B = beside(G, nr);
+  if (!fwd_done) prefetch_stage_factor(S, 0, F, n, m, g.f, r0, r1, false, G);
   // V_G <- 0, V_W <- rhs of the separator, t <- rhs of the first stage
   for (int e = G.tid; e < S.Rs * S.ldV; e += G.nt) S.V[e] = TS(0);
   gsync(G);
+  auto rhs = [&](int j, TS* dst) {
+    const size_t o = (size_t)j * n * ldr;
+    load_vec(dst, S.ldV, ra + o, ldr, rb ? rb + o : nullptr, n, nr, G);
+  };
   if (g.hasW) rhs(g.f - 1, S.V + oW * S.ldV);
   rhs(g.f, S.t);
+  const Div by(nr);
+  // this stage's vector, and the E-rows of the panel product: the next stage's
+  TS *t = S.t, *tn = S.V;
   // a bordered factorization already carried this forward sweep (fwd_done)
   for (int i = 0; i < (fwd_done ? 0 : g.len); ++i) {
     const int j = g.f + i, q = i & 1;
+    const bool more = i + 1 < g.len;
     stage_rows(g, i, n, m, r0, r1);
-    if (i + 1 < g.len) rhs(j + 1, S.V);  // V_E <- next stage's rhs (else 0: F-hat term)
+    VecPrefetch<W ? 0 : 3> bp;  // the next stage's rhs: its loads pass during the solve
+    if (more) {
+      const size_t o = (size_t)(j + 1) * n * ldr;
+      bp.load(ra + o, ldr, rb ? rb + o : nullptr, n, nr, by, B);
+    }
     cp_async_wait_all();
     gsync(G);
-    if (i + 1 < g.len) {
+    if (more) {
       int p0, p1;
       stage_rows(g, i + 1, n, m, p0, p1);
-      prefetch_stage_factor(S, q ^ 1, d, j + 1, p0, p1, false, G);
+      prefetch_stage_factor(S, q ^ 1, F, n, m, j + 1, p0, p1, false, B);
     }
-    trsv_warp(S.t, S.ldV, S.L(q), S.ldL, S.rinv(q), n, nr, false, G);
-    const VecView y = level_vec(d, b, ldb, j, c0);
-    store_vec(y.p, y.ld, S.t, S.ldV, n, nr, G);
+    trsv_group<TS, W, false>(t, S.ldV, S.L(q), S.ldL, S.rinv(q), n, nr, G);
+    if (more) bp.store(tn, S.ldV, n, nr, by, B);
+    else
+      for (int e = G.tid; e < n * S.ldV; e += G.nt) tn[e] = TS(0);  // the F-hat term
+    gsync(G);
+    store_vec(X.at(j), X.ld, t, S.ldV, n, nr, G);
     // [V_E; V_G; V_W] -= Z y over the active panel rows: four lanes per output
     // (each a quarter of the dot product, two partial sums), shuffle-reduced
     const TS* Z = S.Z(q);
     {
       const int outs = (r1 - r0) * nr, span = (outs * 4 + 31) & ~31;
+#pragma unroll 1
       for (int e = G.tid; e < span; e += G.nt) {
         const int o = e >> 2, qq = e & 3;
         const bool act = o < outs;
         const int oo = act ? o : 0;
-        const int r = r0 + oo / nr, c = oo - (oo / nr) * nr;
+        const int r = r0 + by(oo), c = oo - (r - r0) * nr;
         const int k0 = (qq * n) >> 2, k1 = ((qq + 1) * n) >> 2;
         TS a0 = 0, a1 = 0;
         int t2 = k0;
         if (act) {
+#pragma unroll(W ? 1 : 4)
           for (; t2 + 1 < k1; t2 += 2) {
-            a0 = fma(Z[r * S.ldZ + t2], S.t[t2 * S.ldV + c], a0);
-            a1 = fma(Z[r * S.ldZ + t2 + 1], S.t[(t2 + 1) * S.ldV + c], a1);
+            a0 = fma(Z[r * S.ldZ + t2], t[t2 * S.ldV + c], a0);
+            a1 = fma(Z[r * S.ldZ + t2 + 1], t[(t2 + 1) * S.ldV + c], a1);
           }
-          if (t2 < k1) a0 = fma(Z[r * S.ldZ + t2], S.t[t2 * S.ldV + c], a0);
+          if (t2 < k1) a0 = fma(Z[r * S.ldZ + t2], t[t2 * S.ldV + c], a0);
         }
         TS a = a0 + a1;
         a += __shfl_xor_sync(0xffffffffu, a, 1);
         a += __shfl_xor_sync(0xffffffffu, a, 2);
-        if (act && qq == 0) S.V[r * S.ldV + c] -= a;
+        if (act && qq == 0) (r < n ? tn : S.V)[r * S.ldV + c] -= a;
       }
     }
-    gsync(G);
-    if (i + 1 < g.len) {
-      for (int e = G.tid; e < n * nr; e += G.nt) {
-        const int r = e / nr, c = e - r * nr;
-        S.t[r * S.ldV + c] = S.V[r * S.ldV + c];
-        S.V[r * S.ldV + c] = TS(0);
-      }
-      gsync(G);  // V_E is reloaded at the top of the next stage
-    }
+    TS* const sw = t;
+    t = tn;
+    tn = sw;
   }
   gsync(G);
   if (!d.is_top) {
-    if (g.hasF) store_vec(d.YB + (size_t)k * n * kRhsChunk + c0, kRhsChunk, S.V, S.ldV, n, nr, G);
+    if (g.hasF) store_vec(d.YB + (size_t)k * n * kRhsChunk + c0, kRhsChunk, t, S.ldV, n, nr, G);
     if (g.hasW)
       store_vec(d.YA + (size_t)(k - 1) * n * kRhsChunk + c0, kRhsChunk, S.V + oW * S.ldV, S.ldV, n, nr, G);
     if (m) store_vec(d.ygpart + (size_t)k * m * kRhsChunk + c0, kRhsChunk, S.V + oG * S.ldV, S.ldV, m, nr, G);
@@ -2428,15 +2552,19 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
             gv[r * S.ldV + c] = (TS)((bg[(size_t)r * ldb + c] + v) + (double)S.V[(oG + r) * S.ldV + c]);
           });
     }
-    for (int e = G.tid; e < mg * mg; e += G.nt) {  // R-hat: columns scaled, rows scaled
+    for (int e = G.tid; e < mg * mg; e += G.nt) {  // R-hat: columns scaled (transposed), rows scaled
       const int r = e / mg, c = e - r * mg;
-      S.L(0)[r * ldR + c] = (TS)(d.Rhat[r * m + c] * d.Rri[c]);
+      S.L(0)[c * ldR + r] = (TS)(d.Rhat[r * m + c] * d.Rri[c]);
       S.L(1)[r * ldR + c] = (TS)(d.Rhat[r * m + c] * d.Rri[r]);
     }
     for (int e = G.tid; e < mg; e += G.nt) S.rinv(0)[e] = (TS)d.Rri[e];
     gsync(G);
-    if (!fwd_done) trsv_warp(gv, S.ldV, S.L(0), ldR, S.rinv(0), mg, nr, false, G);
-    trsv_warp(gv, S.ldV, S.L(1), ldR, S.rinv(0), mg, nr, true, G);
+    if (!fwd_done) {
+      trsv_group<TS, W, false>(gv, S.ldV, S.L(0), ldR, S.rinv(0), mg, nr, G);
+      gsync(G);
+    }
+    trsv_group<TS, W, true>(gv, S.ldV, S.L(1), ldR, S.rinv(0), mg, nr, G);
+    gsync(G);
     store_vec(bg, ldb, gv, S.ldV, mg, nr, G);
   }
   // V <- [0; x_g; 0; -] for the backward sweep of the top level (bordered rows 0)
@@ -2446,13 +2574,13 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
     else S.V[e] = S.t[(r - oG) * S.ldV + (e - r * S.ldV)];
   }
   gsync(G);
-  backward_segment(S, d, g, b, ldb, nr, c0, G);
+  backward_segment<TS, W>(S, d, g, b, ldb, nr, c0, G);
 }
 
 // Backward substitution (Algorithm 3, parallel phase) for one segment below
 // the top level: needs x_g (already in b), the separator solutions of the
 // next level (x at s_k and s_{k+1}), and this level's y.
-template <typename TS>
+template <typename TS, bool W = false>
 __device__ void backward_task(const Task tk, const LevelDesc* __restrict__ descs, double* b, int ldb, int nr,
                               const int* skip, unsigned char* smraw, Grp G, int c0 = 0, bool prefetched = false) {
   const LevelDesc& d = descs[tk.desc];
@@ -2476,7 +2604,7 @@ __device__ void backward_task(const Task tk, const LevelDesc* __restrict__ descs
     store_vec(xs.p, xs.ld, S.V + oW * S.ldV, S.ldV, n, nr, G);
   }
   gsync(G);
-  backward_segment(S, d, g, b, ldb, nr, c0, G, prefetched);
+  backward_segment<TS, W>(S, d, g, b, ldb, nr, c0, G, prefetched);
 }
 
 // The factor blocks of the backward sweep's first stage (the segment's last)
@@ -2488,14 +2616,14 @@ __device__ void backward_prefetch(const Task tk, const LevelDesc& d, unsigned ch
   const SegGeom g = seg_geom(d, tk.seg);
   int r0, r1;
   stage_rows(g, g.len - 1, d.n, d.m, r0, r1);
-  prefetch_stage_factor(S, 0, d, g.f + g.len - 1, r0, r1, true, G);
+  prefetch_stage_factor(S, 0, factor_view(d, TS(0)), d.n, d.m, g.f + g.len - 1, r0, r1, true, G);
 }
 
 
 // One CTA per task (blocks above kWarpMaxN), or one warp per task with a
 // shared-memory slice each (small blocks; `slice` bytes per warp).
 template <typename TS>
-__global__ void __launch_bounds__(kSolveThreads) k_forward(const LevelDesc* __restrict__ descs,
+__global__ void __launch_bounds__(kSolveThreads, 2) k_forward(const LevelDesc* __restrict__ descs,
                                                            const Task* __restrict__ tasks, double* b,
                                                            int ldb, int nr, const int* skip, int fwd_done,
                                                            int split) {
@@ -2506,7 +2634,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_forward(const LevelDesc* __re
   forward_task<TS>(tasks[blockIdx.x / split], descs, b + c0, ldb, cn, skip, smraw, cta_grp(), fwd_done, c0);
 }
 template <typename TS>
-__global__ void __launch_bounds__(kSolveThreads) k_backward(const LevelDesc* __restrict__ descs,
+__global__ void __launch_bounds__(kSolveThreads, 2) k_backward(const LevelDesc* __restrict__ descs,
                                                             const Task* __restrict__ tasks, double* b,
                                                             int ldb, int nr, const int* skip, int split) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -2515,23 +2643,23 @@ __global__ void __launch_bounds__(kSolveThreads) k_backward(const LevelDesc* __r
   backward_task<TS>(tasks[blockIdx.x / split], descs, b + c0, ldb, cn, skip, smraw, cta_grp(), c0);
 }
 template <typename TS>
-__global__ void __launch_bounds__(256) k_forward_w(const LevelDesc* __restrict__ descs,
+__global__ void __launch_bounds__(256, 3) k_forward_w(const LevelDesc* __restrict__ descs,
                                                    const Task* __restrict__ tasks, int ntasks, double* b,
                                                    int ldb, int nr, const int* skip, int slice, int fwd_done) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int wid = threadIdx.x >> 5, t = blockIdx.x * (blockDim.x >> 5) + wid;
   if (t >= ntasks) return;  // whole warp
-  forward_task<TS>(tasks[t], descs, b, ldb, nr, skip, smraw + (size_t)wid * slice,
+  forward_task<TS, true>(tasks[t], descs, b, ldb, nr, skip, smraw + (size_t)wid * slice,
                    Grp{(int)(threadIdx.x & 31), 32, -1}, fwd_done);
 }
 template <typename TS>
-__global__ void __launch_bounds__(256) k_backward_w(const LevelDesc* __restrict__ descs,
+__global__ void __launch_bounds__(256, 3) k_backward_w(const LevelDesc* __restrict__ descs,
                                                     const Task* __restrict__ tasks, int ntasks, double* b,
                                                     int ldb, int nr, const int* skip, int slice) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int wid = threadIdx.x >> 5, t = blockIdx.x * (blockDim.x >> 5) + wid;
   if (t >= ntasks) return;  // whole warp
-  backward_task<TS>(tasks[t], descs, b, ldb, nr, skip, smraw + (size_t)wid * slice,
+  backward_task<TS, true>(tasks[t], descs, b, ldb, nr, skip, smraw + (size_t)wid * slice,
                     Grp{(int)(threadIdx.x & 31), 32, -1});
 }
 
@@ -2549,7 +2677,7 @@ __global__ void __launch_bounds__(256) k_backward_w(const LevelDesc* __restrict_
 // launch. unmet: every wait expects one item more than its level has (a
 // test of the timeout path).
 template <typename TS>
-__global__ void __launch_bounds__(kSolveThreads) k_backward_chain(const LevelDesc* __restrict__ descs,
+__global__ void __launch_bounds__(kSolveThreads, 2) k_backward_chain(const LevelDesc* __restrict__ descs,
                                                                   const Task* __restrict__ tasks, ChainPlan cp,
                                                                   int* ctr, double* b, int ldb, int nr,
                                                                   const int* skip, Info* info,
