@@ -72,6 +72,25 @@ def test_pivot_reciprocal(kkt):
 
 
 @pytest.mark.parametrize("scale", [0, 1014, -1000])
+@pytest.mark.parametrize("N,n,m,P", [(3, 1, 0, 1), (9, 2, 1, 3), (9, 6, 2, 3), (7, 8, 4, 2), (7, 15, 0, 2), (5, 16, 15, 1)])
+def test_small_factor_blocks(kkt, orc, N, n, m, P, scale):
+    """As test_factor_blocks, one warp per task."""
+    D, E, G, R = system(N, n, m)
+    Fo = orc.par_factor(D, E, G, R, P=P)
+    s, h = 2.0 ** scale, 2.0 ** (scale // 2)
+    hd = kkt.kkt_create(N, n, m, P)
+    try:
+        kkt.kkt_factor(hd, dev(D * s), dev(E * s), dev(G * s) if m else None, dev(R * s) if m else None)
+        F = kkt.kkt_get_factor(hd, N, n, m)
+        assert kkt.kkt_get_info(hd)["status"] == 0
+    finally:
+        kkt.kkt_destroy(hd)
+    for k in ("Ld", "Le", "Lw", "Lh", "Lg", "Lr"):
+        if F[k].size:
+            np.testing.assert_allclose(F[k] / h, Fo[k], rtol=0, atol=1e-13 * max(1.0, np.abs(Fo[k]).max()), err_msg=k)
+
+
+@pytest.mark.parametrize("scale", [0, 1014, -1000])
 @pytest.mark.parametrize("N,n,m,P", [(5, 17, 0, 1), (7, 23, 3, 2), (5, 24, 15, 1), (9, 25, 2, 3), (7, 31, 1, 2),
                                      (7, 32, 8, 2), (5, 33, 0, 2), (7, 40, 5, 2), (5, 41, 4, 1), (5, 48, 15, 2)])
 def test_factor_blocks(kkt, orc, N, n, m, P, scale):
