@@ -571,34 +571,45 @@ __device__ __forceinline__ void ldl_rows(double* Z, int ldz, int r0, int r1, con
 }
 
 // digits of the eight columns [c0, c0 + kLB) of rows [r0, r1) of src (ld) into
-// dst[(r - r0) kLB ..] with exponents ex[r - r0]; eight lanes a row
-__device__ __forceinline__ void oz_encode8(const double* src, int ld, int c0, int r0, int r1, oz::u64* dst, int* ex,
-                                           Grp G) {
+// dst[(r - r0) kLB ..] with exponents ex[r - r0]; eight lanes a row. Column k is
+// scaled by 2^s_k (oz::balance of rinv) for the panel rows, 2^-s_k (NEG) for
+// the operand rows: u and m carry L_kk and 1 / L_kk, so without it a row's
+// exponent would be set by a column of another unit than the one that sets
+// its partner's, and the products of the others would lose the ratio of the
+// pivots' roots (one system of N = 50, n = 48, variables in units within 10^+-6:
+// 5e-9 off its solution in equal units, 10^+-9: 3e-3; with the scaling no bit
+// differs). With it the operands are the rows of x and L to a factor of two.
+// Rows that are not split are not stored (their products read src).
+template <bool NEG>
+__device__ __forceinline__ void oz_encode8(const double* src, int ld, int c0, int r0, int r1, const double* rinv,
+                                           oz::u64* dst, int* ex, Grp G) {
   const int sub = G.tid & 7, cnt = (r1 - r0 + 3) & ~3;  // (whole warps: four rows each)
+  const int sc = NEG ? -oz::balance(rinv[c0 + sub]) : oz::balance(rinv[c0 + sub]);
   for (int r = G.tid >> 3; r < cnt; r += G.nt >> 3) {
     const int rr = min(r0 + r, r1 - 1);
     const oz::u64 b = oz::dbits(src[rr * ld + c0 + sub]);
-    int em = oz::mag(b);
-    for (int o = 4; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
-    const int f = oz::row_exp(em);
+    int key = oz::scaled_key(b, sc);
+    for (int o = 4; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+    const int f = oz::scaled_row_exp(key);
     if (r0 + r < r1) {
-      dst[r * kLB + sub] = f == oz::kFp64Row ? b : oz::encode(b, f);
+      dst[r * kLB + sub] = oz::encode(b, f - sc);  // (not read where f is kFp64Row)
       if (sub == 0) ex[r] = f;
     }
   }
 }
 
 // Panel rows [r0, r1) behind the solved block [c0, c0 + kLB): Z[r][c] -= u_r
-// m_c^T for c >= c0 + kLB; by group G, which synchronizes before (u) and after.
+// m_c^T for c >= c0 + kLB; by group G, which synchronizes before (u, and rinv of
+// the block) and after.
 __device__ __forceinline__ void ldl_panel_update(double* Z, int ldz, int n, int r0, int r1, const double* M, int ld,
-                                                 int c0, const SweepBuf& B, Grp G) {
+                                                 const double* rinv, int c0, const SweepBuf& B, Grp G) {
   const int cb = c0 + kLB, nc = (n - cb + 7) >> 3, nr = (r1 - r0 + 15) >> 4, nw = G.nt >> 5;
-  oz_encode8(Z, ldz, c0, r0, r1, B.u, B.eu, G);
-  oz_encode8(M, ld, c0, cb, n, B.m + cb * kLB, B.em + cb, G);
+  oz_encode8<false>(Z, ldz, c0, r0, r1, rinv, B.u, B.eu, G);
+  oz_encode8<true>(M, ld, c0, cb, n, rinv, B.m + cb * kLB, B.em + cb, G);
   gsync(G);
   for (int t = G.tid >> 5; t < nr * nc; t += nw) {
     const int i = t / nc, j = t - i * nc;
-    oz::tile8(Z, ldz, B.u, B.eu, r0, B.m, B.em, 0, r0 + 16 * i, r1, cb + 8 * j, n, G.tid & 31);
+    oz::tile8(Z, ldz, B.u, B.eu, r0, B.m, B.em, 0, r0 + 16 * i, r1, cb + 8 * j, n, Z + c0, ldz, M + c0, ld, G.tid & 31);
   }
 }
 
@@ -640,7 +651,7 @@ __device__ void ldl_sweep(double* A, int ld, int n, double* M, double* rinv, int
       ldl_rows(Z, ldz, r0, r1, M, ld, p0, pn, W);
       if (cn > 0) {
         gsync(W);
-        ldl_panel_update(Z, ldz, n, r0, r1, M, ld, p0, B, W);
+        ldl_panel_update(Z, ldz, n, r0, r1, M, ld, rinv, p0, B, W);
       }
     }
     __syncthreads();
@@ -655,15 +666,16 @@ __device__ void ldl_sweep(double* A, int ld, int n, double* M, double* rinv, int
   }
 }
 
-// Panel rows [r0, r1) against a pivot block received as M: the operations of
-// ldl_sweep (u, unscaled). By the whole CTA; ends with a block barrier.
-__device__ void ldl_panel(double* Z, int ldz, int r0, int r1, const double* M, int ld, int n, const SweepBuf& B) {
+// Panel rows [r0, r1) against a pivot block received as M and rinv: the
+// operations of ldl_sweep (u, unscaled). By the whole CTA; ends with a block barrier.
+__device__ void ldl_panel(double* Z, int ldz, int r0, int r1, const double* M, const double* rinv, int ld, int n,
+                          const SweepBuf& B) {
   const Grp C = cta_grp();
   for (int c0 = 0; c0 < n; c0 += kLB) {
     ldl_rows(Z, ldz, r0, r1, M, ld, c0, min(kLB, n - c0), C);
     __syncthreads();
     if (c0 + kLB < n) {
-      ldl_panel_update(Z, ldz, n, r0, r1, M, ld, c0, B, C);
+      ldl_panel_update(Z, ldz, n, r0, r1, M, ld, rinv, c0, B, C);
       __syncthreads();
     }
   }
@@ -1351,7 +1363,7 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
       const int r0 = eRows ? 0 : n, b = i & 1;
       cluster_arrive();  // done with stage i-1
       cluster_wait();    // stage i's blocks are in buffer b
-      ldl_panel(Z, ldZ, oW, R, Mbuf(b), ldD, n, SB);
+      ldl_panel(Z, ldZ, oW, R, Mbuf(b), rinvbuf(b), ldD, n, SB);
       // (the W-rows' exponents live in buffer 0's array, of which the producer
       // writes the rows below oW only)
       panel_out(Z, ldZ, oW, R, n, rinvbuf(b), rowf, d.Lp + (size_t)j * R * n, oW, R, -1, nullptr, 1, C);

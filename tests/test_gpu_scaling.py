@@ -1,0 +1,139 @@
+"""Variables in different units. With S a diagonal of powers of two, the Cholesky
+factor of S Psi S is S L and the solution for S b is S^-1 x, both exactly: every
+rounding of the elimination, of its digit products and of the substitutions
+scales with the row and column it belongs to. So every layout has to return the
+unscaled answer's bits, S drawn per variable within 2^+-30."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kkt():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2511_00946_gb300 as k
+    return k
+
+
+def dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float64)).cuda()
+
+
+def system(N, n, m, seed=0):
+    """I + perturbations: couplings and arrow of 2-norm at most 1/8, so that the
+    eigenvalues lie in [1/2, 3/2]."""
+    rng = np.random.default_rng([N, n, m, seed])
+
+    def small(*shape):
+        A = rng.normal(size=shape)
+        return A / (8 * np.sqrt((A ** 2).sum(axis=(-2, -1), keepdims=True))) if A.size else A
+
+    S = small(N, n, n)
+    D = np.eye(n) + S + S.transpose(0, 2, 1)
+    return D, small(N - 1, n, n), small(N, m, n) / np.sqrt(N), np.eye(m)
+
+
+def scaled(sys, s, sg):
+    """S Psi S: s (N, n) for the stages, sg (m,) for the arrow."""
+    D, E, G, R = sys
+    return (s[:, :, None] * D * s[:, None, :], s[1:, :, None] * E * s[:-1, None, :],
+            sg[None, :, None] * G * s[:, None, :], sg[:, None] * R * sg[None, :])
+
+
+def units(N, n, m, seed=1):
+    rng = np.random.default_rng([seed, N, n, m])
+    return 2.0 ** rng.integers(-30, 31, (N, n)), 2.0 ** rng.integers(-30, 31, m)
+
+
+def args(sys, m):
+    return [dev(a) if k < 2 or m else None for k, a in enumerate(sys)]
+
+
+@pytest.mark.parametrize("N,n,m,P", [(7, 16, 3, 2), (5, 17, 0, 1), (9, 20, 2, 3), (7, 32, 8, 2), (5, 33, 1, 1),
+                                     (9, 45, 5, 3), (7, 48, 15, 2)])
+def test_factor_and_solutions_of_one_system(kkt, N, n, m, P):
+    """One CTA per task, pairs, and caller-owned memory; factor blocks, several
+    right-hand sides and the bordered pass."""
+    A = system(N, n, m)
+    s, sg = units(N, n, m)
+    S = np.concatenate([s.ravel(), sg])
+    b = np.random.default_rng(n).normal(size=(N * n + m, 2))
+    for pairing in (kkt.KKT_PAIR_OFF, kkt.KKT_PAIR_ON):
+        got = []
+        for M, c in ((A, b), (scaled(A, s, sg), S[:, None] * b)):
+            h = kkt.kkt_create(N, n, m, P)
+            try:
+                kkt.kkt_set_pairing(h, pairing)
+                a = args(M, m)
+                x, y, z = dev(c), dev(c[:, 0]), dev(c[:, 0])
+                kkt.kkt_factor(h, *a)
+                F = kkt.kkt_get_factor(h, N, n, m)
+                kkt.kkt_solve(h, x)
+                kkt.kkt_factor_solve(h, *a, y)
+                kkt.kkt_solve_noalloc(N, n, m, P, *a, z)
+                assert kkt.kkt_get_info(h)["status"] == 0
+                got.append((F, x.cpu().numpy(), y.cpu().numpy(), z.cpu().numpy()))
+            finally:
+                kkt.kkt_destroy(h)
+        (F, *xs), (Fs, *xss) = got
+        for i in range(N):
+            np.testing.assert_array_equal(s[i][:, None] * F["Ld"][i], Fs["Ld"][i], err_msg=f"stage {i}")
+        for x, xsc in zip(xs, xss):
+            sc = S if x.ndim == 1 else S[:, None]
+            np.testing.assert_array_equal(sc * xsc, x, err_msg=f"pairing {pairing}")
+
+
+@pytest.mark.parametrize("N,n,m,levels", [(63, 17, 3, [16, 8, 4, 2, 1]), (63, 32, 8, [16, 8, 4, 2, 1]),
+                                          (47, 48, 0, [12, 6, 3, 1])])
+def test_solutions_on_clusters(kkt, N, n, m, levels):
+    """A plan whose deep levels run on clusters."""
+    A = system(N, n, m)
+    s, sg = units(N, n, m)
+    S = np.concatenate([s.ravel(), sg])
+    b = np.random.default_rng(n).normal(size=N * n + m)
+    got = []
+    for M, c in ((A, b), (scaled(A, s, sg), S * b)):
+        h = kkt.kkt_create_plan(N, n, m, levels)
+        try:
+            assert max(kkt.kkt_factor_ctas_per_task(h, l) for l in range(len(levels))) > 2
+            a = args(M, m)
+            x, y = dev(c), dev(c)
+            kkt.kkt_factor(h, *a)
+            kkt.kkt_solve(h, x)
+            kkt.kkt_factor_solve(h, *a, y)
+            assert kkt.kkt_get_info(h)["status"] == 0
+            got.append((x.cpu().numpy(), y.cpu().numpy()))
+        finally:
+            kkt.kkt_destroy(h)
+    for x, xs in zip(*got):
+        np.testing.assert_array_equal(S * xs, x)
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+@pytest.mark.parametrize("n,m", [(20, 3), (32, 8)])
+def test_solutions_of_a_batch(kkt, n, m, persistent):
+    """More systems than the chip holds tasks of 256 threads; every other one scaled."""
+    import torch
+    count, N, P = 4 * torch.cuda.get_device_properties(0).multi_processor_count + 2, 5, 2
+    A = system(N, n, m)
+    s, sg = units(N, n, m)
+    S = np.concatenate([s.ravel(), sg])
+    pick = [A, scaled(A, s, sg)]
+    b = np.random.default_rng(n).normal(size=N * n + m)
+    a = [dev(np.concatenate([pick[i % 2][k].ravel() for i in range(count)])) for k in range(4)]
+    x = dev(np.concatenate([b if i % 2 == 0 else S * b for i in range(count)]))
+    h = kkt.kkt_batch_create([N] * count, [n] * count, [m] * count, [P] * count)
+    try:
+        kkt.kkt_set_persistent(h, persistent)
+        kkt.kkt_factor(h, *a)
+        kkt.kkt_solve(h, x)
+        assert kkt.kkt_get_info(h)["status"] == 0
+    finally:
+        kkt.kkt_destroy(h)
+    x = x.cpu().numpy().reshape(count, -1)
+    for i in range(count):
+        np.testing.assert_array_equal(x[i] if i % 2 == 0 else S * x[i], x[0], err_msg=f"system {i}")
