@@ -398,13 +398,49 @@ __device__ void syrk_trap(double* T, int ldt, const TZ* Zlo, const TZ* Z, int zs
 // T[a][b] -= sum_t Z[a][t] Z[b][t] for ra0 <= a < ra1, cb0 <= b <= a (cb0 <=
 // ra0), rows in digits (panel_out). Panel rows below `zsplit` are read from
 // (Zlo, flo), the others from (Z, fz). One 16 x 8 tile per warp at a time.
-// Every element is an exact sum rounded once, so the result does not depend
-// on the tiling. Ends with the group's barrier.
+// Every element is one sum rounded once, so the result does not depend on the
+// tiling.
+// BORDER: row ry is a bordered right-hand side. Its entries have no common
+// scale (a right-hand side may hold numbers 10^12 apart that nothing couples),
+// so it keeps its doubles and its products are FP64 FMAs against the solved
+// rows in device memory, Pd (row-major, n columns; complete): two lanes a row,
+// jobs of sixteen rows ahead of the tiles in the warps' list, where the FP64 pipe
+// is idle beside the other warps' tiles (1172 us for N = 777, n = 45; behind the
+// tiles 1175, four lanes a row 1177 and 1190).
+// Ends with the group's barrier.
+template <bool BORDER>
 __device__ void oz_syrk(double* T, int ldt, const double* Zlo, const int* flo, const double* Z, const int* fz,
-                        int zsplit, int ldz, int ra0, int ra1, int cb0, int n, Grp G) {
+                        int zsplit, int ldz, int ra0, int ra1, int cb0, int n, int ry, const double* Pd, Grp G) {
   const int lane = G.tid & 31, nw = G.nt >> 5, w0 = ra0 - cb0;
-  // row tile i has cols(i) column tiles; this warp takes every nw-th tile
   int i = 0, j = G.tid >> 5;
+  if constexpr (BORDER) {
+    // (ry, b) for cb0 <= b < ry, then (a, ry) for the rows a behind ry
+    const int left = ry >= ra0 && ry < ra1 ? ry - cb0 : 0, a0 = max(ra0, ry + 1), tot = left + max(0, ra1 - a0);
+    const double* const y = (ry < zsplit ? Zlo : Z) + ry * ldz;
+    for (; 16 * j < tot; j += nw) {
+      const int e = 16 * j + (lane >> 1), ee = min(e, tot - 1), o = ee < left ? cb0 + ee : a0 + ee - left;
+      const double* const p = Pd + (size_t)o * n;
+      double acc = 0.0;
+#pragma unroll 1
+      for (int k0 = 0; k0 < n; k0 += 16) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int k = k0 + 2 * q + (lane & 1);
+          v[q] = k < n ? p[k] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int k = k0 + 2 * q;
+          if (k < n) acc = fma(v[q], k + (lane & 1) < n ? y[k + (lane & 1)] : 0.0, acc);  // (warp-uniform)
+        }
+      }
+      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+      if (e < tot && (lane & 1) == 0) T[max(o, ry) * ldt + min(o, ry)] -= acc;
+    }
+    j -= (tot + 15) >> 4;
+  }
+  // row tile i has cols(i) column tiles; this warp takes every nw-th tile
   for (;;) {
     for (; ra0 + 16 * i < ra1; ++i) {
       const int cols = (w0 + min(16 * i + 16, ra1 - ra0) + 7) >> 3;
@@ -412,7 +448,7 @@ __device__ void oz_syrk(double* T, int ldt, const double* Zlo, const int* flo, c
       j -= cols;
     }
     if (ra0 + 16 * i >= ra1) break;
-    oz::tile(T, ldt, Zlo, flo, Z, fz, zsplit, ldz, ra0 + 16 * i, ra1, cb0 + 8 * j, ra1, n, lane);
+    oz::tile<BORDER>(T, ldt, Zlo, flo, Z, fz, zsplit, ldz, ra0 + 16 * i, ra1, cb0 + 8 * j, ra1, n, lane, ry);
     j += nw;
   }
   gsync(G);
@@ -579,10 +615,10 @@ __device__ __forceinline__ void ldl_rows(double* Z, int ldz, int r0, int r1, con
 // pivots' roots (one system of N = 50, n = 48, variables in units within 10^+-6:
 // 5e-9 off its solution in equal units, 10^+-9: 3e-3; with the scaling no bit
 // differs). With it the operands are the rows of x and L to a factor of two.
-// Rows that are not split are not stored (their products read src).
-template <bool NEG>
+// Rows that are not split and, BORDER, row ry are not stored (their products read src).
+template <bool NEG, bool BORDER>
 __device__ __forceinline__ void oz_encode8(const double* src, int ld, int c0, int r0, int r1, const double* rinv,
-                                           oz::u64* dst, int* ex, Grp G) {
+                                           int ry, oz::u64* dst, int* ex, Grp G) {
   const int sub = G.tid & 7, cnt = (r1 - r0 + 3) & ~3;  // (whole warps: four rows each)
   const int sc = NEG ? -oz::balance(rinv[c0 + sub]) : oz::balance(rinv[c0 + sub]);
   for (int r = G.tid >> 3; r < cnt; r += G.nt >> 3) {
@@ -590,9 +626,9 @@ __device__ __forceinline__ void oz_encode8(const double* src, int ld, int c0, in
     const oz::u64 b = oz::dbits(src[rr * ld + c0 + sub]);
     int key = oz::scaled_key(b, sc);
     for (int o = 4; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-    const int f = oz::scaled_row_exp(key);
+    const int f = BORDER && rr == ry ? 0 : oz::scaled_row_exp(key);
     if (r0 + r < r1) {
-      dst[r * kLB + sub] = oz::encode(b, f - sc);  // (not read where f is kFp64Row)
+      if (!(BORDER && rr == ry)) dst[r * kLB + sub] = oz::encode(b, f - sc);  // (not read where f is kFp64Row)
       if (sub == 0) ex[r] = f;
     }
   }
@@ -600,16 +636,36 @@ __device__ __forceinline__ void oz_encode8(const double* src, int ld, int c0, in
 
 // Panel rows [r0, r1) behind the solved block [c0, c0 + kLB): Z[r][c] -= u_r
 // m_c^T for c >= c0 + kLB; by group G, which synchronizes before (u, and rinv of
-// the block) and after.
+// the block) and after. BORDER: row ry (a bordered right-hand side, see oz_syrk)
+// in FP64 FMAs, a column per lane, beside the tiles.
+template <bool BORDER>
 __device__ __forceinline__ void ldl_panel_update(double* Z, int ldz, int n, int r0, int r1, const double* M, int ld,
-                                                 const double* rinv, int c0, const SweepBuf& B, Grp G) {
+                                                 const double* rinv, int c0, int ry, const SweepBuf& B, Grp G) {
   const int cb = c0 + kLB, nc = (n - cb + 7) >> 3, nr = (r1 - r0 + 15) >> 4, nw = G.nt >> 5;
-  oz_encode8<false>(Z, ldz, c0, r0, r1, rinv, B.u, B.eu, G);
-  oz_encode8<true>(M, ld, c0, cb, n, rinv, B.m + cb * kLB, B.em + cb, G);
+  oz_encode8<false, BORDER>(Z, ldz, c0, r0, r1, rinv, ry, B.u, B.eu, G);
+  oz_encode8<true, false>(M, ld, c0, cb, n, rinv, -1, B.m + cb * kLB, B.em + cb, G);
   gsync(G);
-  for (int t = G.tid >> 5; t < nr * nc; t += nw) {
+  int t = G.tid >> 5;
+  if constexpr (BORDER) {
+    if (ry >= r0 && ry < r1) {
+      double* const z = Z + ry * ldz;
+      const int jobs = (n - cb + 31) >> 5;
+      for (; t < jobs; t += nw) {
+        const int c = cb + 32 * t + (G.tid & 31);
+        if (c < n) {
+          double acc = z[c];
+#pragma unroll
+          for (int k = 0; k < kLB; ++k) acc = fma(-z[c0 + k], M[c * ld + c0 + k], acc);
+          z[c] = acc;
+        }
+      }
+      t -= jobs;
+    }
+  }
+  for (; t < nr * nc; t += nw) {
     const int i = t / nc, j = t - i * nc;
-    oz::tile8(Z, ldz, B.u, B.eu, r0, B.m, B.em, 0, r0 + 16 * i, r1, cb + 8 * j, n, Z + c0, ldz, M + c0, ld, G.tid & 31);
+    oz::tile8<BORDER>(Z, ldz, B.u, B.eu, r0, B.m, B.em, 0, r0 + 16 * i, r1, cb + 8 * j, n, Z + c0, ldz, M + c0, ld,
+                      G.tid & 31, ry);
   }
 }
 
@@ -625,10 +681,11 @@ __device__ __forceinline__ void ldl_trail(double* A, const double* M, int ld, in
 // Pivot factorization of A and panel solve Z[r0, r1) <- Z L^{-T} diag(L) by the
 // whole CTA (at least two warps). On return A holds v (strict lower part, L_rc
 // = v_rc / L_cc) and d on its diagonal, M the panel operand L_rc / L_cc, rinv
-// 1 / L_cc and Z the unscaled solution u (x_c = u_c rinv_c). The inputs are
-// complete on entry; ends with a block barrier.
+// 1 / L_cc and Z the unscaled solution u (x_c = u_c rinv_c). BORDER: ry
+// is the bordered row. The inputs are complete on entry; ends with a block barrier.
+template <bool BORDER>
 __device__ void ldl_sweep(double* A, int ld, int n, double* M, double* rinv, int* bad, double* Z, int ldz, int r0,
-                          int r1, const SweepBuf& B) {
+                          int r1, int ry, const SweepBuf& B) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   const Grp W{tid - 32, nt - 32, kBarSweep};
   for (int c0 = 0; c0 < n + kLB; c0 += kLB) {
@@ -651,7 +708,7 @@ __device__ void ldl_sweep(double* A, int ld, int n, double* M, double* rinv, int
       ldl_rows(Z, ldz, r0, r1, M, ld, p0, pn, W);
       if (cn > 0) {
         gsync(W);
-        ldl_panel_update(Z, ldz, n, r0, r1, M, ld, rinv, p0, B, W);
+        ldl_panel_update<BORDER>(Z, ldz, n, r0, r1, M, ld, rinv, p0, ry, B, W);
       }
     }
     __syncthreads();
@@ -675,17 +732,18 @@ __device__ void ldl_panel(double* Z, int ldz, int r0, int r1, const double* M, c
     ldl_rows(Z, ldz, r0, r1, M, ld, c0, min(kLB, n - c0), C);
     __syncthreads();
     if (c0 + kLB < n) {
-      ldl_panel_update(Z, ldz, n, r0, r1, M, ld, rinv, c0, B, C);
+      ldl_panel_update<false>(Z, ldz, n, r0, r1, M, ld, rinv, c0, -1, B, C);
       __syncthreads();
     }
   }
 }
 
-// The solved panel rows [r0, r1): x = u rinv to Pd (row-major, n columns; null
-// ydst: no bordered row, otherwise row ry also to ydst with stride yld), and in
-// digits into Z with the exponents in rowf. Rows [z0, r0) and [r1, z1) of Pd
+// The solved panel rows [r0, r1): x = u rinv to Pd (row-major, n columns), and in
+// digits into Z with the exponents in rowf; BORDER: the bordered row ry as doubles
+// into Z, and to ydst with stride yld. Rows [z0, r0) and [r1, z1) of Pd
 // are zeroed. Eight lanes a row; by the whole group, which synchronizes
 // before and after.
+template <bool BORDER>
 __device__ void panel_out(double* Z, int ldz, int r0, int r1, int n, const double* rinv, int* rowf, double* Pd, int z0,
                           int z1, int ry, double* ydst, long long yld, Grp G) {
   const int sub = G.tid & 7, span = r0 + ((r1 - r0 + 3) & ~3);  // (whole warps: four rows each)
@@ -702,7 +760,7 @@ __device__ void panel_out(double* Z, int ldz, int r0, int r1, int n, const doubl
       }
     }
     for (int o = 4; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
-    const int f = oz::row_exp(em);
+    const int f = BORDER && r == ry ? 0 : oz::row_exp(em);
     if (r < r1) {
       if (sub == 0) rowf[r] = f;
 #pragma unroll
@@ -710,8 +768,12 @@ __device__ void panel_out(double* Z, int ldz, int r0, int r1, int n, const doubl
         const int k = sub + 8 * q;
         if (k < n) {
           Pd[(size_t)r * n + k] = x[q];
-          if (ydst && r == ry) ydst[(size_t)k * yld] = x[q];
-          ((oz::u64*)z)[k] = f == oz::kFp64Row ? oz::dbits(x[q]) : oz::encode(oz::dbits(x[q]), f);
+          if (BORDER && r == ry) {
+            ydst[(size_t)k * yld] = x[q];
+            z[k] = x[q];
+          } else {
+            ((oz::u64*)z)[k] = f == oz::kFp64Row ? oz::dbits(x[q]) : oz::encode(oz::dbits(x[q]), f);
+          }
         }
       }
     }
@@ -1021,6 +1083,7 @@ struct FacCtx {
   static constexpr bool mixed = sizeof(TZ) == 4;
   const LevelDesc* d;
   int n, m, R, ldD, ldZ, ldT, oG, oW, s;
+  int ry;  // panel row of a bordered right-hand side (the last arrow row), -1 without one
   size_t nn, mn;
   SegGeom g;
   double *Dfac, *rinv, *T;
@@ -1034,6 +1097,7 @@ struct FacCtx {
     n = dd.n; m = dd.m; R = 2 * n + m;
     ldD = odd(n); ldZ = lay.ldZ; ldT = lay.ldT;
     oG = n; oW = n + m;  // panel row offsets
+    ry = dd.mr ? oW - 1 : -1;
     g = seg_geom(dd, seg);
     s = g.f - 1;         // separator of this segment (k >= 1)
     nn = (size_t)n * n; mn = (size_t)m * n;
@@ -1279,6 +1343,7 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
 // the E- and G-rows received through distributed shared memory (buffer i % 2);
 // see the roles above. Every element is computed by the same operations
 // whatever the layout.
+template <bool BORDER>
 __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc* __restrict__ descs,
                                                const double* __restrict__ uD, const double* __restrict__ uE,
                                                const double* __restrict__ uG, const double* __restrict__ uR,
@@ -1325,11 +1390,12 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
       const bool eRows = (i < g.len - 1) || g.hasF;
       const int r0 = eRows ? 0 : n;
       if (d.level == 1) cx.prefetch_next(i, j, C);
-      ldl_sweep(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, r0, pr1, SB);
+      ldl_sweep<BORDER>(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, r0, pr1, cx.ry, SB);
       if (threadIdx.x == 0 && bad) { record_breakdown(info, d.sys, d.nat[j], d.level); bad = 0; }
       long long yld = 1;
       double* const yd = cx.y_dst(j, yb, ldyb, yld);
-      panel_out(Z, ldZ, r0, pr1, n, rinv, rowf, d.Lp + (size_t)j * R * n, 0, pair ? n + m : R, oG + m - d.mr, yd, yld, C);
+      double* const Pd = d.Lp + (size_t)j * R * n;
+      panel_out<BORDER>(Z, ldZ, r0, pr1, n, rinv, rowf, Pd, 0, pair ? n + m : R, cx.ry, yd, yld, C);
       __syncthreads();
       if (push) {
         if (i > 0) cluster_wait();  // the consumer is done with stage i-2 (buffer i % 2)
@@ -1351,7 +1417,7 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
         cluster_arrive();
       }
       cx.store_pivot_ldl(j, Dfac, M, rinv, C);
-      oz_syrk(T, ldT, Z, rowf, Z, rowf, 0, ldZ, r0, pr1, r0, n, C);
+      oz_syrk<BORDER>(T, ldT, Z, rowf, Z, rowf, 0, ldZ, r0, pr1, r0, n, cx.ry, Pd, C);
       if (i + 1 < g.len) cx.rotate_cta(i, j, wr, C);
     }
     if (push) cluster_wait();  // phase of the last stage
@@ -1366,9 +1432,10 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
       ldl_panel(Z, ldZ, oW, R, Mbuf(b), rinvbuf(b), ldD, n, SB);
       // (the W-rows' exponents live in buffer 0's array, of which the producer
       // writes the rows below oW only)
-      panel_out(Z, ldZ, oW, R, n, rinvbuf(b), rowf, d.Lp + (size_t)j * R * n, oW, R, -1, nullptr, 1, C);
+      double* const Pd = d.Lp + (size_t)j * R * n;
+      panel_out<false>(Z, ldZ, oW, R, n, rinvbuf(b), rowf, Pd, oW, R, -1, nullptr, 1, C);
       __syncthreads();
-      oz_syrk(T, ldT, Zbuf(b), fbuf(b), Z, rowf, oW, ldZ, oW, R, r0, n, C);
+      oz_syrk<BORDER>(T, ldT, Zbuf(b), fbuf(b), Z, rowf, oW, ldZ, oW, R, r0, n, cx.ry, Pd, C);
       if (i + 1 < g.len) {
         copy_blk(Z + oW * ldZ, ldZ, T + oW * ldT, ldT, n, n, C);  // W_{i+1}
         gsync(C);
@@ -1422,9 +1489,11 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
   // backward sweep of the top level's stages (Algorithm 3, sequential phase)
   // here instead of in a launch of their own; the blocks it reads were
   // written by this CTA, and the shared memory is free by now
-  if (top_solve && d.is_top && d.mr && yb && eg) {
-    __syncthreads();
-    forward_task<double>(tk, descs, yb, ldyb, 1, nullptr, smraw, C, 1);
+  if constexpr (BORDER) {
+    if (top_solve && d.is_top && d.mr && yb && eg) {
+      __syncthreads();
+      forward_task<double>(tk, descs, yb, ldyb, 1, nullptr, smraw, C, 1);
+    }
   }
   if (pair) {
     // a segment without fill-in leaves its consumer idle; every CTA of the
@@ -1435,6 +1504,8 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
 }
 
 // Two CTAs of 256 threads per SM: up to 128 registers (the products' fragments).
+// BORDER: bordered descriptors (kkt_factor_solve); the others carry none of that code.
+template <bool BORDER>
 __global__ void __launch_bounds__(kFactorThreads, 2) k_factor_fp64(const LevelDesc* __restrict__ descs,
                                                                  const Task* __restrict__ tasks,
                                                                  const double* __restrict__ uD,
@@ -1444,7 +1515,7 @@ __global__ void __launch_bounds__(kFactorThreads, 2) k_factor_fp64(const LevelDe
                                                                  double* yb, int ldyb, int top_solve) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int bad;
-  factor_task_fp64(tasks[pair ? blockIdx.x >> 1 : blockIdx.x], descs, uD, uE, uG, uR, info, pair, yb, ldyb, top_solve,
+  factor_task_fp64<BORDER>(tasks[pair ? blockIdx.x >> 1 : blockIdx.x], descs, uD, uE, uG, uR, info, pair, yb, ldyb, top_solve,
                    smraw, bad);
 }
 
@@ -1710,6 +1781,7 @@ __global__ void __launch_bounds__(kFactorThreads, MINB) k_factor(const LevelDesc
 // computed by the same operations in the same order as in the one- and
 // two-CTA layouts, so the results are bitwise theirs.
 // ---------------------------------------------------------------------------
+template <bool BORDER>
 __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __restrict__ descs,
                                           const double* __restrict__ uD, const double* __restrict__ uE,
                                           const double* __restrict__ uG, Info* info, double* yb, int ldyb, int C,
@@ -1803,15 +1875,15 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
     }
   }
   __syncthreads();
-  ldl_sweep(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, t0, t1, sweep_buf(smraw, lay, n));
+  ldl_sweep<BORDER>(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, t0, t1, cx.ry, sweep_buf(smraw, lay, n));
   // its panel rows to device memory (rank 0 also writes the zero rows [0, r0);
   // the bordered row is y_j of the forward substitution), then in digits to the
   // other CTAs
+  double* const Pd = d.Lp + (size_t)j * cx.R * n;
   {
     long long yld = 1;
     double* const yd = cx.y_dst(j, yb, ldyb, yld);
-    panel_out(Z, ldZ, t0, t1, n, rinv, rowf, d.Lp + (size_t)j * cx.R * n, rank == 0 ? 0 : t0, t1, oG + m - d.mr, yd, yld,
-              cta_grp());
+    panel_out<BORDER>(Z, ldZ, t0, t1, n, rinv, rowf, Pd, rank == 0 ? 0 : t0, t1, cx.ry, yd, yld, cta_grp());
   }
   __syncthreads();
   cluster_wait();  // every CTA of the cluster runs
@@ -1833,8 +1905,8 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
     if (tid == 0 && bad) record_breakdown(info, d.sys, d.nat[j], d.level);
     cx.store_pivot_ldl(j, Dfac, M, rinv, cta_grp());
   }
-  cluster_wait();  // every solved panel row is here
-  oz_syrk(T, ldT, Z, rowf, Z, rowf, 0, ldZ, s0, s1, r0, n, cta_grp());
+  cluster_wait();  // every solved panel row is here (and in device memory)
+  oz_syrk<BORDER>(T, ldT, Z, rowf, Z, rowf, 0, ldZ, s0, s1, r0, n, cx.ry, Pd, cta_grp());
   {
     const unsigned a0 = cluster_addr(T, 0u), a1 = cluster_addr(T, 1u);
     const int w0 = s0 - r0;  // row s0 + i holds w0 + i + 1 elements
@@ -1858,6 +1930,7 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
   else if (rank == 1) cx.store_slots(tk.seg, false, g.hasW, cta_grp());
 }
 
+template <bool BORDER>
 __global__ void __launch_bounds__(kFactorThreads, 2) k_factor_clus(const LevelDesc* __restrict__ descs,
                                                                    const Task* __restrict__ tasks,
                                                                    const double* __restrict__ uD,
@@ -1866,7 +1939,7 @@ __global__ void __launch_bounds__(kFactorThreads, 2) k_factor_clus(const LevelDe
                                                                    double* yb, int ldyb, int C) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int bad;
-  clus_task(tasks[blockIdx.x / C], descs, uD, uE, uG, info, yb, ldyb, C, smraw, bad);
+  clus_task<BORDER>(tasks[blockIdx.x / C], descs, uD, uE, uG, info, yb, ldyb, C, smraw, bad);
 }
 
 
@@ -2042,7 +2115,7 @@ __global__ void __launch_bounds__(kFactorThreads, sizeof(TZ) == 8 ? 2 : 3)
     if (ok) {
       if (!w.warp) {
         if constexpr (sizeof(TZ) == 8)
-          factor_task_fp64(tasks[w.first], descs, uD, uE, uG, uR, info, 0, nullptr, 1, 0, smraw, bad);
+          factor_task_fp64<false>(tasks[w.first], descs, uD, uE, uG, uR, info, 0, nullptr, 1, 0, smraw, bad);
         else
           factor_task<TZ, false>(tasks[w.first], descs, uD, uE, uG, uR, info, 0, nullptr, 1, 0, smraw, bad, tslot,
                                  tbar);
@@ -3679,7 +3752,7 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
   const int tcm = tc_mode_for(tc, mixed, pair, maxn, maxm, fill);
   size_t sm = factor_smem_bytes(maxn, maxm, mixed, fill);
   if (top_solve) sm = std::max(sm, solve_smem_bytes(maxn, maxm, 0, fill));
-  const void* fn = !mixed ? (const void*)k_factor_fp64
+  const void* fn = !mixed ? (b ? (const void*)k_factor_fp64<true> : (const void*)k_factor_fp64<false>)
                    : pair ? (const void*)k_factor<float, 1>
                    : tcm  ? (const void*)k_factor<float, 4, true>
                           : (const void*)k_factor<float, 4>;
@@ -3714,7 +3787,9 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
     cfg.numAttrs = 1;
   }
   const int p = pair ? 1 : 0;
-  if (!mixed) return (int)cudaLaunchKernelEx(&cfg, k_factor_fp64, d, t, D, E, G, R, info, p, b, ldb, top_solve);
+  if (!mixed)
+    return b ? (int)cudaLaunchKernelEx(&cfg, k_factor_fp64<true>, d, t, D, E, G, R, info, p, b, ldb, top_solve)
+             : (int)cudaLaunchKernelEx(&cfg, k_factor_fp64<false>, d, t, D, E, G, R, info, p, b, ldb, top_solve);
   return pair ? (int)cudaLaunchKernelEx(&cfg, k_factor<float, 1>, d, t, D, E, G, R, info, p, b, ldb, 0)
          : tcm ? (int)cudaLaunchKernelEx(&cfg, k_factor<float, 4, true>, d, t, D, E, G, R, info, p, b, ldb, tcm)
                : (int)cudaLaunchKernelEx(&cfg, k_factor<float, 4>, d, t, D, E, G, R, info, p, b, ldb, 0);
@@ -3723,9 +3798,9 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
 int factor_clus_size(int ntasks, int maxn, int maxm, int sms) {
   if (ntasks <= 0) return 0;
   const size_t sm = factor_smem_bytes(maxn, maxm, 0, 1);
-  if (set_smem((const void*)k_factor_clus, sm)) return 0;
+  if (set_smem((const void*)k_factor_clus<false>, sm)) return 0;
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_factor_clus, kFactorThreads, sm) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_factor_clus<false>, kFactorThreads, sm) != cudaSuccess ||
       occ < 1)
     return 0;
   occ = std::min(occ, 2);
@@ -3743,7 +3818,7 @@ int factor_clus_size(int ntasks, int maxn, int maxm, int sms) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int ncl = 0;
-    if (cudaOccupancyMaxActiveClusters(&ncl, k_factor_clus, &cfg) == cudaSuccess && ncl >= ntasks) return C;
+    if (cudaOccupancyMaxActiveClusters(&ncl, k_factor_clus<false>, &cfg) == cudaSuccess && ncl >= ntasks) return C;
   }
   return 0;
 }
@@ -3753,7 +3828,7 @@ int launch_factor_clus(const LevelDesc* d, const Task* t, int ntasks, int maxn, 
   if (ntasks <= 0) return 0;
   if (C < 2 || C > 8) return (int)cudaErrorInvalidValue;
   const size_t sm = factor_smem_bytes(maxn, maxm, 0, 1);
-  const int e = set_smem((const void*)k_factor_clus, sm);
+  const int e = set_smem(b ? (const void*)k_factor_clus<true> : (const void*)k_factor_clus<false>, sm);
   if (e) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
@@ -3767,7 +3842,8 @@ int launch_factor_clus(const LevelDesc* d, const Task* t, int ntasks, int maxn, 
   cfg.stream = (cudaStream_t)stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return (int)cudaLaunchKernelEx(&cfg, k_factor_clus, d, t, D, E, G, info, b, ldb, C);
+  return b ? (int)cudaLaunchKernelEx(&cfg, k_factor_clus<true>, d, t, D, E, G, info, b, ldb, C)
+           : (int)cudaLaunchKernelEx(&cfg, k_factor_clus<false>, d, t, D, E, G, info, b, ldb, C);
 }
 
 int launch_forward(const LevelDesc* d, const Task* t, int ntasks, int maxn, int maxm, int single,

@@ -214,10 +214,12 @@ __device__ __noinline__ void element8(double* t, const u64* pa, int fa, const u6
 // columns b0 + 0..7 (< eb), elements b <= a. Lane (g, t) = (lane / 4, lane % 4)
 // holds the fragments' rows a0 + g, a0 + g + 8 and column row b0 + g. The 28
 // digit products per 16 columns of Z are ordered so that neighbouring ones
-// go to different accumulators.
+// go to different accumulators. SKIP: row and column `skip` are left as they are
+// (a row that holds no digits, with any exponent but kFp64Row).
+template <bool SKIP = false>
 __device__ __forceinline__ void tile(double* T, int ldt, const double* Zlo, const int* flo, const double* Z,
                                      const int* fz, int zsplit, int ldz, int a0, int ea, int b0, int eb, int n,
-                                     int lane) {
+                                     int lane, int skip = -1) {
   const int g = lane >> 2, t = lane & 3;
   const int ra = a0 + g, rc = ra + 8, rb = b0 + g;
   const int qa = min(ra, ea - 1), qc = min(rc, ea - 1), qb = min(rb, eb - 1);  // rows for addresses
@@ -227,10 +229,16 @@ __device__ __forceinline__ void tile(double* T, int ldt, const double* Zlo, cons
   const int xa = (qa < zsplit ? flo : fz)[qa], xc = (qc < zsplit ? flo : fz)[qc], xb = (qb < zsplit ? flo : fz)[qb];
   // this lane's outputs: rows ra, rc, columns b0 + 2 t, + 1
   const int c0 = b0 + 2 * t, c1 = c0 + 1;
+  unsigned on = 0;  // (formed here, so that the bounds are not kept through the products)
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
+    if (a < ea && b < eb && b <= a && !(SKIP && (a == skip || b == skip))) on |= 1u << e;
+  }
   if (__any_sync(0xffffffffu, max(max(xa, xc), xb) == kFp64Row)) {
     for (int e = 0; e < 4; ++e) {
       const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
-      if (a < ea && b < eb && b <= a)
+      if (on >> e & 1)
         element(T + a * ldt + b, e < 2 ? za : zc, e < 2 ? xa : xc,
                    (const u64*)((b < zsplit ? Zlo : Z) + b * ldz), (b < zsplit ? flo : fz)[b], n);
     }
@@ -260,7 +268,7 @@ __device__ __forceinline__ void tile(double* T, int ldt, const double* Zlo, cons
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
-    if (a < ea && b < eb && b <= a) {
+    if (on >> e & 1) {
       int p[kDig];
 #pragma unroll
       for (int i = 0; i < kDig; ++i) p[i] = (int)acc[i][e];
@@ -279,19 +287,27 @@ __device__ __forceinline__ void mma_f16_k8(float* d, const uint32_t* a, uint32_t
 // a = a0 + 0..15 (< ea), b = b0 + 0..7 (< eb). U: digit
 // rows of the a (row a at U + (a - ua) 8, exponents eU[a - ua]), V: of the b
 // (V, eV indexed by b - vb). Us, Vs: the rows as doubles (row a at Us + a ldu,
-// row b at Vs + b ldv), for products with a row that is not split.
+// row b at Vs + b ldv), for products with a row that is not split. SKIP: row
+// `skip` of dst is left as it is.
+template <bool SKIP>
 __device__ __forceinline__ void tile8(double* dst, int ldd, const u64* U, const int* eU, int ua,
                                          const u64* V, const int* eV, int vb, int a0, int ea, int b0, int eb,
-                                         const double* Us, int ldu, const double* Vs, int ldv, int lane) {
+                                         const double* Us, int ldu, const double* Vs, int ldv, int lane, int skip) {
   const int g = lane >> 2, t = lane & 3;
   const int ra = a0 + g, rc = ra + 8;
   const int qa = min(ra, ea - 1) - ua, qc = min(rc, ea - 1) - ua, qb = min(b0 + g, eb - 1) - vb;
   const int xa = eU[qa], xc = eU[qc], xb = eV[qb];
   const int c0 = b0 + 2 * t, c1 = c0 + 1;
+  unsigned on = 0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
+    if (a < ea && b < eb && !(SKIP && a == skip)) on |= 1u << e;
+  }
   if (__any_sync(0xffffffffu, max(max(xa, xc), xb) == kFp64Row)) {
     for (int e = 0; e < 4; ++e) {
       const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
-      if (a < ea && b < eb)
+      if (on >> e & 1)
         element8(dst + a * ldd + b, U + (a - ua) * 8, e < 2 ? xa : xc, V + (b - vb) * 8, eV[b - vb], Us + a * ldu,
                  Vs + b * ldv);
     }
@@ -316,7 +332,7 @@ __device__ __forceinline__ void tile8(double* dst, int ldd, const u64* U, const 
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
-    if (a < ea && b < eb) {
+    if (on >> e & 1) {
       int p[kDig];
 #pragma unroll
       for (int i = 0; i < kDig; ++i) p[i] = (int)acc[i][e];

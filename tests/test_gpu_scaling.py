@@ -137,3 +137,82 @@ def test_solutions_of_a_batch(kkt, n, m, persistent):
     x = x.cpu().numpy().reshape(count, -1)
     for i in range(count):
         np.testing.assert_array_equal(x[i] if i % 2 == 0 else S * x[i], x[0], err_msg=f"system {i}")
+
+
+def halves(N, n, m, far, seed=0):
+    """Two systems that nothing couples, their variables (and arrow rows) in turn,
+    the second one's right-hand side smaller by `far`; both solutions' exact
+    values to rounding."""
+    D, E, G, R = system(N, n, m, seed)
+    own = np.arange(n)[:, None] % 2 == np.arange(n) % 2
+    D, E, G = D * own, E * own, G * (np.arange(m)[:, None] % 2 == np.arange(n) % 2)
+    rng = np.random.default_rng([2, N, n, m, seed])
+    second = np.concatenate([np.tile(np.arange(n) % 2 == 1, N), np.arange(m) % 2 == 1])
+    b = rng.normal(size=N * n + m) * np.where(second, far, 1.0)
+    return (D, E, G, R), b, second
+
+
+def check_halves(A, b, second, x, assemble):
+    """Each half within 1e-13 of its own largest entry (the tolerance of the
+    one-system tests: backward errors of a few n 2^-53 at a condition of 3)."""
+    Psi = assemble(*A)
+    for part in (second, ~second):
+        ref = np.linalg.solve(Psi[np.ix_(part, part)], b[part])
+        np.testing.assert_allclose(x[part], ref, rtol=0, atol=1e-13 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("far", [1e-8, 1e-20])
+@pytest.mark.parametrize("N,n,m,levels", [(9, 12, 2, [3, 1]), (7, 17, 0, [1]), (40, 24, 1, [4, 1]), (40, 32, 8, [1]),
+                                          (63, 33, 2, [16, 8, 4, 2, 1]), (63, 48, 14, [16, 8, 4, 2, 1])])
+def test_right_hand_side_without_a_common_scale(kkt, orc, N, n, m, levels, far):
+    """The bordered pass (kkt_factor_solve) carries the right-hand side as a row of
+    the factorization: it has to keep the small half as accurate as the large
+    one, in every layout alike."""
+    A, b, second = halves(N, n, m, far)
+    out = []
+    for pairing in (kkt.KKT_PAIR_OFF, kkt.KKT_PAIR_ON, kkt.KKT_PAIR_AUTO):
+        h = kkt.kkt_create_plan(N, n, m, levels)
+        try:
+            kkt.kkt_set_pairing(h, pairing)
+            x = dev(b)
+            kkt.kkt_factor_solve(h, *args(A, m), x)
+            assert kkt.kkt_get_info(h)["status"] == 0
+            out.append(x.cpu().numpy())
+        finally:
+            kkt.kkt_destroy(h)
+    check_halves(A, b, second, out[0], orc.assemble_dense)
+    for x in out[1:]:
+        np.testing.assert_array_equal(x, out[0])
+
+
+@pytest.mark.parametrize("P", [1, 2])
+@pytest.mark.parametrize("n,m", [(17, 2), (32, 8)])
+def test_right_hand_sides_of_a_batch(kkt, orc, n, m, P):
+    """More systems than the chip holds tasks of 256 threads: as above, and
+    bitwise the result of a handle of its own."""
+    import torch
+    count, N = 4 * torch.cuda.get_device_properties(0).multi_processor_count + 2, 5
+    two = [halves(N, n, m, 1e-12, seed) for seed in (0, 1)]
+    a = [dev(np.concatenate([two[i % 2][0][k].ravel() for i in range(count)])) for k in range(4)]
+    x = dev(np.concatenate([two[i % 2][1] for i in range(count)]))
+    h = kkt.kkt_batch_create([N] * count, [n] * count, [m] * count, [P] * count)
+    try:
+        kkt.kkt_factor_solve(h, *a, x)
+        assert kkt.kkt_get_info(h)["status"] == 0
+    finally:
+        kkt.kkt_destroy(h)
+    x = x.cpu().numpy().reshape(count, -1)
+    for seed, (A, b, second) in enumerate(two):
+        check_halves(A, b, second, x[seed], orc.assemble_dense)
+        for i in range(seed, count, 2):
+            np.testing.assert_array_equal(x[i], x[seed], err_msg=f"system {i}")
+        if P == 1:  # (one system's backward sweep runs in the factor kernel, a batch's in its own)
+            continue
+        h = kkt.kkt_create(N, n, m, P)
+        try:
+            y = dev(b)
+            kkt.kkt_set_pairing(h, kkt.KKT_PAIR_OFF)
+            kkt.kkt_factor_solve(h, *args(A, m), y)
+        finally:
+            kkt.kkt_destroy(h)
+        np.testing.assert_array_equal(x[seed], y.cpu().numpy())
