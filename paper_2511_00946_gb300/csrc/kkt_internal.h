@@ -144,7 +144,7 @@ struct Info {
 // global memory.
 struct FacLayout {
   int q, R, Rs, ldD, ldZ, ldT, oDfac, oM, oRinv, oRinvZ, oZ, oT, oTab, oCorner, total;
-  int oDig, oDex, oF[2];  // cta_layout only
+  int oF[2];  // cta_layout only
 };
 __host__ __device__ inline int kkt_align16(int b) { return (b + 15) & ~15; }
 __host__ __device__ inline FacLayout fac_layout(int n, int m, int zb, bool fill = true) {
@@ -175,9 +175,8 @@ __host__ __device__ inline FacLayout fac_layout_w(int n, int m, int zb, bool fil
   return L;
 }
 // FP64 segment task of a CTA (k_factor_fp64, k_factor_clus): the pivot block,
-// its panel operand M, the panel and T as above; digit blocks of the sweep
-// (kkt_oz.cuh: eight columns of M and of the panel) with their exponents; the
-// exponents of the solved panel rows, two buffers (a pair's consumer alternates).
+// its panel operand M, the panel and T as above; the exponents of the solved
+// panel rows in digits (kkt_oz.cuh), two buffers (a pair's consumer alternates).
 __host__ __device__ inline FacLayout cta_layout(int n, int m, bool fill = true) {
   FacLayout L{};
   L.q = n > m ? n : m;
@@ -193,9 +192,7 @@ __host__ __device__ inline FacLayout cta_layout(int n, int m, bool fill = true) 
   L.oZ = L.oRinvZ + kkt_align16(8 * L.q);
   L.oT = L.oZ + kkt_align16(8 * L.Rs * L.ldZ);
   L.oTab = L.oT + kkt_align16(8 * L.Rs * L.ldT);  // the corner's element table
-  L.oDig = L.oTab + kkt_align16(4 * (m * (m - 1) / 2 + 1));
-  L.oDex = L.oDig + 64 * (n + L.Rs);
-  L.oF[0] = L.oDex + kkt_align16(4 * (n + L.Rs));
+  L.oF[0] = L.oTab + kkt_align16(4 * (m * (m - 1) / 2 + 1));
   L.oF[1] = L.oF[0] + kkt_align16(4 * L.Rs);
   L.oCorner = L.oF[1] + kkt_align16(4 * L.Rs);
   L.total = L.oCorner + kkt_align16(8 * kMaxM * kMaxM);

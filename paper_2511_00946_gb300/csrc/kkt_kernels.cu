@@ -463,10 +463,13 @@ __device__ void oz_syrk(double* T, int ldt, const double* Zlo, const int* flo, c
 // (pivot_rcp), one multiply and one FMA (the lanes keep their own diagonal
 // elements up to date), against six dependent FP64 instructions and a block
 // barrier per column before (1080-1250 cycles a column); 1 / L_cc =
-// 1 / sqrt(d_c) is formed off the chain. The updates of the panel behind a
-// block (u m^T, u the unscaled solution) are tensor-core products of eight
-// columns (oz::tile8); in FP64 FMAs they were most of the sweep's FP64
-// instructions.
+// 1 / sqrt(d_c) is formed off the chain. The panel behind a block (u m^T, u the
+// unscaled solution) is updated by FP64 FMAs, one element per lane. (Digit
+// products of eight columns took the FMAs off the FP64 pipe but stood longer in
+// the sweep: encoding, a barrier and a tile of 28 products for eight columns.
+// Digits against FMAs, us: one system of N = 300, m = 4, n = 26 438, 396, n = 32
+// 485, 453, n = 48 853, 818; 1200 systems of N = 40, n = 26 3396, 2898, n = 32
+// 4274, 4132, n = 48 10703, 10946.)
 // Schedule: warp 0 eliminates block J. Meanwhile the other warps finish block
 // J - 1: the pivot block's columns beyond block J, the panel's block J - 1
 // (one row per thread, or eight lanes per row where the rows are few) and the
@@ -474,18 +477,6 @@ __device__ void oz_syrk(double* T, int ldt, const double* Zlo, const int* flo, c
 // ---------------------------------------------------------------------------
 constexpr int kLB = 8;         // columns per block
 constexpr int kBarSweep = 2;   // barrier of warps 1 and up
-struct SweepBuf {              // digit blocks (kLB per row) and their exponents
-  oz::u64 *m, *u;              // panel operand rows, panel rows
-  int *em, *eu;
-};
-__device__ __forceinline__ SweepBuf sweep_buf(unsigned char* sm, const FacLayout& lay, int n) {
-  SweepBuf b;
-  b.m = (oz::u64*)(sm + lay.oDig);
-  b.u = b.m + kLB * n;
-  b.em = (int*)(sm + lay.oDex);
-  b.eu = b.em + n;
-  return b;
-}
 
 // Warp 0: columns [c0, c0 + cn) of the pivot block A (row-major FP64, updated
 // by the blocks before), rows c0 + lane + 32 q: v and d into A, m into M (same
@@ -606,66 +597,21 @@ __device__ __forceinline__ void ldl_rows(double* Z, int ldz, int r0, int r1, con
   }
 }
 
-// digits of the eight columns [c0, c0 + kLB) of rows [r0, r1) of src (ld) into
-// dst[(r - r0) kLB ..] with exponents ex[r - r0]; eight lanes a row. Column k is
-// scaled by 2^s_k (oz::balance of rinv) for the panel rows, 2^-s_k (NEG) for
-// the operand rows: u and m carry L_kk and 1 / L_kk, so without it a row's
-// exponent would be set by a column of another unit than the one that sets
-// its partner's, and the products of the others would lose the ratio of the
-// pivots' roots (one system of N = 50, n = 48, variables in units within 10^+-6:
-// 5e-9 off its solution in equal units, 10^+-9: 3e-3; with the scaling no bit
-// differs). With it the operands are the rows of x and L to a factor of two.
-// Rows that are not split and, BORDER, row ry are not stored (their products read src).
-template <bool NEG, bool BORDER>
-__device__ __forceinline__ void oz_encode8(const double* src, int ld, int c0, int r0, int r1, const double* rinv,
-                                           int ry, oz::u64* dst, int* ex, Grp G) {
-  const int sub = G.tid & 7, cnt = (r1 - r0 + 3) & ~3;  // (whole warps: four rows each)
-  const int sc = NEG ? -oz::balance(rinv[c0 + sub]) : oz::balance(rinv[c0 + sub]);
-  for (int r = G.tid >> 3; r < cnt; r += G.nt >> 3) {
-    const int rr = min(r0 + r, r1 - 1);
-    const oz::u64 b = oz::dbits(src[rr * ld + c0 + sub]);
-    int key = oz::scaled_key(b, sc);
-    for (int o = 4; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-    const int f = BORDER && rr == ry ? 0 : oz::scaled_row_exp(key);
-    if (r0 + r < r1) {
-      if (!(BORDER && rr == ry)) dst[r * kLB + sub] = oz::encode(b, f - sc);  // (not read where f is kFp64Row)
-      if (sub == 0) ex[r] = f;
-    }
-  }
-}
-
 // Panel rows [r0, r1) behind the solved block [c0, c0 + kLB): Z[r][c] -= u_r
-// m_c^T for c >= c0 + kLB; by group G, which synchronizes before (u, and rinv of
-// the block) and after. BORDER: row ry (a bordered right-hand side, see oz_syrk)
-// in FP64 FMAs, a column per lane, beside the tiles.
-template <bool BORDER>
+// m_c^T for c >= c0 + kLB, in column order; by group G, which synchronizes before
+// (u) and after.
 __device__ __forceinline__ void ldl_panel_update(double* Z, int ldz, int n, int r0, int r1, const double* M, int ld,
-                                                 const double* rinv, int c0, int ry, const SweepBuf& B, Grp G) {
-  const int cb = c0 + kLB, nc = (n - cb + 7) >> 3, nr = (r1 - r0 + 15) >> 4, nw = G.nt >> 5;
-  oz_encode8<false, BORDER>(Z, ldz, c0, r0, r1, rinv, ry, B.u, B.eu, G);
-  oz_encode8<true, false>(M, ld, c0, cb, n, rinv, -1, B.m + cb * kLB, B.em + cb, G);
-  gsync(G);
-  int t = G.tid >> 5;
-  if constexpr (BORDER) {
-    if (ry >= r0 && ry < r1) {
-      double* const z = Z + ry * ldz;
-      const int jobs = (n - cb + 31) >> 5;
-      for (; t < jobs; t += nw) {
-        const int c = cb + 32 * t + (G.tid & 31);
-        if (c < n) {
-          double acc = z[c];
+                                                 int c0, Grp G) {
+  const int cb = c0 + kLB, w = n - cb;
+  const Div by(w);
+  for (int e = G.tid; e < (r1 - r0) * w; e += G.nt) {
+    const int q = by(e), c = cb + e - q * w;
+    double* const z = Z + (r0 + q) * ldz;
+    const double* const mc = M + c * ld + c0;
+    double x = z[c];
 #pragma unroll
-          for (int k = 0; k < kLB; ++k) acc = fma(-z[c0 + k], M[c * ld + c0 + k], acc);
-          z[c] = acc;
-        }
-      }
-      t -= jobs;
-    }
-  }
-  for (; t < nr * nc; t += nw) {
-    const int i = t / nc, j = t - i * nc;
-    oz::tile8<BORDER>(Z, ldz, B.u, B.eu, r0, B.m, B.em, 0, r0 + 16 * i, r1, cb + 8 * j, n, Z + c0, ldz, M + c0, ld,
-                      G.tid & 31, ry);
+    for (int k = 0; k < kLB; ++k) x = fma(-z[c0 + k], mc[k], x);
+    z[c] = x;
   }
 }
 
@@ -681,11 +627,10 @@ __device__ __forceinline__ void ldl_trail(double* A, const double* M, int ld, in
 // Pivot factorization of A and panel solve Z[r0, r1) <- Z L^{-T} diag(L) by the
 // whole CTA (at least two warps). On return A holds v (strict lower part, L_rc
 // = v_rc / L_cc) and d on its diagonal, M the panel operand L_rc / L_cc, rinv
-// 1 / L_cc and Z the unscaled solution u (x_c = u_c rinv_c). BORDER: ry
-// is the bordered row. The inputs are complete on entry; ends with a block barrier.
-template <bool BORDER>
+// 1 / L_cc and Z the unscaled solution u (x_c = u_c rinv_c). The inputs are
+// complete on entry; ends with a block barrier.
 __device__ void ldl_sweep(double* A, int ld, int n, double* M, double* rinv, int* bad, double* Z, int ldz, int r0,
-                          int r1, int ry, const SweepBuf& B) {
+                          int r1) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   const Grp W{tid - 32, nt - 32, kBarSweep};
   for (int c0 = 0; c0 < n + kLB; c0 += kLB) {
@@ -708,7 +653,7 @@ __device__ void ldl_sweep(double* A, int ld, int n, double* M, double* rinv, int
       ldl_rows(Z, ldz, r0, r1, M, ld, p0, pn, W);
       if (cn > 0) {
         gsync(W);
-        ldl_panel_update<BORDER>(Z, ldz, n, r0, r1, M, ld, rinv, p0, ry, B, W);
+        ldl_panel_update(Z, ldz, n, r0, r1, M, ld, p0, W);
       }
     }
     __syncthreads();
@@ -723,16 +668,15 @@ __device__ void ldl_sweep(double* A, int ld, int n, double* M, double* rinv, int
   }
 }
 
-// Panel rows [r0, r1) against a pivot block received as M and rinv: the
-// operations of ldl_sweep (u, unscaled). By the whole CTA; ends with a block barrier.
-__device__ void ldl_panel(double* Z, int ldz, int r0, int r1, const double* M, const double* rinv, int ld, int n,
-                          const SweepBuf& B) {
+// Panel rows [r0, r1) against a pivot block received as M: the operations of
+// ldl_sweep (u, unscaled). By the whole CTA; ends with a block barrier.
+__device__ void ldl_panel(double* Z, int ldz, int r0, int r1, const double* M, int ld, int n) {
   const Grp C = cta_grp();
   for (int c0 = 0; c0 < n; c0 += kLB) {
     ldl_rows(Z, ldz, r0, r1, M, ld, c0, min(kLB, n - c0), C);
     __syncthreads();
     if (c0 + kLB < n) {
-      ldl_panel_update<false>(Z, ldz, n, r0, r1, M, ld, rinv, c0, -1, B, C);
+      ldl_panel_update(Z, ldz, n, r0, r1, M, ld, c0, C);
       __syncthreads();
     }
   }
@@ -1368,7 +1312,6 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
   auto Zbuf = [&](int b) { return b ? T : Z; };
   auto fbuf = [&](int b) { return (int*)(smraw + lay.oF[b]); };  // exponents of the solved rows
   int* const rowf = fbuf(0);
-  const SweepBuf SB = sweep_buf(smraw, lay, n);
   const bool eg = !pair || rank == 0;             // this CTA holds the E/G rows
   const bool wr = g.hasW && (!pair || rank == 1);  // this CTA holds the W rows
   const Grp C = cta_grp();
@@ -1390,7 +1333,7 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
       const bool eRows = (i < g.len - 1) || g.hasF;
       const int r0 = eRows ? 0 : n;
       if (d.level == 1) cx.prefetch_next(i, j, C);
-      ldl_sweep<BORDER>(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, r0, pr1, cx.ry, SB);
+      ldl_sweep(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, r0, pr1);
       if (threadIdx.x == 0 && bad) { record_breakdown(info, d.sys, d.nat[j], d.level); bad = 0; }
       long long yld = 1;
       double* const yd = cx.y_dst(j, yb, ldyb, yld);
@@ -1429,7 +1372,7 @@ __device__ __forceinline__ void factor_task_fp64(const Task tk, const LevelDesc*
       const int r0 = eRows ? 0 : n, b = i & 1;
       cluster_arrive();  // done with stage i-1
       cluster_wait();    // stage i's blocks are in buffer b
-      ldl_panel(Z, ldZ, oW, R, Mbuf(b), rinvbuf(b), ldD, n, SB);
+      ldl_panel(Z, ldZ, oW, R, Mbuf(b), ldD, n);
       // (the W-rows' exponents live in buffer 0's array, of which the producer
       // writes the rows below oW only)
       double* const Pd = d.Lp + (size_t)j * R * n;
@@ -1875,7 +1818,7 @@ __device__ __forceinline__ void clus_task(const Task tk, const LevelDesc* __rest
     }
   }
   __syncthreads();
-  ldl_sweep<BORDER>(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, t0, t1, cx.ry, sweep_buf(smraw, lay, n));
+  ldl_sweep(Dfac, ldD, n, M, rinv, &bad, Z, ldZ, t0, t1);
   // its panel rows to device memory (rank 0 also writes the zero rows [0, r0);
   // the bordered row is y_j of the forward substitution), then in digits to the
   // other CTAs

@@ -94,25 +94,6 @@ KKT_OZ int row_exp(int m) {
   return f > kExpMax || (f < kExpMin && m != 0) ? kFp64Row : f;  // (infinities and NaN included)
 }
 
-// As mag() and row_exp() for elements scaled by powers of two of their own: the
-// biased exponent of v 2^s (kZeroKey: a zero; infinities, NaN and subnormals
-// keep their row in FP64) and the row exponent from the largest one. The
-// digits of v 2^s at exponent f are encode(v, f - s).
-constexpr int kZeroKey = -(1 << 20);
-KKT_OZ int scaled_key(u64 b, int s) {
-  const int ef = expo(b);
-  return ef == 0 ? ((b << 1) == 0 ? kZeroKey : kFp64Row) : ef == 0x7ff ? kFp64Row : ef + s;
-}
-KKT_OZ int scaled_row_exp(int key) {
-  const int f = key - 1022;
-  return key == kZeroKey ? -1022 : f > kExpMax || f < kExpMin ? kFp64Row : f;
-}
-
-// The power of two that brings a column of the panel update u m^T back to the
-// scale of its rows: u_rk = x_rk L_kk and m_ck = L_ck / L_kk are split as
-// u_rk 2^s and m_ck 2^-s with 2^s <= 1 / L_kk < 2^(s + 1).
-KKT_OZ int balance(double rinv) { return expo(dbits(rinv)) - 1023; }
-
 // digits of z at exponent f (|z| < 2^f), 256 added to each
 KKT_OZ u64 encode(u64 b, int f) {
   const int ef = expo(b), q = f + 1022 - ef;  // q >= 0
@@ -198,18 +179,6 @@ __device__ __noinline__ void element(double* t, const u64* pa, int fa, const u64
   *t = acc;
 }
 
-// the same over eight columns of a panel update, the doubles beside the digits
-__device__ __noinline__ void element8(double* t, const u64* pa, int fa, const u64* pb, int fb, const double* ua,
-                                      const double* vb) {
-  if (fa == kFp64Row || fb == kFp64Row) {
-    double acc = *t;
-    for (int k = 0; k < 8; ++k) acc = fma(-ua[k], vb[k], acc);
-    *t = acc;
-  } else {
-    element(t, pa, fa, pb, fb, 8);
-  }
-}
-
 // One 16 x 8 tile of T -= Z Z^T by a warp: rows a0 + 0..15 (< ea) against
 // columns b0 + 0..7 (< eb), elements b <= a. Lane (g, t) = (lane / 4, lane % 4)
 // holds the fragments' rows a0 + g, a0 + g + 8 and column row b0 + g. The 28
@@ -273,70 +242,6 @@ __device__ __forceinline__ void tile(double* T, int ldt, const double* Zlo, cons
 #pragma unroll
       for (int i = 0; i < kDig; ++i) p[i] = (int)acc[i][e];
       T[a * ldt + b] -= to_double(combine(p), (e < 2 ? xa : xc) + (e & 1 ? x1 : x0) + kUnit);
-    }
-  }
-}
-
-__device__ __forceinline__ void mma_f16_k8(float* d, const uint32_t* a, uint32_t b) {
-  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
-               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-               : "r"(a[0]), "r"(a[1]), "r"(b));
-}
-
-// One 16 x 8 tile of dst -= U V^T over eight columns by a warp: dst[a][b] for
-// a = a0 + 0..15 (< ea), b = b0 + 0..7 (< eb). U: digit
-// rows of the a (row a at U + (a - ua) 8, exponents eU[a - ua]), V: of the b
-// (V, eV indexed by b - vb). Us, Vs: the rows as doubles (row a at Us + a ldu,
-// row b at Vs + b ldv), for products with a row that is not split. SKIP: row
-// `skip` of dst is left as it is.
-template <bool SKIP>
-__device__ __forceinline__ void tile8(double* dst, int ldd, const u64* U, const int* eU, int ua,
-                                         const u64* V, const int* eV, int vb, int a0, int ea, int b0, int eb,
-                                         const double* Us, int ldu, const double* Vs, int ldv, int lane, int skip) {
-  const int g = lane >> 2, t = lane & 3;
-  const int ra = a0 + g, rc = ra + 8;
-  const int qa = min(ra, ea - 1) - ua, qc = min(rc, ea - 1) - ua, qb = min(b0 + g, eb - 1) - vb;
-  const int xa = eU[qa], xc = eU[qc], xb = eV[qb];
-  const int c0 = b0 + 2 * t, c1 = c0 + 1;
-  unsigned on = 0;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
-    if (a < ea && b < eb && !(SKIP && a == skip)) on |= 1u << e;
-  }
-  if (__any_sync(0xffffffffu, max(max(xa, xc), xb) == kFp64Row)) {
-    for (int e = 0; e < 4; ++e) {
-      const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
-      if (on >> e & 1)
-        element8(dst + a * ldd + b, U + (a - ua) * 8, e < 2 ? xa : xc, V + (b - vb) * 8, eV[b - vb], Us + a * ldu,
-                 Vs + b * ldv);
-    }
-    return;
-  }
-  float acc[kDig][4];
-#pragma unroll
-  for (int i = 0; i < kDig; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
-  {
-    const ulonglong2 pa = *(const ulonglong2*)(U + qa * 8 + 2 * t), pc = *(const ulonglong2*)(U + qc * 8 + 2 * t),
-                     pb = *(const ulonglong2*)(V + qb * 8 + 2 * t);
-    const u64 u[4] = {pa.x, pa.y, pc.x, pc.y}, v[2] = {pb.x, pb.y};
-    uint32_t A[kDig][2], B[kDig][1];
-    Split<0>::run<2>(A, u);
-    Split<0>::run<1>(B, v);
-#pragma unroll
-    for (int i = 0; i < kDig; ++i)
-#pragma unroll
-      for (int j = kDig - 1; j >= kLow - i; --j) mma_f16_k8(acc[i + j - kLow], A[i], B[j][0]);
-  }
-  const int x0 = __shfl_sync(0xffffffffu, xb, 8 * t), x1 = __shfl_sync(0xffffffffu, xb, 8 * t + 4);
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const int a = e < 2 ? ra : rc, b = e & 1 ? c1 : c0;
-    if (on >> e & 1) {
-      int p[kDig];
-#pragma unroll
-      for (int i = 0; i < kDig; ++i) p[i] = (int)acc[i][e];
-      dst[a * ldd + b] -= to_double(combine(p), (e < 2 ? xa : xc) + (e & 1 ? x1 : x0) + kUnit);
     }
   }
 }
