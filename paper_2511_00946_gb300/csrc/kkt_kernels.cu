@@ -395,8 +395,18 @@ __device__ void syrk_trap(double* T, int ldt, const TZ* Zlo, const TZ* Z, int zs
 // FP64 Schur products on the tensor cores (kkt_oz.cuh).
 // ---------------------------------------------------------------------------
 
+// Smallest block whose Schur products take digits; smaller ones take FP64 FMAs
+// (syrk_trap) and keep their doubles. A tile costs the same 28 products per 16
+// columns however few rows and columns are left, so small panels are faster in
+// FMAs, most of all where a task has its SM to itself. Digits against FMAs, us:
+// one system of N = 300, m = 4 in one pass, n = 17 309, 289, n = 19 321, 314, n = 20
+// 328, 323, n = 22 344, 338; 160 systems of four segments, N = 40, n = 17 542, 586,
+// n = 19 577, 705, n = 20 600, 745. One line for every layout, whose results agree
+// bit for bit.
+constexpr int kDigMin = 20;
+
 // T[a][b] -= sum_t Z[a][t] Z[b][t] for ra0 <= a < ra1, cb0 <= b <= a (cb0 <=
-// ra0), rows in digits (panel_out). Panel rows below `zsplit` are read from
+// ra0), rows in digits (panel_out; n < kDigMin: doubles). Panel rows below `zsplit` are read from
 // (Zlo, flo), the others from (Z, fz). One 16 x 8 tile per warp at a time.
 // Every element is one sum rounded once, so the result does not depend on the
 // tiling.
@@ -411,6 +421,10 @@ __device__ void syrk_trap(double* T, int ldt, const TZ* Zlo, const TZ* Z, int zs
 template <bool BORDER>
 __device__ void oz_syrk(double* T, int ldt, const double* Zlo, const int* flo, const double* Z, const int* fz,
                         int zsplit, int ldz, int ra0, int ra1, int cb0, int n, int ry, const double* Pd, Grp G) {
+  if (n < kDigMin) {
+    syrk_trap(T, ldt, Zlo, Z, zsplit, ldz, ra0, ra1, cb0, n, G);
+    return;
+  }
   const int lane = G.tid & 31, nw = G.nt >> 5, w0 = ra0 - cb0;
   int i = 0, j = G.tid >> 5;
   if constexpr (BORDER) {
@@ -683,7 +697,7 @@ __device__ void ldl_panel(double* Z, int ldz, int r0, int r1, const double* M, i
 }
 
 // The solved panel rows [r0, r1): x = u rinv to Pd (row-major, n columns), and in
-// digits into Z with the exponents in rowf; BORDER: the bordered row ry as doubles
+// digits (n >= kDigMin) into Z with the exponents in rowf; BORDER: the bordered row ry as doubles
 // into Z, and to ydst with stride yld. Rows [z0, r0) and [r1, z1) of Pd
 // are zeroed. Eight lanes a row; by the whole group, which synchronizes
 // before and after.
@@ -704,7 +718,7 @@ __device__ void panel_out(double* Z, int ldz, int r0, int r1, int n, const doubl
       }
     }
     for (int o = 4; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
-    const int f = BORDER && r == ry ? 0 : oz::row_exp(em);
+    const int f = n < kDigMin ? oz::kFp64Row : BORDER && r == ry ? 0 : oz::row_exp(em);
     if (r < r1) {
       if (sub == 0) rowf[r] = f;
 #pragma unroll
@@ -712,12 +726,9 @@ __device__ void panel_out(double* Z, int ldz, int r0, int r1, int n, const doubl
         const int k = sub + 8 * q;
         if (k < n) {
           Pd[(size_t)r * n + k] = x[q];
-          if (BORDER && r == ry) {
-            ydst[(size_t)k * yld] = x[q];
-            z[k] = x[q];
-          } else {
-            ((oz::u64*)z)[k] = f == oz::kFp64Row ? oz::dbits(x[q]) : oz::encode(oz::dbits(x[q]), f);
-          }
+          if (BORDER && r == ry) ydst[(size_t)k * yld] = x[q];
+          if (f == oz::kFp64Row || (BORDER && r == ry)) z[k] = x[q];
+          else ((oz::u64*)z)[k] = oz::encode(oz::dbits(x[q]), f);
         }
       }
     }
