@@ -507,7 +507,7 @@ kkt_status kkt_plan_flops(int N, int n, int m, int nlevels, const int* P_levels,
  * allocator, a plugin whose host framework owns every allocation, or a
  * process whose memory pool is exhausted). Same method as
  * kkt_create(N, n, m, P, KKT_FP64) followed by kkt_factor and kkt_solve,
- * with the same results.
+ * with the same results up to rounding.
  *  - D, E, G, R, b: device pointers as for kkt_factor / kkt_solve; b is
  *    overwritten with the solution. `info`: optional device pointer to 4
  *    ints that receive the kkt_info record of a breakdown (zeroed first by

@@ -499,8 +499,11 @@ constexpr int kBarSweep = 2;   // barrier of warps 1 and up
 // pivot is one shuffle, one reciprocal and one FMA. FULL: cn = kLB. Without SAFE
 // the code has no branch inside (the updates fill the reciprocal's latency:
 // 4.3k cycles a block against 5.5k) and returns false, with nothing written to A,
-// where a pivot fails pivot_rcp_ok; SAFE divides, forms no square and takes any
-// pivot, *bad is then the first column + 1 that is not positive.
+// where a pivot fails pivot_rcp_ok; SAFE forms no square, divides by the pivots
+// that fail it and takes any, *bad is then the first column + 1 that is not
+// positive. Blocks that a handle runs one warp per task (potrf_w) take SAFE at
+// once: its operations are potrf_w's, and kkt_solve_noalloc then agrees with a
+// handle on systems so ill-conditioned that no other rounding would.
 template <int SL, bool FULL, bool SAFE>
 __device__ __forceinline__ bool ldl_block_t(double* A, double* M, int ld, int n, int c0, int cn, int* bad, int lane) {
   double v[SL][kLB];
@@ -522,7 +525,10 @@ __device__ __forceinline__ bool ldl_block_t(double* A, double* M, int ld, int n,
       if (SAFE) {
         if (not_positive(d) && first == 0) first = c0 + c + 1;
 #pragma unroll
-        for (int q = 0; q < SL; ++q) m[q] = not_positive(d) ? __longlong_as_double(0x7ff8000000000000LL) : v[q][c] / d;
+        for (int q = 0; q < SL; ++q)
+          m[q] = pivot_rcp_ok(d)   ? v[q][c] * pivot_rcp(d)
+                 : not_positive(d) ? __longlong_as_double(0x7ff8000000000000LL)
+                                   : v[q][c] / d;
         dn = fma(-v[0][c], m[0], dg);
       } else {
         ok = ok && pivot_rcp_ok(d);
@@ -561,14 +567,19 @@ __device__ __forceinline__ bool ldl_block_t(double* A, double* M, int ld, int n,
   if (SAFE && lane == 0 && first && *bad == 0) *bad = first;
   return true;
 }
+template <int SL>
 __device__ __noinline__ void ldl_block_safe(double* A, double* M, int ld, int n, int c0, int cn, int* bad, int lane) {
-  ldl_block_t<2, false, true>(A, M, ld, n, c0, cn, bad, lane);
+  ldl_block_t<SL, false, true>(A, M, ld, n, c0, cn, bad, lane);
 }
 __device__ __forceinline__ void ldl_block(double* A, double* M, int ld, int n, int c0, int cn, int* bad, int lane) {
+  if (n <= kWarpMaxN) {
+    ldl_block_safe<1>(A, M, ld, n, c0, cn, bad, lane);
+    return;
+  }
   const bool done = cn < kLB      ? ldl_block_t<1, false, false>(A, M, ld, n, c0, cn, bad, lane)
                     : n - c0 > 32 ? ldl_block_t<2, true, false>(A, M, ld, n, c0, cn, bad, lane)
                                   : ldl_block_t<1, true, false>(A, M, ld, n, c0, cn, bad, lane);
-  if (!done) ldl_block_safe(A, M, ld, n, c0, cn, bad, lane);
+  if (!done) ldl_block_safe<2>(A, M, ld, n, c0, cn, bad, lane);
 }
 
 // Columns [c0, c0 + cn) of the panel rows [r0, r1): u_i = z_i - sum_{c < i} u_c

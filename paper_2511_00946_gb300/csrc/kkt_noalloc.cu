@@ -177,10 +177,15 @@ extern "C" kkt_status kkt_solve_noalloc(int N, int n, int m, int P, const double
 
   const kkt::LevelDesc* ddesc = (const kkt::LevelDesc*)(base + oDesc);
   const kkt::Task* dtask = (const kkt::Task*)(base + oTask);
-  // (small blocks one warp per task, as the handle path: the same arithmetic)
+  // Blocks up to n = 5 one warp per task, larger ones a CTA: the call has few tasks,
+  // so a task's own time counts, and from n = 6 on eight warps beat one at any
+  // number of them. One warp against a CTA, us (m = 4): N = 24, P = 4, n = 4 146, 145,
+  // n = 6 175, 163, n = 12 293, 203, n = 16 415, 233; N = 600, P = 120, n = 4 1119,
+  // 1322, n = 5 1237, 1137 (m = 0: 1048, 1376), n = 6 1431, 1242, n = 16 4073, 1954.
+  constexpr int kWarpTaskN = 5;
   auto factor = [&](const kkt::Task* t, int cnt) {
-    return n <= kkt::kWarpMaxN ? kkt::launch_factor_w(ddesc, t, cnt, n, m, 0, D, E, G, R, dinfo, stream)
-                               : kkt::launch_factor(ddesc, t, cnt, n, m, 0, 0, D, E, G, R, dinfo, stream);
+    return n <= kWarpTaskN ? kkt::launch_factor_w(ddesc, t, cnt, n, m, 0, D, E, G, R, dinfo, stream)
+                           : kkt::launch_factor(ddesc, t, cnt, n, m, 0, 0, D, E, G, R, dinfo, stream);
   };
   if (factor(dtask, P) || (two && factor(dtask + P, 1))) return KKT_ERR_CUDA;
   for (int c0 = 0; c0 < nrhs; c0 += kkt::kRhsChunk) {
