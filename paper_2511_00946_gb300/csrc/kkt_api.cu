@@ -234,7 +234,7 @@ struct kkt_handle {
   kkt::PCons* pcons = nullptr;
   Task* ptasks = nullptr;
   int* pready = nullptr;        // [pn] counters, then the ticket
-  int pn = 0, pgrid = 0, pslice = 0, pmixed = 0, punmet = 0;
+  int pn = 0, pgrid = 0, pthreads = 0, pslice = 0, pmixed = 0, punmet = 0;
   size_t psmem = 0;
   long long pwait = 1LL << 31;  // clock cycles a dependency wait may take (about a second)
   std::vector<kkt::PItem> hpitems;
@@ -966,9 +966,27 @@ kkt_status build_persistent(kkt_handle* h) {
     }
   }
   const int slice = any_w ? (int)kkt::factor_w_slice_bytes(wn, wm, mixed, wfill) : 0;
-  const int wpc = any_w ? std::max(1, std::min(8, (200 * 1024) / slice)) : 8;
-  const size_t smem = std::max(any_cta ? kkt::factor_smem_bytes(cn, cm, mixed, cfill) : 0, (size_t)wpc * slice);
-  const int best_occ = kkt::persist_occupancy(mixed, smem);
+  int threads = kkt::kFactorThreads, wpc = 8;
+  size_t smem = 0;
+  auto occupancy = [&](int nthreads) {
+    threads = nthreads;
+    wpc = any_w ? std::max(1, std::min(threads / 32, (200 * 1024) / slice)) : threads / 32;
+    smem = std::max(any_cta ? kkt::factor_smem_bytes(cn, cm, mixed, cfill) : 0, (size_t)wpc * slice);
+    return kkt::persist_occupancy(mixed, smem, threads);
+  };
+  int best_occ = occupancy(kkt::kFactorThreads);
+  if (!mixed && any_cta) {
+    // half as many threads where twice as many tasks then share an SM and there
+    // are more of them than CTAs of 256 threads, as launch_factor (1200 systems of
+    // N = 40, m = 4, us with 256 and 128 threads: n = 17 2347, 1625, n = 20 2749,
+    // 2000, n = 32 5025, 4008)
+    long long ncta = 0;
+    for (const SysPlan& sp : h->sys)
+      if (sp.n > kkt::kWarpMaxN) ncta += sp.lv[0].P;
+    const int occ = best_occ;
+    if (ncta > (long long)occ * sms && (best_occ = occupancy(kkt::kFactorThreads / 2)) < 2 * occ)
+      best_occ = occupancy(kkt::kFactorThreads);
+  }
   if (best_occ < 1) return KKT_ERR_ARG;
   // items
   struct Cand { double cost; std::vector<std::pair<int, int>> tasks; bool warp; };
@@ -1068,6 +1086,7 @@ kkt_status build_persistent(kkt_handle* h) {
   h->pgrid = (int)std::min<long long>((long long)n_it, (long long)best_occ * sms);
   h->psmem = smem;
   h->pslice = slice;
+  h->pthreads = threads;
   h->pmixed = mixed;
   h->punmet = 0;
   return KKT_OK;
@@ -1152,7 +1171,7 @@ kkt_status kkt_factor(kkt_handle* h, const double* D, const double* E, const dou
   if (h->persistent) {
     if (cudaMemsetAsync(h->pready, 0, sizeof(int) * (h->pn + 1), (cudaStream_t)stream) != cudaSuccess ||
         kkt::launch_factor_persist(h->ddesc, h->ptasks, h->pitems, h->pn, h->pcons, h->pready, h->pmixed, D, E, G, R,
-                                   h->dinfo, h->pgrid, h->psmem, h->pslice, h->pwait, stream) ||
+                                   h->dinfo, h->pgrid, h->pthreads, h->psmem, h->pslice, h->pwait, stream) ||
         !mark(h, 0, stream))
       return KKT_ERR_CUDA;
     h->factored = true;

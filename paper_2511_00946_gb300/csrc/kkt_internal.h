@@ -385,19 +385,21 @@ int launch_adjoint_grad(const LevelDesc* d, const ResTask* t, int ntasks, const 
 int launch_fill_identity(const LevelDesc* d, const int* sys_desc, int count, double* D, double* R,
                          void* stream);
 // Persistent factorization of a handle whose levels share one precision:
-// items [0, nitems) over `grid` CTAs with `smem` bytes of shared memory;
+// items [0, nitems) over `grid` CTAs of `threads` threads (kFactorThreads; FP64
+// also half as many, with at most four warp tasks an item) with `smem` bytes of
+// shared memory;
 // ready[0..nitems) and the ticket counter ready[nitems] must be zero; a
 // dependency wait gives up after wait_cycles clock cycles (KKT_ERR_TIMEOUT).
 // `slice`: shared memory of one warp task.
 int launch_factor_persist(const LevelDesc* d, const Task* t, const PItem* items, int nitems, const PCons* cons,
                           int* ready, int mixed, const double* D, const double* E, const double* G,
-                          const double* R, Info* info, int grid, size_t smem, int slice,
+                          const double* R, Info* info, int grid, int threads, size_t smem, int slice,
                           long long wait_cycles, void* stream);
 // the debug build's index-check record (status 8 on a failed check; zero in
 // the normal build); `clear` resets it
 int debug_info(Info* out, int clear);
 // occupancy (CTAs per SM) of the persistent kernel with `smem` bytes
-int persist_occupancy(int mixed, size_t smem);
+int persist_occupancy(int mixed, size_t smem, int threads);
 size_t factor_smem_bytes(int maxn, int maxm, int mixed, int fill = 1);
 size_t factor_w_slice_bytes(int maxn, int maxm, int mixed, int fill = 1);
 size_t solve_smem_bytes(int maxn, int maxm, int single, int fill = 1);

@@ -3646,17 +3646,17 @@ size_t factor_w_slice_bytes(int n, int m, int mixed, int fill) {
   return (size_t)fac_layout_w(n, m, mixed ? 4 : 8, fill != 0).total;
 }
 
-int persist_occupancy(int mixed, size_t smem) {
+int persist_occupancy(int mixed, size_t smem, int threads) {
   const void* fn = mixed ? (const void*)k_factor_persist<float> : (const void*)k_factor_persist<double>;
   if (set_smem(fn, smem)) return 0;
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kFactorThreads, smem) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess) return 0;
   return occ;
 }
 
 int launch_factor_persist(const LevelDesc* d, const Task* t, const PItem* items, int nitems, const PCons* cons,
                           int* ready, int mixed, const double* D, const double* E, const double* G,
-                          const double* R, Info* info, int grid, size_t smem, int slice,
+                          const double* R, Info* info, int grid, int threads, size_t smem, int slice,
                           long long wait_cycles, void* stream) {
   if (nitems <= 0) return 0;
   const void* fn = mixed ? (const void*)k_factor_persist<float> : (const void*)k_factor_persist<double>;
@@ -3664,11 +3664,11 @@ int launch_factor_persist(const LevelDesc* d, const Task* t, const PItem* items,
   if (e) return e;
   cudaStream_t st = (cudaStream_t)stream;
   if (mixed)
-    k_factor_persist<float><<<grid, kFactorThreads, smem, st>>>(d, t, items, nitems, cons, ready, D, E, G, R, info,
-                                                                slice, wait_cycles);
+    k_factor_persist<float><<<grid, threads, smem, st>>>(d, t, items, nitems, cons, ready, D, E, G, R, info, slice,
+                                                         wait_cycles);
   else
-    k_factor_persist<double><<<grid, kFactorThreads, smem, st>>>(d, t, items, nitems, cons, ready, D, E, G, R,
-                                                                 info, slice, wait_cycles);
+    k_factor_persist<double><<<grid, threads, smem, st>>>(d, t, items, nitems, cons, ready, D, E, G, R, info, slice,
+                                                          wait_cycles);
   return (int)cudaGetLastError();
 }
 

@@ -216,3 +216,30 @@ def test_right_hand_sides_of_a_batch(kkt, orc, n, m, P):
         finally:
             kkt.kkt_destroy(h)
         np.testing.assert_array_equal(x[seed], y.cpu().numpy())
+
+
+def test_persistent_schedule_of_uneven_blocks(kkt):
+    """One-warp and CTA tasks of two levels in one persistent launch of 128-thread
+    CTAs (more CTA tasks than the chip holds at 256 threads): bitwise the
+    solutions of the launches per level."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shapes = [(5, 17, 2, 2), (9, 4, 1, 3), (5, 20, 0, 1), (7, 16, 3, 2), (6, 24, 1, 2)]
+    pick = [shapes[i % 5] for i in range(10 * sms)]
+    sys = {q: system(*q[:3]) for q in shapes}
+    a = [dev(np.concatenate([sys[q][k].ravel() for q in pick])) for k in range(4)]
+    b = np.random.default_rng(5).normal(size=sum(N * n + m for N, n, m, _ in pick))
+    out = []
+    for persistent in (False, True):
+        h = kkt.kkt_batch_create(*[[q[k] for q in pick] for k in range(4)])
+        try:
+            kkt.kkt_set_persistent(h, persistent)
+            x = dev(b)
+            kkt.kkt_factor(h, *a)
+            kkt.kkt_solve(h, x)
+            assert kkt.kkt_get_info(h)["status"] == 0
+            out.append(x.cpu().numpy())
+        finally:
+            kkt.kkt_destroy(h)
+    assert np.isfinite(out[0]).all()
+    np.testing.assert_array_equal(out[0], out[1])
