@@ -1298,7 +1298,11 @@ struct FacCtx {
 // Forward substitution task of the solve kernels (defined below); the factor
 // kernel of a bordered pass runs it for the top level (corner solve and the
 // backward sweep of the top level) right after the corner.
-template <typename TS, bool W = false>
+// KIND: how the tasks share the chip.
+constexpr int kAlone = 0;  // a CTA each, at most two on an SM: registers for the loads ahead
+constexpr int kWarp = 1;   // a warp each (small blocks)
+constexpr int kDense = 2;  // a CTA each, several on an SM hide the latency for one another
+template <typename TS, int KIND = kAlone>
 __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs, double* b, int ldb, int nr,
                              const int* skip, unsigned char* smraw, Grp G, int fwd_done, int c0 = 0);
 
@@ -2248,7 +2252,12 @@ __device__ __forceinline__ void cp_async_flat(T* dst, const T* src, int cnt, Grp
 // with a branch per step and its multipliers' latency: they are read four steps
 // ahead. (A broadcast through shared memory takes 119; one broadcast for two steps and
 // another FMA in its place, 133.)
-template <typename TS, int NC, bool TWO, bool BW, bool EXACT = false>
+// LEAN, for tasks that share an SM by the dozen: their number hides the latency,
+// the FP64 pipe and the registers are the limit, so no step too many and four
+// multipliers at a time (eight in flight cost registers: 8 systems of 2000 stages, n = 12
+// in 300 segments solved in 3847 us against 3367; of 4000 stages, n = 8, 64 systems 1388
+// against 1317).
+template <typename TS, int NC, bool TWO, bool BW, bool LEAN = false>
 __device__ __forceinline__ void trsv_cols(TS* t, int ldt, const TS* M, int ldl, const TS* rinv, int n, int c, int dc,
                                           int lane) {
   const int i0 = lane, i1 = lane + 32, r0 = min(i0, n - 1), r1 = min(i1, n - 1);  // (r: rows for addresses)
@@ -2267,12 +2276,12 @@ __device__ __forceinline__ void trsv_cols(TS* t, int ldt, const TS* M, int ldl, 
       m1[s] = TWO ? M[j * ldl + r1] : TS(0);
     }
   };
-  // four steps (those past the last one change dead rows only; EXACT leaves them
-  // out, where the FP64 pipe is the limit); no branch a lane could take alone
+  // four steps (those past the last one change dead rows only; LEAN leaves them
+  // out); no branch a lane could take alone
   auto run = [&](int s0, const TS* m0, const TS* m1) {
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
-      if (EXACT && s0 + s >= steps) break;
+      if (LEAN && s0 + s >= steps) break;
       const int j = BW ? n - 1 - s0 - s : s0 + s;
       TS x[NC];
 #pragma unroll
@@ -2296,6 +2305,11 @@ __device__ __forceinline__ void trsv_cols(TS* t, int ldt, const TS* M, int ldl, 
   load(0, ma0, ma1);
 #pragma unroll 1
   for (int s0 = 0; s0 < steps; s0 += 4) {
+    if (LEAN) {
+      run(s0, ma0, ma1);
+      if (s0 + 4 < steps) load(s0 + 4, ma0, ma1);
+      continue;
+    }
     load(s0 + 4, mb0, mb1);
     run(s0, ma0, ma1);
 #pragma unroll
@@ -2324,16 +2338,19 @@ __device__ __noinline__ void trsv_warp(TS* t, int ldt, const TS* M, int ldl, con
     }
   }
 }
-// (W: the one-warp tasks of small blocks, n <= 32 and a column at a time, which
-// share an SM by the dozen and want few registers)
-template <typename TS, bool W, bool BW>
+// (kWarp, kDense: a column at a time; one-warp tasks have n <= 32)
+template <typename TS, int KIND, bool BW>
 __device__ __forceinline__ void trsv_group(TS* t, int ldt, const TS* M, int ldl, const TS* rinv, int n, int nr,
                                            Grp G) {
-  if (W) {
-    for (int c = 0; c < nr; ++c) trsv_cols<TS, 1, false, BW, true>(t, ldt, M, ldl, rinv, n, c, 0, G.tid);
+  if (KIND == kAlone) {
+    trsv_warp<TS, BW>(t, ldt, M, ldl, rinv, n, nr, G);
     return;
   }
-  trsv_warp<TS, BW>(t, ldt, M, ldl, rinv, n, nr, G);
+  const int lane = G.tid & 31;
+  for (int c = KIND == kWarp ? 0 : G.tid >> 5; c < nr; c += KIND == kWarp ? 1 : G.nt >> 5) {
+    if (KIND == kWarp || n <= 32) trsv_cols<TS, 1, false, BW, true>(t, ldt, M, ldl, rinv, n, c, 0, lane);
+    else trsv_cols<TS, 1, true, BW, true>(t, ldt, M, ldl, rinv, n, c, 0, lane);
+  }
 }
 
 // Shared-memory view of a substitution task: double-buffered factor blocks
@@ -2417,7 +2434,7 @@ __device__ __forceinline__ void stage_rows(const SegGeom& g, int i, int n, int m
 // blocks of the next stage stream in while the current one is solved.
 // (prefetched: the last stage's factor blocks were already requested into
 // buffer 0, see backward_prefetch)
-template <typename TS, bool W>
+template <typename TS, int KIND>
 __device__ void backward_segment(const SolveSmem<TS>& S, const LevelDesc& d, const SegGeom& g,
                                  double* b, int ldb, int nr, int c0, Grp G, bool prefetched = false) {
   const int n = d.n, m = d.m;
@@ -2433,7 +2450,7 @@ __device__ void backward_segment(const SolveSmem<TS>& S, const LevelDesc& d, con
   for (int i = g.len - 1; i >= 0; --i) {
     const int j = g.f + i, q = (g.len - 1 - i) & 1;
     stage_rows(g, i, n, m, r0, r1);
-    VecPrefetch<W ? 0 : 3> yp;  // y_{j-1}: its loads pass during this stage
+    VecPrefetch<KIND == kAlone ? 3 : 0> yp;  // y_{j-1}: its loads pass during this stage
     cp_async_wait_all();
     gsync(G);
     if (i > 0) {
@@ -2455,7 +2472,7 @@ __device__ void backward_segment(const SolveSmem<TS>& S, const LevelDesc& d, con
         TS a0 = 0, a1 = 0;
         int r = ra;
         if (act) {
-#pragma unroll(W ? 1 : 4)
+#pragma unroll(KIND == kAlone ? 4 : 1)
           for (; r + 1 < rb; r += 2) {
             a0 = fma(Z[r * S.ldZ + c2], v(r, c), a0);
             a1 = fma(Z[(r + 1) * S.ldZ + c2], v(r + 1, c), a1);
@@ -2474,7 +2491,7 @@ __device__ void backward_segment(const SolveSmem<TS>& S, const LevelDesc& d, con
       stage_rows(g, i - 1, n, m, p0, p1);
       prefetch_stage_factor(S, q ^ 1, F, n, m, j - 1, p0, p1, true, B);
     }
-    trsv_group<TS, W, true>(t, S.ldV, S.L(q), S.ldL, S.rinv(q), n, nr, G);
+    trsv_group<TS, KIND, true>(t, S.ldV, S.L(q), S.ldL, S.rinv(q), n, nr, G);
     if (i > 0) yp.store(xe, S.ldV, n, nr, by, B);
     gsync(G);
     store_vec(X.at(j), X.ld, t, S.ldV, n, nr, G);
@@ -2488,7 +2505,7 @@ __device__ void backward_segment(const SolveSmem<TS>& S, const LevelDesc& d, con
 // Forward substitution (Algorithm 2) for one segment; the top level (P = 1)
 // also solves the corner and runs its own backward sweep (Algorithm 3,
 // sequential phase). `skip`: per-system flags; a set flag returns at once.
-template <typename TS, bool W>
+template <typename TS, int KIND>
 __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs, double* b, int ldb, int nr,
                              const int* skip, unsigned char* smraw, Grp G, int fwd_done, int c0) {
   const LevelDesc& d = descs[tk.desc];
@@ -2527,7 +2544,7 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
     const int j = g.f + i, q = i & 1;
     const bool more = i + 1 < g.len;
     stage_rows(g, i, n, m, r0, r1);
-    VecPrefetch<W ? 0 : 3> bp;  // the next stage's rhs: its loads pass during the solve
+    VecPrefetch<KIND == kAlone ? 3 : 0> bp;  // the next stage's rhs: its loads pass during the solve
     if (more) {
       const size_t o = (size_t)(j + 1) * n * ldr;
       bp.load(ra + o, ldr, rb ? rb + o : nullptr, n, nr, by, B);
@@ -2539,7 +2556,7 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
       stage_rows(g, i + 1, n, m, p0, p1);
       prefetch_stage_factor(S, q ^ 1, F, n, m, j + 1, p0, p1, false, B);
     }
-    trsv_group<TS, W, false>(t, S.ldV, S.L(q), S.ldL, S.rinv(q), n, nr, G);
+    trsv_group<TS, KIND, false>(t, S.ldV, S.L(q), S.ldL, S.rinv(q), n, nr, G);
     if (more) bp.store(tn, S.ldV, n, nr, by, B);
     else
       for (int e = G.tid; e < n * S.ldV; e += G.nt) tn[e] = TS(0);  // the F-hat term
@@ -2560,7 +2577,7 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
         TS a0 = 0, a1 = 0;
         int t2 = k0;
         if (act) {
-#pragma unroll(W ? 1 : 4)
+#pragma unroll(KIND == kAlone ? 4 : 1)
           for (; t2 + 1 < k1; t2 += 2) {
             a0 = fma(Z[r * S.ldZ + t2], t[t2 * S.ldV + c], a0);
             a1 = fma(Z[r * S.ldZ + t2 + 1], t[(t2 + 1) * S.ldV + c], a1);
@@ -2614,10 +2631,10 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
     for (int e = G.tid; e < mg; e += G.nt) S.rinv(0)[e] = (TS)d.Rri[e];
     gsync(G);
     if (!fwd_done) {
-      trsv_group<TS, W, false>(gv, S.ldV, S.L(0), ldR, S.rinv(0), mg, nr, G);
+      trsv_group<TS, KIND, false>(gv, S.ldV, S.L(0), ldR, S.rinv(0), mg, nr, G);
       gsync(G);
     }
-    trsv_group<TS, W, true>(gv, S.ldV, S.L(1), ldR, S.rinv(0), mg, nr, G);
+    trsv_group<TS, KIND, true>(gv, S.ldV, S.L(1), ldR, S.rinv(0), mg, nr, G);
     gsync(G);
     store_vec(bg, ldb, gv, S.ldV, mg, nr, G);
   }
@@ -2628,13 +2645,13 @@ __device__ void forward_task(const Task tk, const LevelDesc* __restrict__ descs,
     else S.V[e] = S.t[(r - oG) * S.ldV + (e - r * S.ldV)];
   }
   gsync(G);
-  backward_segment<TS, W>(S, d, g, b, ldb, nr, c0, G);
+  backward_segment<TS, KIND>(S, d, g, b, ldb, nr, c0, G);
 }
 
 // Backward substitution (Algorithm 3, parallel phase) for one segment below
 // the top level: needs x_g (already in b), the separator solutions of the
 // next level (x at s_k and s_{k+1}), and this level's y.
-template <typename TS, bool W = false>
+template <typename TS, int KIND = kAlone>
 __device__ void backward_task(const Task tk, const LevelDesc* __restrict__ descs, double* b, int ldb, int nr,
                               const int* skip, unsigned char* smraw, Grp G, int c0 = 0, bool prefetched = false) {
   const LevelDesc& d = descs[tk.desc];
@@ -2658,7 +2675,7 @@ __device__ void backward_task(const Task tk, const LevelDesc* __restrict__ descs
     store_vec(xs.p, xs.ld, S.V + oW * S.ldV, S.ldV, n, nr, G);
   }
   gsync(G);
-  backward_segment<TS, W>(S, d, g, b, ldb, nr, c0, G, prefetched);
+  backward_segment<TS, KIND>(S, d, g, b, ldb, nr, c0, G, prefetched);
 }
 
 // The factor blocks of the backward sweep's first stage (the segment's last)
@@ -2676,8 +2693,8 @@ __device__ void backward_prefetch(const Task tk, const LevelDesc& d, unsigned ch
 
 // One CTA per task (blocks above kWarpMaxN), or one warp per task with a
 // shared-memory slice each (small blocks; `slice` bytes per warp).
-template <typename TS>
-__global__ void __launch_bounds__(kSolveThreads, 2) k_forward(const LevelDesc* __restrict__ descs,
+template <typename TS, int KIND>
+__global__ void __launch_bounds__(kSolveThreads, KIND == kDense ? 4 : 2) k_forward(const LevelDesc* __restrict__ descs,
                                                            const Task* __restrict__ tasks, double* b,
                                                            int ldb, int nr, const int* skip, int fwd_done,
                                                            int split) {
@@ -2685,16 +2702,16 @@ __global__ void __launch_bounds__(kSolveThreads, 2) k_forward(const LevelDesc* _
   // `split` CTAs per task, each on its own group of right-hand-side columns
   const int cg = blockIdx.x % split, nc = (nr + split - 1) / split, c0 = cg * nc, cn = min(nc, nr - c0);
   if (cn <= 0) return;
-  forward_task<TS>(tasks[blockIdx.x / split], descs, b + c0, ldb, cn, skip, smraw, cta_grp(), fwd_done, c0);
+  forward_task<TS, KIND>(tasks[blockIdx.x / split], descs, b + c0, ldb, cn, skip, smraw, cta_grp(), fwd_done, c0);
 }
-template <typename TS>
-__global__ void __launch_bounds__(kSolveThreads, 2) k_backward(const LevelDesc* __restrict__ descs,
+template <typename TS, int KIND>
+__global__ void __launch_bounds__(kSolveThreads, KIND == kDense ? 4 : 2) k_backward(const LevelDesc* __restrict__ descs,
                                                             const Task* __restrict__ tasks, double* b,
                                                             int ldb, int nr, const int* skip, int split) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int cg = blockIdx.x % split, nc = (nr + split - 1) / split, c0 = cg * nc, cn = min(nc, nr - c0);
   if (cn <= 0) return;
-  backward_task<TS>(tasks[blockIdx.x / split], descs, b + c0, ldb, cn, skip, smraw, cta_grp(), c0);
+  backward_task<TS, KIND>(tasks[blockIdx.x / split], descs, b + c0, ldb, cn, skip, smraw, cta_grp(), c0);
 }
 template <typename TS>
 __global__ void __launch_bounds__(256, 3) k_forward_w(const LevelDesc* __restrict__ descs,
@@ -2703,7 +2720,7 @@ __global__ void __launch_bounds__(256, 3) k_forward_w(const LevelDesc* __restric
   extern __shared__ __align__(16) unsigned char smraw[];
   const int wid = threadIdx.x >> 5, t = blockIdx.x * (blockDim.x >> 5) + wid;
   if (t >= ntasks) return;  // whole warp
-  forward_task<TS, true>(tasks[t], descs, b, ldb, nr, skip, smraw + (size_t)wid * slice,
+  forward_task<TS, kWarp>(tasks[t], descs, b, ldb, nr, skip, smraw + (size_t)wid * slice,
                    Grp{(int)(threadIdx.x & 31), 32, -1}, fwd_done);
 }
 template <typename TS>
@@ -2713,7 +2730,7 @@ __global__ void __launch_bounds__(256, 3) k_backward_w(const LevelDesc* __restri
   extern __shared__ __align__(16) unsigned char smraw[];
   const int wid = threadIdx.x >> 5, t = blockIdx.x * (blockDim.x >> 5) + wid;
   if (t >= ntasks) return;  // whole warp
-  backward_task<TS, true>(tasks[t], descs, b, ldb, nr, skip, smraw + (size_t)wid * slice,
+  backward_task<TS, kWarp>(tasks[t], descs, b, ldb, nr, skip, smraw + (size_t)wid * slice,
                     Grp{(int)(threadIdx.x & 31), 32, -1});
 }
 
@@ -3811,19 +3828,39 @@ int launch_factor_clus(const LevelDesc* d, const Task* t, int ntasks, int maxn, 
            : (int)cudaLaunchKernelEx(&cfg, k_factor_clus<false>, d, t, D, E, G, info, b, ldb, C);
 }
 
+// The substitution kernel of a launch of `grid` CTAs: the dense one (64 registers,
+// four CTAs per SM where shared memory allows) if the launch has more CTAs than the
+// other one (128 registers, loads a stage ahead, two columns a warp) holds at once.
+// Alone against dense, us: 1000 systems of N = 40, m = 4, n = 17 796, 472 (one
+// column) and 2289, 1686 (eight), n = 33 1885, 1168, n = 41, sixteen 12793, 12942;
+// 400 systems, m = 0, n = 33 929, 549.
+template <typename F>
+static F pick_solve(F alone, F dense, unsigned grid, size_t sm, int* err) {
+  int dev = 0, sms = 0, o1 = 0, o2 = 0;
+  *err = set_smem((const void*)alone, sm);
+  if (*err) return alone;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || grid <= (unsigned)sms)
+    return alone;
+  if (set_smem((const void*)dense, sm) == 0 &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, alone, kSolveThreads, sm) == cudaSuccess &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, dense, kSolveThreads, sm) == cudaSuccess && o2 > o1 &&
+      grid > (unsigned)(o1 * sms))
+    return dense;
+  return alone;
+}
+
 int launch_forward(const LevelDesc* d, const Task* t, int ntasks, int maxn, int maxm, int single,
                    double* b, int ldb, int nrhs, const int* skip, void* stream, int fwd_done, int split, int fill) {
   if (ntasks <= 0) return 0;
   const size_t sm = solve_smem_bytes(maxn, maxm, single, fill);
-  const void* fn = single ? (const void*)k_forward<float> : (const void*)k_forward<double>;
-  int e = set_smem(fn, sm);
-  if (e) return e;
   split = std::max(1, std::min(split, nrhs));
   const unsigned grid = (unsigned)(ntasks * split);
-  if (single)
-    k_forward<float><<<grid, kSolveThreads, sm, (cudaStream_t)stream>>>(d, t, b, ldb, nrhs, skip, fwd_done, split);
-  else
-    k_forward<double><<<grid, kSolveThreads, sm, (cudaStream_t)stream>>>(d, t, b, ldb, nrhs, skip, fwd_done, split);
+  int e = 0;
+  auto* const fn = single ? pick_solve(k_forward<float, kAlone>, k_forward<float, kDense>, grid, sm, &e)
+                          : pick_solve(k_forward<double, kAlone>, k_forward<double, kDense>, grid, sm, &e);
+  if (e) return e;
+  fn<<<grid, kSolveThreads, sm, (cudaStream_t)stream>>>(d, t, b, ldb, nrhs, skip, fwd_done, split);
   return (int)cudaGetLastError();
 }
 
@@ -3831,15 +3868,13 @@ int launch_backward(const LevelDesc* d, const Task* t, int ntasks, int maxn, int
                     double* b, int ldb, int nrhs, const int* skip, void* stream, int split, int fill) {
   if (ntasks <= 0) return 0;
   const size_t sm = solve_smem_bytes(maxn, maxm, single, fill);
-  const void* fn = single ? (const void*)k_backward<float> : (const void*)k_backward<double>;
-  int e = set_smem(fn, sm);
-  if (e) return e;
   split = std::max(1, std::min(split, nrhs));
   const unsigned grid = (unsigned)(ntasks * split);
-  if (single)
-    k_backward<float><<<grid, kSolveThreads, sm, (cudaStream_t)stream>>>(d, t, b, ldb, nrhs, skip, split);
-  else
-    k_backward<double><<<grid, kSolveThreads, sm, (cudaStream_t)stream>>>(d, t, b, ldb, nrhs, skip, split);
+  int e = 0;
+  auto* const fn = single ? pick_solve(k_backward<float, kAlone>, k_backward<float, kDense>, grid, sm, &e)
+                          : pick_solve(k_backward<double, kAlone>, k_backward<double, kDense>, grid, sm, &e);
+  if (e) return e;
+  fn<<<grid, kSolveThreads, sm, (cudaStream_t)stream>>>(d, t, b, ldb, nrhs, skip, split);
   return (int)cudaGetLastError();
 }
 

@@ -243,3 +243,35 @@ def test_persistent_schedule_of_uneven_blocks(kkt):
             kkt.kkt_destroy(h)
     assert np.isfinite(out[0]).all()
     np.testing.assert_array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n,m,P", [(17, 2, 1), (32, 0, 2), (33, 3, 1), (41, 1, 2)])
+def test_substitutions_of_many_and_few_systems(kkt, n, m, P, precision):
+    """More systems than the chip holds CTAs at two per SM: the dense substitution
+    kernels, whose every system is bitwise the few systems' of a handle of five."""
+    import torch
+    many, N = 2 * torch.cuda.get_device_properties(0).multi_processor_count + 5, 7
+    sys = [system(N, n, m, seed) for seed in range(5)]
+    for nrhs in (1, 3, 9, 16):
+        b = np.random.default_rng(nrhs).normal(size=(5, N * n + m, nrhs))
+        out = []
+        for count in (5, many):
+            a = [dev(np.concatenate([sys[i % 5][k].ravel() for i in range(count)])) if k < 2 or m else None for k in range(4)]
+            x = dev(np.concatenate([b[i % 5] for i in range(count)]))
+            h = kkt.kkt_batch_create([N] * count, [n] * count, [m] * count, [P] * count, precision)
+            try:
+                kkt.kkt_factor(h, *a)
+                if precision == 0:
+                    kkt.kkt_solve(h, x)
+                else:
+                    y = torch.zeros_like(x)
+                    kkt.kkt_solve_refined(h, *a, x, y)
+                    x = y
+                assert kkt.kkt_get_info(h)["status"] == 0
+            finally:
+                kkt.kkt_destroy(h)
+            out.append(x.cpu().numpy().reshape(count, N * n + m, nrhs))
+        assert np.isfinite(out[0]).all()
+        for i in range(many):
+            np.testing.assert_array_equal(out[1][i], out[0][i % 5], err_msg=f"system {i} of {nrhs} columns")
