@@ -268,6 +268,11 @@ class ClockSampler:
                 "samples": len(self.samples), "source": "nvml" if self.nvml else "nvidia-smi"}
 
 
+ROOFLINE_NOTE = ("the Schur products of blocks n >= 20 run as FP16 digit products on the tensor cores, so frac "
+                 "compares with the FP64 FMA units and is no utilization; the launch is bound by the pivot "
+                 "chains' latency, its counters are in profiles/")
+
+
 def read_traffic(kernel_src_sha: str):
     """DRAM bytes per launch of the dominant kernel from the committed ncu
     summary, or None when that summary was taken on other kernel source."""
@@ -286,7 +291,7 @@ def read_traffic(kernel_src_sha: str):
 def kernel_source_sha() -> str:
     import hashlib
     h = hashlib.sha256()
-    for f in ("kkt_kernels.cu", "kkt_internal.h"):
+    for f in ("kkt_kernels.cu", "kkt_internal.h", "kkt_oz.cuh", "kkt_numerics.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2511_00946_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
 
@@ -389,7 +394,8 @@ def per_launch_flops(kkt, plan, partition, nrhs=1, chain=False):
         names.append("k_border (bordered arrow copy)")
         flops.append(0.0)
     tag = " (+forward)" if fused else ""
-    names += [f"k_factor level {l + 1}{tag}" for l in range(L)]
+    # level 1 runs k_factor_fp64; deeper levels of one-stage segments k_factor_clus
+    names += [f"{'k_factor_fp64' if l == 0 else 'factor'} level {l + 1}{tag}" for l in range(L)]
     flops += list(fac)
     if not fused:
         for l in range(L - 1):
@@ -398,7 +404,7 @@ def per_launch_flops(kkt, plan, partition, nrhs=1, chain=False):
         names.append(f"k_forward level {L} (forward, corner, backward)")
         flops.append(sol[L - 1])
     else:
-        names[-1] = f"k_factor level {L} (+forward, corner, corner solve, backward)"
+        names[-1] = f"{'k_factor_fp64' if L == 1 else 'factor'} level {L} (+forward, corner, corner solve, backward)"
         flops[-1] += sol[L - 1] / 2.0
     if chain:
         names.append(f"k_backward_chain (levels {L - 1}..1)")
@@ -722,7 +728,7 @@ def measure_batch(name, args, world, rank, local, host_check=64, paths=None):
             r["refinement"] = {"sweeps_max": args.sweeps, "tol": args.tol,
                                "stop": "eta <= tol, or eta <= 4 u and a sweep that cuts it by less than 10 % (rounding floor)"}
         if split is not None:
-            names = [f"{'k_factor_w' if n <= 16 else 'k_factor'} n={n} ({len(sy)} systems)" for n, sy in fgroups]
+            names = [f"{'k_factor_w' if n <= 16 else 'k_factor' if mixed else 'k_factor_fp64'} n={n} ({len(sy)} systems)" for n, sy in fgroups]
             r["factor_launch_ms"] = {nm: round(v, 4) for nm, v in zip(names, split)}
             dom_avg = statistics.mean(dom_ms)
             r["dominant_factor_launch"] = {"kernel": names[dom], "launch_ms": dom_avg}
@@ -736,11 +742,12 @@ def measure_batch(name, args, world, rank, local, host_check=64, paths=None):
                     flops += cache[key]
                 ach = flops / (dom_avg * 1e-3) / 1e12
                 peak = FP64_PEAK_GFLOPS / 1000.0
-                r["roofline"] = {"bound": "alu", "kernel": names[dom], "launch_ms": dom_avg, "achieved": ach,
+                r["roofline"] = {"bound": "latency", "kernel": names[dom], "launch_ms": dom_avg, "achieved": ach,
                                  "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                                  "flops_per_launch": flops, "traffic": None,
                                  "note": "FP64 sequential factor flops of the launch's systems (standard "
-                                         "convention) over its event-timed duration in the timed graph"}
+                                         "convention) over its event-timed duration in the timed graph; "
+                                         + ROOFLINE_NOTE}
         results[path] = r
         kkt.kkt_destroy(h)
         del graph
@@ -1231,9 +1238,9 @@ def main():
             "launches_per_step_note": "ms per launch from 27 diagnostic graph replays with an event after "
                                       "every launch (those event nodes add about 5 us each); the timed steps "
                                       "record only the two events around the dominant launch",
-            "roofline": {"bound": "alu", "kernel": names[dom], "launch_ms": dom_avg, "achieved": achieved, "peak": peak,
+            "roofline": {"bound": "latency", "kernel": names[dom], "launch_ms": dom_avg, "achieved": achieved, "peak": peak,
                          "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None,
-                         "traffic": traffic, "peak_note": "FP64 FMA: 152 SMs x 2/clk x 2 flop x 2.07 GHz"},
+                         "traffic": traffic, "peak_note": "FP64 FMA: 152 SMs x 2/clk x 2 flop x 2.07 GHz; " + ROOFLINE_NOTE},
             "flops_per_step": {"factor": fl["factor"], "solve": fl["solve"],
                                "sequential_factor": fl["sequential_factor"]},
             "clocks": clk.summary(),

@@ -6,16 +6,18 @@
 // stacked panel Z = [E; G; W] and the Schur accumulator T in shared memory
 // (row-major, odd leading dimensions: row- and column-wise accesses are free
 // of bank conflicts) and runs
-//   potrf(D)  ->  Z <- Z D-hat^{-T}  ->  T -= Z Z^T (lower triangle)
-// with every thread on the element loops. FP64 is the scarce resource on this
-// part: one FP64 warp-instruction occupies a sub-partition's FP64 pipe for
-// about 64-76 cycles whether 1 or 32 lanes are active, and FP32 runs about
-// 70x faster. So the loops issue FP64 instructions from full warps only
-// (lower triangles are enumerated linearly instead of masked squares), and
-// the mixed variant (TZ = float) keeps only the pivot Cholesky and the
-// Schur accumulator in FP64: the panel trsm and the dot products of the
-// syrk run in FP32 and each dot product is subtracted from the FP64
-// accumulator once.
+//   D-hat = chol(D)  ->  Z <- Z D-hat^{-T}  ->  T -= Z Z^T (lower triangle)
+// FP64 is the scarce resource on this part: one FP64 warp-instruction occupies
+// a sub-partition's FP64 pipe for about 64-76 cycles whether 1 or 32 lanes are
+// active, and FP32 runs about 70x faster. So the loops issue FP64 instructions
+// from full warps only (lower triangles are enumerated linearly instead of
+// masked squares). FP64 tasks (k_factor_fp64, k_factor_clus) eliminate the pivot
+// block without square roots in blocks of eight columns, the panel solve beside
+// it (ldl_sweep), and take the Schur products of blocks n >= kDigMin from the
+// tensor cores by exact digit splitting (kkt_oz.cuh). Mixed tasks (k_factor) keep
+// the pivot Cholesky and the Schur accumulator in FP64: the panel solve and the
+// dot products run in FP32 and each dot product is subtracted from the FP64
+// accumulator once. Blocks n <= kWarpMaxN run one warp per task (k_factor_w).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -323,8 +325,7 @@ __device__ void potrf_trsm_sm(double* A, int ld, int n, double* rinv, TZ* M, con
 // (in k order) and x_c = u_c / L_cc (times rinv). Column sweep: every thread
 // works on every column (FP64 from full warps), thread t owning row
 // r0 + t % rows and every (nt/rows)-th column. The group needs at least as
-// many threads as rows (true for every panel: rows <= kMaxN + kMaxM per
-// role of a split CTA, 2 kMaxN + kMaxM otherwise).
+// many threads as rows (true for every panel: at most 2 kMaxN + kMaxM rows).
 template <typename TZ>
 __device__ void trsm_panel(TZ* Z, int ldz, int r0, int r1, const TZ* M, int ldm, int n, const TZ* rinv,
                            Grp g) {
@@ -925,9 +926,8 @@ __device__ __forceinline__ SegGeom seg_geom(const LevelDesc& d, int k) {
 // Factorization: Algorithm 1 for one segment (parallel phase); the top level
 // (P = 1) is the sequential phase on the reduced system and also factors the
 // corner R-hat = chol(R + sum of every R~_k partial).
-// TZ = double: every operation in FP64. TZ = float: FP64 pivots and Schur
-// accumulator, FP32 panel (trsm and dot products), FP32 factor copy written
-// for the correction solves.
+// FP64 tasks: factor_task_fp64. Mixed tasks (FP64 pivots and Schur accumulator,
+// FP32 panel, FP32 factor copy written for the correction solves): factor_task.
 //
 // Roles. The panel rows of a segment with fill-in (k >= 1) fall into two
 // groups. The producer runs the chain of Algorithm 1 proper: potrf(D_i), the
@@ -946,8 +946,6 @@ __device__ __forceinline__ SegGeom seg_geom(const LevelDesc& d, int k) {
 //           it before stage i; the producer waits for phase i-1 before it
 //           overwrites buffer i % 2 (double buffering). A last phase, after
 //           every remote store, ends the task.
-// FP64 tasks run factor_task_fp64 (k_factor_fp64, block fixed point), mixed ones
-// (FP32 panel) factor_task (k_factor).
 // ---------------------------------------------------------------------------
 static_assert(kFactorThreads == 256, "the factor roles assume 8 warps per CTA");
 constexpr int kWhole = 0, kPair = 2;
@@ -1488,51 +1486,44 @@ __global__ void __launch_bounds__(kFactorThreads, 2) k_factor_fp64(const LevelDe
                    smraw, bad);
 }
 
-// MINB: CTAs per SM the register allocation must allow. Launches of CTA pairs
-// (one CTA per SM, latency-bound) take the unconstrained allocation (1);
-// the others four (at most 64 registers), so that several segment CTAs share
-// an SM when shared memory allows it.
-// TC: the instantiation with the tensor-core Schur products (mixed launches
-// that use them); the others carry none of that code.
-// One segment task of the mixed factorization (TZ = float) by the whole CTA (or, with `pair`,
+// One segment task of the mixed factorization by the whole CTA (or, with `pair`,
 // by this CTA's half of a two-CTA cluster): the body of k_factor, also run
 // task after task by the persistent kernel. `bad`, `tslot`, `tbar`: shared
 // variables of the caller (breakdown flag, TMEM address slot, mbarrier).
-template <typename TZ, bool TC>
+template <bool TC>
 __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __restrict__ descs,
                                             const double* __restrict__ uD, const double* __restrict__ uE,
                                             const double* __restrict__ uG, const double* __restrict__ uR,
-                                            Info* info, int pair, double* yb, int ldyb,
+                                            Info* info, int pair,
                                             int tcm, unsigned char* smraw, int& bad, uint32_t& tslot,
                                             uint64_t& tbar) {
   const unsigned rank = pair ? cluster_rank() : 0u;
   const LevelDesc& d = descs[tk.desc];
-  constexpr bool mixed = sizeof(TZ) == 4;
-  const FacLayout lay = fac_layout(d.n, d.m, (int)sizeof(TZ), d.P > 1);
+  const FacLayout lay = fac_layout(d.n, d.m, (int)sizeof(float), d.P > 1);
   if (!task_geometry_ok(d, tk.seg, smraw, lay.total)) return;  // debug build only (both CTAs of a pair alike)
-  const FacCtx<TZ, 4> cx(d, tk.seg, smraw, lay, uD, uE, uG);
+  const FacCtx<float, 4> cx(d, tk.seg, smraw, lay, uD, uE, uG);
   const int n = cx.n, m = cx.m, R = cx.R, ldD = cx.ldD, ldZ = cx.ldZ, ldT = cx.ldT, oG = cx.oG, oW = cx.oW;
   double* const Dfac = cx.Dfac;
   double* const rinv = cx.rinv;
   double* const T = cx.T;
-  TZ* const M = cx.M;
-  TZ* const rinvZ = cx.rinvZ;
-  TZ* const Z = cx.Z;
+  float* const M = cx.M;
+  float* const rinvZ = cx.rinvZ;
+  float* const Z = cx.Z;
   int* const tab = cx.tab;
   const SegGeom g = cx.g;
   const int mode = pair ? kPair : kWhole;
   // consumer buffers of the pair layout: buffer 0 is (M, rinvZ, Z rows [0, n+m)),
   // buffer 1 reuses the pivot block, rinv and the first rows of T, which a
   // consumer CTA has no other use for
-  auto Mbuf = [&](int b) { return b ? (TZ*)Dfac : M; };
-  auto rinvbuf = [&](int b) { return b ? (TZ*)rinv : rinvZ; };
-  auto Zbuf = [&](int b) { return b ? (TZ*)T : Z; };
+  auto Mbuf = [&](int b) { return b ? (float*)Dfac : M; };
+  auto rinvbuf = [&](int b) { return b ? (float*)rinv : rinvZ; };
+  auto Zbuf = [&](int b) { return b ? (float*)T : Z; };
   const bool eg = mode != kPair || rank == 0;       // this CTA holds the E/G rows
   const bool wr = g.hasW && (mode != kPair || rank == 1);  // this CTA holds the W rows
 
   // tensor-core Schur products (mixed whole-CTA layout; the pivot buffers'
   // region stages the operands)
-  const bool use_tc = TC && mixed && tcm && mode == kWhole;
+  const bool use_tc = TC && tcm && mode == kWhole;
   const uint32_t tc_cols = ((lay.Rs + 15) & ~15) <= 64 ? 64u : 128u;
   uint32_t tmem = 0u, tphase = 0u;
   if constexpr (TC) {
@@ -1561,13 +1552,13 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
   }
 
   const bool producer = mode == kWhole || rank == 0;
-  auto store_pivot = [&](int j, const double* Dp_, const double* rv, const TZ* Ms, Grp G) {
+  auto store_pivot = [&](int j, const double* Dp_, const double* rv, const float* Ms, Grp G) {
     cx.store_pivot(j, Dp_, rv, Ms, G);
   };
   auto store_panel = [&](int j, int r0, int r1, int rows, Grp G) { cx.store_panel(j, r0, r1, rows, G); };
   // hand the trsm operand (strict lower triangle of Msrc, ld ldD), its
   // 1/diag and panel rows [r0, r1) of stage i to the consumer CTA of a pair
-  auto push_stage = [&](int i, const TZ* Msrc, const TZ* rsrc, int r0, int r1, Grp G) {
+  auto push_stage = [&](int i, const float* Msrc, const float* rsrc, int r0, int r1, Grp G) {
     const int b = i & 1;
     const unsigned aM = cluster_addr(Mbuf(b), 1), aR = cluster_addr(rinvbuf(b), 1),
                    aZ = cluster_addr(Zbuf(b), 1);
@@ -1576,13 +1567,13 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
       int a, c;
       tri_rc(e, a, c);
       const int off = (a + 1) * ldD + c;
-      st_cluster(aM + off * (unsigned)sizeof(TZ), Msrc[off]);
+      st_cluster(aM + off * (unsigned)sizeof(float), Msrc[off]);
     }
-    for (int e = G.tid; e < n; e += G.nt) st_cluster(aR + e * (unsigned)sizeof(TZ), rsrc[e]);
+    for (int e = G.tid; e < n; e += G.nt) st_cluster(aR + e * (unsigned)sizeof(float), rsrc[e]);
     for (int e = G.tid; e < (r1 - r0) * n; e += G.nt) {
       const int r = r0 + e / n, c = e - (r - r0) * n;
       const int off = r * ldZ + c;
-      st_cluster(aZ + off * (unsigned)sizeof(TZ), Z[off]);
+      st_cluster(aZ + off * (unsigned)sizeof(float), Z[off]);
     }
   };
   auto rotate = [&](int i, int j, bool withW, Grp G) { cx.rotate(i, j, withW, G); };
@@ -1602,9 +1593,8 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
       __syncthreads();
       if (threadIdx.x == 0 && bad) { record_breakdown(info, d.sys, d.nat[j], d.level); bad = 0; }
       store_pivot(j, Dfac, rinv, nullptr, P);  // read before the copy of D_{i+1} below
-      if (d.mr) cx.store_y(j, yb, ldyb, P);
       if (push) {
-        for (int e = P.tid; e < n; e += P.nt) rinvZ[e] = (TZ)rinv[e];
+        for (int e = P.tid; e < n; e += P.nt) rinvZ[e] = (float)rinv[e];
         __syncthreads();
         if (i > 0) cluster_wait();  // the consumer is done with stage i-2 (buffer i % 2)
         push_stage(i, M, rinvZ, r0, n + m, P);
@@ -1612,7 +1602,7 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
       }
       store_panel(j, r0, pr1, mode == kWhole ? R : n + m, P);
       bool tc_done = false;
-      if constexpr (mixed && TC) {
+      if constexpr (TC) {
         if (use_tc) {
           if (!syrk_tc(T, ldT, (const float*)Z, ldZ, r0, pr1, n, smraw + lay.oDfac, tmem, &tbar, tphase & 1, tcm) &&
               threadIdx.x == 0)
@@ -1641,12 +1631,12 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
       trsm_panel(Z, ldZ, oW, R, Mbuf(b), ldD, n, rinvbuf(b), C);
       {
         double* Pd = d.Lp + (size_t)j * R * n + (size_t)oW * n;
-        float* Pf = mixed ? d.Lpf + (size_t)j * R * n + (size_t)oW * n : nullptr;
+        float* Pf = d.Lpf + (size_t)j * R * n + (size_t)oW * n;
         for (int e = C.tid; e < n * n; e += C.nt) {
           const int r = e / n, c = e - r * n;
-          const TZ v = Z[(oW + r) * ldZ + c];
+          const float v = Z[(oW + r) * ldZ + c];
           Pd[e] = (double)v;
-          if (mixed) Pf[e] = (float)v;
+          Pf[e] = v;
         }
       }
       syrk_trap(T, ldT, Zbuf(b), Z, oW, ldZ, oW, R, r0, n, C);
@@ -1714,20 +1704,26 @@ __device__ __forceinline__ void factor_task(const Task tk, const LevelDesc* __re
   }
 }
 
-template <typename TZ, int MINB, bool TC = false>
+// MINB: CTAs per SM the register allocation must allow. Launches of CTA pairs
+// (one CTA per SM, latency-bound) take the unconstrained allocation (1);
+// the others four (at most 64 registers), so that several segment CTAs share
+// an SM when shared memory allows it.
+// TC: the instantiation with the tensor-core Schur products (mixed launches
+// that use them); the others carry none of that code.
+template <int MINB, bool TC = false>
 __global__ void __launch_bounds__(kFactorThreads, MINB) k_factor(const LevelDesc* __restrict__ descs,
                                                            const Task* __restrict__ tasks,
                                                            const double* __restrict__ uD,
                                                            const double* __restrict__ uE,
                                                            const double* __restrict__ uG,
                                                            const double* __restrict__ uR,
-                                                           Info* info, int pair, double* yb, int ldyb,
+                                                           Info* info, int pair,
                                                            int tcm) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int bad;
   __shared__ uint32_t tslot;               // TMEM address of the tensor-core accumulator
   __shared__ __align__(8) uint64_t tbar;   // its completion mbarrier
-  factor_task<TZ, TC>(tasks[pair ? blockIdx.x >> 1 : blockIdx.x], descs, uD, uE, uG, uR, info, pair, yb, ldyb,
+  factor_task<TC>(tasks[pair ? blockIdx.x >> 1 : blockIdx.x], descs, uD, uE, uG, uR, info, pair,
                       tcm, smraw, bad, tslot, tbar);
 }
 
@@ -1917,8 +1913,7 @@ __global__ void __launch_bounds__(kFactorThreads, 2) k_factor_clus(const LevelDe
 // stage warp-synchronous, several tasks per CTA with a shared-memory slice
 // each. The CTA kernel's role split needs blocks large enough to keep eight
 // warps busy; at n = 6 a stage is a few hundred FMAs, and what counts is how
-// many independent stage chains an SM interleaves. The operations per
-// element are those of the CTA kernel, in the same order.
+// many independent stage chains an SM interleaves.
 // ---------------------------------------------------------------------------
 
 // Z[r0:r1) <- Z[r0:r1) L^{-T} by one warp, one panel row per lane: the
@@ -2086,8 +2081,7 @@ __global__ void __launch_bounds__(kFactorThreads, sizeof(TZ) == 8 ? 2 : 3)
         if constexpr (sizeof(TZ) == 8)
           factor_task_fp64<false>(tasks[w.first], descs, uD, uE, uG, uR, info, 0, nullptr, 1, 0, smraw, bad);
         else
-          factor_task<TZ, false>(tasks[w.first], descs, uD, uE, uG, uR, info, 0, nullptr, 1, 0, smraw, bad, tslot,
-                                 tbar);
+          factor_task<false>(tasks[w.first], descs, uD, uE, uG, uR, info, 0, 0, smraw, bad, tslot, tbar);
       } else {
         const int wid = threadIdx.x >> 5;
         if (wid < w.cnt)
@@ -3735,9 +3729,9 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
   size_t sm = factor_smem_bytes(maxn, maxm, mixed, fill);
   if (top_solve) sm = std::max(sm, solve_smem_bytes(maxn, maxm, 0, fill));
   const void* fn = !mixed ? (b ? (const void*)k_factor_fp64<true> : (const void*)k_factor_fp64<false>)
-                   : pair ? (const void*)k_factor<float, 1>
-                   : tcm  ? (const void*)k_factor<float, 4, true>
-                          : (const void*)k_factor<float, 4>;
+                   : pair ? (const void*)k_factor<1>
+                   : tcm  ? (const void*)k_factor<4, true>
+                          : (const void*)k_factor<4>;
   const int e = set_smem(fn, sm);
   if (e) return e;
   cudaLaunchConfig_t cfg = {};
@@ -3772,9 +3766,9 @@ int launch_factor(const LevelDesc* d, const Task* t, int ntasks, int maxn, int m
   if (!mixed)
     return b ? (int)cudaLaunchKernelEx(&cfg, k_factor_fp64<true>, d, t, D, E, G, R, info, p, b, ldb, top_solve)
              : (int)cudaLaunchKernelEx(&cfg, k_factor_fp64<false>, d, t, D, E, G, R, info, p, b, ldb, top_solve);
-  return pair ? (int)cudaLaunchKernelEx(&cfg, k_factor<float, 1>, d, t, D, E, G, R, info, p, b, ldb, 0)
-         : tcm ? (int)cudaLaunchKernelEx(&cfg, k_factor<float, 4, true>, d, t, D, E, G, R, info, p, b, ldb, tcm)
-               : (int)cudaLaunchKernelEx(&cfg, k_factor<float, 4>, d, t, D, E, G, R, info, p, b, ldb, 0);
+  return pair ? (int)cudaLaunchKernelEx(&cfg, k_factor<1>, d, t, D, E, G, R, info, p, 0)
+         : tcm ? (int)cudaLaunchKernelEx(&cfg, k_factor<4, true>, d, t, D, E, G, R, info, p, tcm)
+               : (int)cudaLaunchKernelEx(&cfg, k_factor<4>, d, t, D, E, G, R, info, p, 0);
 }
 
 int factor_clus_size(int ntasks, int maxn, int maxm, int sms) {

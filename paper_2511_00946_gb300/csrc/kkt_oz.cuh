@@ -16,21 +16,37 @@
 // every digit, so that a digit is a bit field of its own; a pair of fields
 // becomes a pair of FP16 numbers with two logical operations (1024 + field is
 // the bit pattern 0x6400 | field) and one subtraction. The products d_i d_j
-// are accumulated over k separately for every i + j = 6 .. 12: sums of
-// integers below 2^24, which FP32 accumulators hold exactly (a test on the
-// device checks it); the digit pairs with i + j <= 5 are dropped: below 2^-58
-// of the rows' scales (root mean square). The seven sums are combined in 64-bit
-// integers, rounded to double once and subtracted from T.
+// are accumulated over k separately for every i + j = 6 .. 12 in FP32. Sums
+// below 2^24 are exact there (a test on the device checks it): all of them up to
+// K = 36 columns; beyond, the two lowest sums (five and six pairs of full
+// digits) can pass it and lose units that weigh 2^-59 of the rows' scales. The
+// digit pairs with i + j <= 5 are dropped: below 2^-58 of the rows' scales (root
+// mean square). The seven sums are combined in 64-bit integers, rounded to
+// double once and subtracted from T.
 //
-// Error against FP64 FMAs: the sum is rounded once instead of once per term.
-// Solutions of the timed systems are 1.4 to 3.4 times closer to the exact ones
-// than with FP64 products (block sizes 12 to 48, barrier scalings of 4 to 10
-// decades); tests/test_oz_cpu.py bounds the products against exact arithmetic.
+// Accuracy. The error of element (a, b) is one rounding of the sum and about
+// 2^-58 2^(f_a + f_b), whatever the columns hold. In a Cholesky factorization
+// |Z_ak| <= sqrt(Psi_aa), so that is 2^-58 sqrt(Psi_aa Psi_bb): a backward error
+// below that of FP64 FMAs, and invariant to the scaling of the variables (row a of
+// the factor scales with variable a. The unscaled operands of the pivot sweep
+// are not split: their columns carry the pivots' roots, and one exponent per
+// row loses the ratio of those). It is a bound on the
+// scale of the two variables, not on the element: entries of the factor far below
+// it, between variables that are coupled by less than 1e-4 of their own scales, keep
+// fewer digits of their own than FMAs would leave them (an answer that reaches one
+// half of a stage through couplings of 1e-6 alone has 13 digits, of 1e-9 ten). A
+// right-hand side has no such bound, which is why a bordered one is not split.
+// Errors of the timed systems against 64-bit arithmetic, after those with FMAs:
+// N = 1024, n = 32 3.7e-12, 1.0e-12; N = 777, n = 45 4.6e-13, 1.3e-13; 4096 uneven
+// systems 2.7e-12, 1.8e-12; 512 systems, n = 32 5.6e-12, 1.8e-12.
+// tests/test_oz_cpu.py bounds the products against exact arithmetic,
+// tests/test_gpu_scaling.py asks for the same bits in any units.
 //
 // Measured (whole-CTA stage, 256 threads, 2070 MHz): the update of a 73-row
 // panel of 32 columns takes 16k cycles on one SM alone, against 42k of FP64
 // issue alone; one system of N = 1024, n = 32, m = 8 factored and solved 708 ->
-// 653 us, N = 777, n = 45 1527 -> 1238 us, 4096 uneven systems 70.8 -> 63.6 ms.
+// 653 us, N = 777, n = 45 1527 -> 1238 us, 4096 uneven systems 70.8 -> 63.6 ms (with
+// the pivot sweep as it was then).
 //
 // A row with infinities, NaN or an exponent above 400, or whose elements are
 // near the subnormal range, keeps its doubles (flag kFp64Row) and takes FP64
