@@ -269,8 +269,7 @@ class ClockSampler:
 
 
 ROOFLINE_NOTE = ("the Schur products of blocks n >= 20 run as FP16 digit products on the tensor cores, so frac "
-                 "compares with the FP64 FMA units and is no utilization; the launch is bound by the pivot "
-                 "chains' latency, its counters are in profiles/")
+                 "compares with the FP64 FMA units and is no utilization; the counters are in profiles/")
 
 
 def read_traffic(kernel_src_sha: str):
@@ -742,7 +741,7 @@ def measure_batch(name, args, world, rank, local, host_check=64, paths=None):
                     flops += cache[key]
                 ach = flops / (dom_avg * 1e-3) / 1e12
                 peak = FP64_PEAK_GFLOPS / 1000.0
-                r["roofline"] = {"bound": "latency", "kernel": names[dom], "launch_ms": dom_avg, "achieved": ach,
+                r["roofline"] = {"bound": "alu", "kernel": names[dom], "launch_ms": dom_avg, "achieved": ach,
                                  "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                                  "flops_per_launch": flops, "traffic": None,
                                  "note": "FP64 sequential factor flops of the launch's systems (standard "
